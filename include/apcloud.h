@@ -247,8 +247,9 @@ apcloud_status apcloud_solve_system(apcloud_ctx *ctx, int which, const double *d
  * larger problems return APCLOUD_E_INVALID.  The context's device must be
  * the current device (APCLOUD_E_INVALID otherwise).  The first call on a
  * device also looks up the array's device address (cudaGetSymbolAddress).
- * The call reads the residual back to the host once per restart cycle, so it
- * synchronises the context stream every cycle and must not be called while
+ * The call reads the outcome back to the host (once per solve, or once per
+ * restart cycle for a system the one-kernel solve does not take), so it
+ * synchronises the context stream and must not be called while
  * that stream is being captured into a CUDA graph.  All calls share the one
  * array: two calls whose work overlaps on the GPU (other streams, other
  * contexts, other host threads) race and give undefined results; each call
@@ -337,7 +338,11 @@ apcloud_status apcloud_push_particles(apcloud_ctx *ctx, double *d_x, double *d_y
  * enable = 0 launches every kernel directly and reads the stopping flag back
  * after every Arnoldi step (the same kernels in the same order, the same
  * results).  Kernel timers (apcloud_set_timing) also run cycles as direct
- * launches, stopped the same way.  Synchronises the context stream.  The
+ * launches, stopped the same way.  A single-beam solve whose matrix fits the
+ * shared memory of the SMs together runs as one cooperative kernel (restart
+ * up to 31; about 2.4e5 nodes in the mixed polynomial form, 1.2e5 in FP64),
+ * with graphs on replayed as a graph of that one kernel: the same results
+ * either way.  Synchronises the context stream.  The
  * paper has no counterpart (launch mechanics). */
 apcloud_status apcloud_set_graphs(apcloud_ctx *ctx, int enable);
 
@@ -487,7 +492,9 @@ apcloud_status apcloud_solve_learned(apcloud_ctx *ctx, apcloud_mpnn *net, unsign
  * the last reset (reset = 1 clears).  Consecutive launches of one timed kind
  * share one pair of events (before the first, after the last), so their time
  * includes the gaps between them; a launch of any other kind or a host
- * read-back closes the pair. */
+ * read-back closes the pair.  A solve that runs as one kernel (see
+ * apcloud_set_graphs) reports the time its first block spent in each kind of
+ * work and counts each phase as a launch of that kind. */
 #define APCLOUD_NUM_KINDS 19
 apcloud_status apcloud_set_timing(apcloud_ctx *ctx, unsigned mask);
 apcloud_status apcloud_get_timing(apcloud_ctx *ctx, double *h_ms, int64_t *h_launches, double *h_bytes,

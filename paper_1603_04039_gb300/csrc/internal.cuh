@@ -1,6 +1,7 @@
 // internal.cuh -- shared declarations of the GB300 AP-Cloud library (not part of the ABI).
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -140,6 +141,46 @@ struct IluDev {
     std::vector<IluSeg> lseg, useg;
 };
 
+// Resident solves (resident.cu): what the kernel gets and reports.
+constexpr int RES_MAX_RESTART = 31;
+constexpr int RES_KINDS = 6;
+enum { RES_SPMV = 0, RES_SWEEP, RES_DOT, RES_UPDDOT, RES_UPDNORM, RES_CYCLE };
+enum { RES_OK = 0, RES_MAXITER, RES_UNFIT, RES_TIMEOUT, RES_MORE };
+struct ResidentIn {
+    const double *b;
+    double *x;               // guess in, solution out
+    double rtol, omega;
+    int max_iter, resume;    // resume: go on from the iterate of the launch before
+    uint32_t tag0;           // first number of this launch's exchanges
+};
+struct ResidentOut {
+    double relres;
+    int64_t sumj;            // sum of the Arnoldi indices of all steps
+    uint64_t ns[RES_KINDS];
+    uint32_t count[RES_KINDS];
+    int status, iters, cycles, abort;
+};
+struct ResidentState {
+    ResidentIn in;
+    ResidentOut out;
+};
+struct ResidentArgs {
+    const uint32_t *sw, *so;
+    const int32_t *col;
+    const double *val64;
+    const float *val32;
+    const __half *val16;
+    const double *d;
+    double *u;               // iterate (first ldv entries) and, FP32 cycles, the FP64 residual
+    void *V, *Z;             // Krylov basis and preconditioned basis (the same: Jacobi in FP64)
+    uint64_t *xll, *ull, *red;   // tagged words: sweep vectors, iterate, sums
+    const ResidentIn *in;
+    ResidentOut *out;
+    int64_t ldv;
+    int n, nsl, spc, m, pdeg, smem;
+    unsigned timing;
+};
+
 }  // namespace apc
 
 struct apcloud_ctx {
@@ -232,6 +273,9 @@ struct apcloud_ctx {
     apc::DBuf pz0, pz1, pt;                         // polynomial preconditioner sweeps
     apc::DBuf zbasis;                               // preconditioned basis Z (flexible cycle end)
     apc::DBuf ell_rd;                               // reciprocal diagonals while the ELL is filled
+    // resident solves: tagged words, parameters and report, next unused tag
+    apc::DBuf res_words, res_state;
+    uint32_t res_tag = 1;
     // device staging for apcloud_field_host
     apc::DBuf hx, hy, hz, hq, hphi, hex, hey, hez;
     // error word, small host-visible values
@@ -305,6 +349,15 @@ apcloud_status build_stencils(apcloud_ctx *c);
 apcloud_status deposit(apcloud_ctx *c, const double *q, double q_uniform);
 apcloud_status gmres_solve(apcloud_ctx *c, int which, const double *b, double *x_inout_scaled, double rtol,
                            int max_iter, apcloud_solve_info *info);
+// Solves in one cooperative kernel (resident.cu); *ran is false when the
+// system is not one for it, and nothing has been done then
+apcloud_status resident_solve(apcloud_ctx *c, int which, const double *b, double *x, double rtol, int max_iter,
+                              apcloud_solve_info *info, bool *ran);
+apcloud_status resident_run(apcloud_ctx *c, ResidentArgs a, const double *b, double *x, double rtol, int max_iter,
+                            uint32_t *tag, int grid, bool graph, apcloud_solve_info *info, bool *ran);
+bool resident_ok(const apcloud_ctx *c, int which);
+void resident_grid(const apcloud_ctx *c, int *spc, int *grid);
+int64_t resident_red_words(int grid);
 bool ilu0_factor(int64_t n, const int64_t *rp, const int32_t *cj, const int64_t *dg, double *a);
 double *ilu_apply(apcloud_ctx *c, const IluDev &I, const double *v, double *z, const GmresState *st);
 apcloud_status spmv(apcloud_ctx *c, int which, const double *x, double *y, double scale, double *copy_out);

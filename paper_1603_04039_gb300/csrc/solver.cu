@@ -2785,6 +2785,11 @@ apcloud_status spmv(apcloud_ctx *c, int which, const double *x, double *y, doubl
 // restarted GMRES whose restarts recompute the residual in FP64.
 apcloud_status gmres_solve(apcloud_ctx *c, int which, const double *b, double *x, double rtol, int max_iter,
                            apcloud_solve_info *info) {
+    {
+        bool ran = false;
+        const apcloud_status st = resident_solve(c, which, b, x, rtol, max_iter, info, &ran);
+        if (st < 0 || ran) return st;
+    }
     const int n = c->n_tot;
     const int m = c->P.restart;
     const int64_t ldv = ((int64_t)n + 31) / 32 * 32;
@@ -3135,8 +3140,50 @@ extern "C" apcloud_status apcloud_solve_system_noalloc(apcloud_ctx *c, int which
                     "(precision %d, poly_degree %d, beams %d)", c->P.precision, c->P.poly_degree, c->nbeams);
     unsigned char *base = nullptr;
     APC_TRY(noalloc_base(c, &base));
-    // carve: state | basis | w | wraw | u | partials
     const int64_t ldv = ((int64_t)n + 31) / 32 * 32;
+    if (resident_ok(c, which)) {
+        // the resident solve of apcloud_solve_system with its buffers carved
+        // from the array; the tagged words are cleared at every call
+        int spc = 0, grid = 0;
+        resident_grid(c, &spc, &grid);
+        ResidentArgs a{};
+        a.sw = ptr<uint32_t>(c->slice_w);
+        a.so = ptr<uint32_t>(c->slice_off);
+        a.col = ptr<int32_t>(c->ell_col);
+        a.val64 = ptr<double>(which ? c->ell_A : c->ell_B);
+        a.d = ptr<double>(which ? c->dA : c->dB);
+        a.n = n;
+        a.nsl = c->n_slices;
+        a.spc = spc;
+        a.ldv = ldv;
+        a.m = m;
+        a.pdeg = 1;
+        size_t off = align256(sizeof(ResidentState));
+        ResidentState *rs = reinterpret_cast<ResidentState *>(base);
+        a.in = &rs->in;
+        a.out = &rs->out;
+        a.V = a.Z = base + off;
+        off = align256(off + sizeof(double) * (size_t)(m + 1) * ldv);
+        a.u = reinterpret_cast<double *>(base + off);
+        off = align256(off + sizeof(double) * 2 * (size_t)ldv);
+        const size_t words = off, nw = 4 * (size_t)n + (size_t)resident_red_words(grid);
+        a.ull = reinterpret_cast<uint64_t *>(base + off);
+        a.xll = a.ull + 2 * (size_t)n;
+        a.red = a.xll + 2 * (size_t)n;
+        off += nw * sizeof(uint64_t);
+        if (off <= NOALLOC_BYTES) {
+            const unsigned saved = c->timer.mask;   // event timers may allocate: off for this call
+            c->timer.mask = 0;
+            uint32_t tag = 1;
+            bool ran = false;
+            apcloud_status st = cuda_check(
+                c, cudaMemsetAsync(base + words, 0, nw * sizeof(uint64_t), c->s), "solve_system_noalloc");
+            if (st == APCLOUD_OK) st = resident_run(c, a, b, x, rtol, max_iter, &tag, grid, false, info, &ran);
+            c->timer.mask = saved;
+            if (st < 0 || ran) return st;
+        }
+    }
+    // carve: state | basis | w | wraw | u | partials
     const int nblk = reduction_blocks(c, n);
     size_t off = 0;
     GmresState *st = reinterpret_cast<GmresState *>(base + off);
