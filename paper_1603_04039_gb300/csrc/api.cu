@@ -274,13 +274,18 @@ apcloud_status read_back(apcloud_ctx *c, void *host, const void *dev, size_t byt
 apcloud_status check_device_errors(apcloud_ctx *c) {
     unsigned e[4];
     APC_TRY(read_back(c, e, c->derr.p, sizeof e));
+    return device_errors(c, e[0]);
+}
+
+apcloud_status device_errors(apcloud_ctx *c, unsigned bits) {
+    const unsigned e[1] = {bits};
     if (e[0] & ERR_DOMAIN) return fail(c, APCLOUD_E_DOMAIN, "a particle position is outside the domain or NaN");
     if (e[0] & ERR_OVERFLOW)
         return fail(c, APCLOUD_E_STENCIL, "a k-ring holds more than %d candidates", MAXC);
     if (e[0] & ERR_STENCIL)
         return fail(c, APCLOUD_E_STENCIL, "a node has no full-rank stencil within ring %d", c->P.ring_max);
     if (e[0] & ERR_BALANCE) return fail(c, APCLOUD_E_INVALID, "internal: 2:1 balance violated");
-    if (e[0] & ERR_TIMEOUT) return fail(c, APCLOUD_E_TIMEOUT, "a kernel gave up waiting for its bulk copy");
+    if (e[0] & ERR_TIMEOUT) return fail(c, APCLOUD_E_TIMEOUT, "a kernel gave up waiting for another block");
     return APCLOUD_OK;
 }
 
@@ -380,9 +385,9 @@ apcloud_status apcloud_create(const apcloud_params *params, const apcloud_alloca
 void apcloud_destroy(apcloud_ctx *c) {
     if (!c) return;
     cudaStreamSynchronize(c->s);
-    DBuf *bufs[] = {&c->key[0], &c->key[1], &c->val[0], &c->val[1], &c->ucell[0], &c->ucell[1], &c->ustart[0],
-                    &c->ustart[1], &c->opened, &c->cand[0], &c->cand[1], &c->cval[0], &c->cval[1], &c->flags,
-                    &c->scan, &c->scan_blk, &c->lkey, &c->lval, &c->leaf_anchor, &c->leaf_level, &c->leaf_first,
+    DBuf *bufs[] = {&c->key[0], &c->key[1], &c->val[0], &c->val[1], &c->opened,
+                    &c->cand[0], &c->cand[1], &c->cval[0], &c->cval[1], &c->flags,
+                    &c->scan, &c->scan_blk, &c->bkt, &c->leaf_anchor, &c->leaf_level, &c->leaf_first,
                     &c->leaf_count, &c->pleaf, &c->spos, &c->qsort, &c->node_ic, &c->bowner, &c->bface, &c->bidx, &c->adj, &c->nbr, &c->msz,
                     &c->ring, &c->lap, &c->lapd, &c->D, &c->rcond, &c->slice_w, &c->slice_off, &c->ell_col,
                     &c->ell_A, &c->ell_B, &c->dA, &c->dB, &c->V, &c->w0, &c->w1, &c->u, &c->b, &c->partial,

@@ -29,29 +29,12 @@ enum Kind {
 static_assert(NKIND == APCLOUD_NUM_KINDS, "kind count");
 
 // device error word bits
-enum : unsigned { ERR_DOMAIN = 1u, ERR_STENCIL = 2u, ERR_BALANCE = 4u, ERR_OVERFLOW = 8u, ERR_TIMEOUT = 16u };
+enum : unsigned { ERR_DOMAIN = 1u, ERR_STENCIL = 2u, ERR_BALANCE = 4u, ERR_OVERFLOW = 8u, ERR_TIMEOUT = 16u, ERR_CELLS = 32u };
 
 struct DBuf {
     void *p = nullptr;
     size_t bytes = 0;
 };
-
-// Leaves are in Morton order and so are the particles, so the particle ranges
-// [first_j, first_j + count_j) of consecutive leaves tile the key-sorted
-// particles in order.  A warp can own 32 consecutive leaves (lane l holding
-// leaf j0 + l's first particle, INT_MAX past the last leaf) and stream their
-// particles coalesced.  The leaf of sorted particle i within such a group is
-// the last lane whose first is <= i; an empty leaf shares its first with the
-// next leaf and is never chosen.  All 32 lanes must call it.
-__device__ __forceinline__ int group_leaf(int my_first, int i) {
-    int lo = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-        const int f = __shfl_sync(0xffffffffu, my_first, lo + step);
-        if (f <= i) lo += step;
-    }
-    return lo;
-}
 
 // GMRES bookkeeping kept on the device so that a whole restart cycle runs
 // without host round trips.
@@ -230,13 +213,15 @@ struct apcloud_ctx {
     int64_t sum_m = 0;  // total stencil neighbours over interior nodes
     int64_t n_fp64_wls = 0;  // mixed form: stencils refactored in FP64
 
-    // sorted particle keys and permutation (result in key[kbuf], val[kbuf])
+    // sorted particle keys (32 or 64 bits) and permutation (result in key[kbuf], val[kbuf])
     apc::DBuf key[2], val[2];
     int kbuf = 0;
-    // tree temporaries
-    apc::DBuf ucell[2], ustart[2], opened, cand[2], cval[2], flags, scan, scan_blk, lkey, lval;
+    // tree temporaries: opened cells (hash table and list), leaves before and after
+    // their sort, look-back words (scan) and digit counts (flags) of the radix sort
+    apc::DBuf opened, cand[2], cval[2], flags, scan, scan_blk, bkt;
+    uint32_t rs_epoch = 0;   // last number used in the look-back words
     // nodes
-    apc::DBuf leaf_anchor, leaf_level, leaf_first, leaf_count, node_ic, bowner, bface, bidx, adj;
+    apc::DBuf leaf_anchor, leaf_level, leaf_first, leaf_count, node_ic, bowner, bface, bidx, adj;   // bidx: boundary faces per block and face
     apc::DBuf pleaf;   // leaf of every particle, in the caller's particle order
     apc::DBuf spos;    // key-sorted position of every particle, in the caller's order
     apc::DBuf qsort;   // charges in key-sorted order (deposit)
@@ -320,6 +305,7 @@ inline void account(apcloud_ctx *c, int kind, double bytes, double flops) {
 // read `bytes` from device to host on the context stream and synchronise
 apcloud_status read_back(apcloud_ctx *c, void *host, const void *dev, size_t bytes);
 apcloud_status check_device_errors(apcloud_ctx *c);
+apcloud_status device_errors(apcloud_ctx *c, unsigned bits);   // the same for an error word already read
 
 // ---- primitives (prims.cu) ----
 // exclusive scan of n uint32 values; writes the total to *d_total if non-null
@@ -328,6 +314,33 @@ apcloud_status scan_u32(apcloud_ctx *c, const uint32_t *in, uint32_t *out, int64
 // 0/1 = which of the two buffers holds the result
 apcloud_status radix_sort(apcloud_ctx *c, uint64_t *k0, uint32_t *v0, uint64_t *k1, uint32_t *v1, int64_t n,
                           int nbits, int *which);
+apcloud_status radix_sort(apcloud_ctx *c, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, int64_t n,
+                          int nbits, int *which);
+// the same for keys whose digits the kernel that wrote them has counted
+// (clear_radix_counts first, then rs_count / rs_flush below); the values are
+// the positions 0 .. n - 1 (v0 is not read)
+constexpr int RS_BITS = 9, RS_BINS = 1 << RS_BITS, RS_MAX_PASS = 8;
+struct RadixDigits {
+    int passes;
+    int shift[RS_MAX_PASS], bits[RS_MAX_PASS];
+};
+RadixDigits radix_digits(int nbits);
+uint32_t *radix_counts(apcloud_ctx *c, const RadixDigits &dg);
+apcloud_status clear_radix_counts(apcloud_ctx *c, const RadixDigits &dg);
+template <class K>
+apcloud_status radix_sort_counted(apcloud_ctx *c, K *k0, uint32_t *v0, K *k1, uint32_t *v1, int64_t n,
+                                  const RadixDigits &dg, int *which);
+// the block's digit counts in shared memory, [pass][RS_BINS]
+template <class K>
+__device__ __forceinline__ void rs_count(K key, const RadixDigits &dg, uint32_t *h) {
+#pragma unroll
+    for (int p = 0; p < RS_MAX_PASS; ++p)
+        if (p < dg.passes) atomicAdd(&h[p * RS_BINS + ((uint32_t)(key >> dg.shift[p]) & ((1u << dg.bits[p]) - 1u))], 1u);
+}
+__device__ __forceinline__ void rs_flush(const uint32_t *h, const RadixDigits &dg, uint32_t *hist) {
+    for (int i = threadIdx.x; i < dg.passes * RS_BINS; i += blockDim.x)
+        if (h[i]) atomicAdd(hist + i, h[i]);
+}
 
 // ---- stages ----
 apcloud_status build_octree(apcloud_ctx *c, const double *x, const double *y, const double *z, int64_t n,

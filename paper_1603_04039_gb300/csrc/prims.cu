@@ -4,6 +4,8 @@
 // the primitives it (and the node ordering) is built from.  Both are written
 // for determinism: the scan is a fixed two-phase tree (integer sums, exact in
 // any order), the sort is stable.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace apc {
@@ -90,112 +92,266 @@ __global__ void k_scan_down(const uint32_t *__restrict__ in, uint32_t *__restric
 }
 
 // ---------------------------------------------------------------- radix sort
-constexpr int RS_T = 256;         // threads per block
-constexpr int RS_I = 8;           // keys per thread
-constexpr int RS_TILE = RS_T * RS_I;
-constexpr int RS_BITS = 8;
-constexpr int RS_BINS = 1 << RS_BITS;
+// Stable LSD sort of (key, value) pairs, one kernel per digit after one pass
+// that counts every digit at once (the counts of a digit do not depend on the
+// order of the keys).  A block takes the next tile of the input, orders it by
+// digit in shared memory and learns where each of its digits' runs goes from
+// the tiles before it by decoupled look-back (Merrill and Garland, "Single-
+// pass parallel prefix scan with decoupled look-back", 2016; Adinets and
+// Merrill, "Onesweep", 2022): it publishes its own counts at once, adds up its
+// predecessors' until it meets one that already knows its inclusive sum, and
+// publishes its own.  Tiles are handed out by a counter, so the tiles a block
+// waits for are always running.
+//
+// Against a histogram, a scan and a scatter kernel per digit (keys read twice,
+// 256 x tiles counts written, scanned and read): 24 instead of 32 bytes per
+// pair and digit, 16 with 32-bit keys, digits of up to 9 bits instead of 8
+// and P + 2 launches instead of 4 P.
+constexpr int RS_T = 512;         // threads per block
+// pairs per thread: 12 are the faster for many tiles, 8 for a few (two blocks
+// per SM either way).  2e7 / 1e5 pairs, all passes: 585 / 84 us at 12, 647 / 67
+// at 8; one block per SM (no register bound) 800 us.
+constexpr int RS_I_FEW = 8, RS_I_MANY = 12;
+constexpr int64_t RS_MANY = 4 << 20;
+constexpr int RS_W = RS_T / 32;
+constexpr int RS_LOOK = 8;        // predecessors polled at once
+static_assert(RS_BINS == RS_T, "one digit per thread");
+constexpr unsigned RS_SPIN = 1u << 22;   // polls of one predecessor before the sort is given up
 
-__global__ void k_rs_hist(const uint64_t *__restrict__ keys, int64_t n, int shift, uint32_t mask,
-                          uint32_t *__restrict__ hist, int nblk) {
-    __shared__ uint32_t h[RS_BINS];
-    for (int i = threadIdx.x; i < RS_BINS; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-#pragma unroll
-    for (int i = 0; i < RS_I; ++i) {
-        int64_t idx = base + (int64_t)i * RS_T + threadIdx.x;
-        if (idx < n) atomicAdd(&h[(uint32_t)(keys[idx] >> shift) & mask], 1u);
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < RS_BINS; d += blockDim.x) hist[(int64_t)d * nblk + blockIdx.x] = h[d];
+// status word of (tile, digit): the pass's number and the kind of sum above
+// the value; a number is never used twice with the same words
+__device__ __forceinline__ uint64_t rs_word(uint32_t epoch, uint32_t inclusive, uint32_t v) {
+    return (uint64_t)(epoch << 1 | inclusive) << 32 | v;
+}
+__device__ __forceinline__ void rs_put(uint64_t *p, uint64_t w) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ uint64_t rs_get(const uint64_t *p) {
+    uint64_t w;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+    return w;
 }
 
-// Stable scatter: warp w of the block owns keys [w*256, w*256+256) of the
-// tile and walks them 32 at a time in index order; equal digits inside a
-// step are ranked by lane with __match_any_sync.  The tile is then ordered
-// by digit in shared memory (same order inside a digit: warp, step, lane)
-// and written out with consecutive threads on consecutive destinations, so
-// the writes of a digit's run land together instead of one 8-byte key per
-// lane in 32 places.
-__global__ void __launch_bounds__(RS_T) k_rs_scatter(const uint64_t *__restrict__ kin,
-                                                     const uint32_t *__restrict__ vin, uint64_t *__restrict__ kout,
-                                                     uint32_t *__restrict__ vout, int64_t n, int shift, uint32_t mask,
-                                                     const uint32_t *__restrict__ offs, int nblk) {
-    static_assert(RS_T == RS_BINS, "one digit per thread in the block scan");
-    __shared__ uint32_t cnt[RS_T / 32][RS_BINS];
-    __shared__ uint32_t loc[RS_BINS], gof[RS_BINS], wtot[RS_T / 32];
-    __shared__ uint64_t sk[RS_TILE];
-    __shared__ uint32_t sv[RS_TILE];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
-    for (int i = tid; i < (RS_T / 32) * RS_BINS; i += blockDim.x) (&cnt[0][0])[i] = 0;
+// exclusive sum over the block of one value per thread
+__device__ __forceinline__ uint32_t rs_block_excl(uint32_t v, uint32_t *wtot) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t inc = warp_incl_scan(v);
+    if (lane == 31) wtot[w] = inc;
     __syncthreads();
-    const int64_t tile0 = (int64_t)blockIdx.x * RS_TILE;
+    uint32_t base = 0;
+#pragma unroll
+    for (int q = 0; q < RS_W; ++q)
+        if (q < w) base += wtot[q];
+    __syncthreads();
+    return base + inc - v;
+}
+
+// every digit's counts, [pass][RS_BINS]
+template <class K>
+__global__ void __launch_bounds__(RS_T) k_rs_hist(const K *__restrict__ keys, int64_t n, RadixDigits dg,
+                                                  uint32_t *__restrict__ hist) {
+    __shared__ uint32_t h[RS_MAX_PASS * RS_BINS];
+    for (int i = threadIdx.x; i < dg.passes * RS_BINS; i += RS_T) h[i] = 0;
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * RS_T + threadIdx.x; i < n; i += (int64_t)gridDim.x * RS_T)
+        rs_count(keys[i], dg, h);
+    __syncthreads();
+    rs_flush(h, dg, hist);
+}
+
+template <class K, int RS_I>
+struct RsShared {
+    K sk[RS_T * RS_I];
+    uint32_t sv[RS_T * RS_I];
+    uint16_t cnt[RS_W][RS_BINS];
+    uint32_t loc[RS_BINS], gof[RS_BINS], wtot[RS_W];
+    uint32_t tile;
+};
+
+// One digit.  Warp w of the block owns the w-th part of the tile and walks it
+// 32 pairs at a time in index order; equal digits inside a step are
+// ranked by lane.  IOTA: the values are the pairs' positions.
+template <class K, bool IOTA, int RS_I>
+__global__ void __launch_bounds__(RS_T, 2) k_rs_pass(const K *__restrict__ kin, const uint32_t *__restrict__ vin,
+                                                  K *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n,
+                                                  int shift, uint32_t mask, const uint32_t *__restrict__ hist,
+                                                  uint32_t *__restrict__ ticket, uint64_t *__restrict__ status,
+                                                  uint32_t epoch, unsigned *__restrict__ err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int RS_TILE = RS_T * RS_I;
+    RsShared<K, RS_I> &S = *reinterpret_cast<RsShared<K, RS_I> *>(smem);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
+    if (tid == 0) S.tile = atomicAdd(ticket, 1u);
+    for (int i = tid; i < RS_W * RS_BINS / 2; i += RS_T) reinterpret_cast<uint32_t *>(&S.cnt[0][0])[i] = 0u;
+    // where the digit's keys start in the output
+    const uint32_t first = rs_block_excl(hist[tid], S.wtot);   // ends with a barrier
+    const int64_t tile = S.tile, tile0 = tile * RS_TILE;
     const int64_t base = tile0 + (int64_t)w * (32 * RS_I);
     const unsigned lt = (1u << lane) - 1u;
-    uint64_t k[RS_I];
+    K k[RS_I];
     uint32_t v[RS_I];
     uint32_t d[RS_I], r[RS_I];
 #pragma unroll
     for (int i = 0; i < RS_I; ++i) {
-        int64_t idx = base + i * 32 + lane;
-        bool ok = idx < n;
-        k[i] = ok ? kin[idx] : 0ull;
-        v[i] = ok ? vin[idx] : 0u;
-        d[i] = ok ? ((uint32_t)(k[i] >> shift) & mask) : RS_BINS;   // RS_BINS = not a key
-        unsigned peers = __match_any_sync(0xffffffffu, d[i]);
+        const int64_t idx = base + i * 32 + lane;
+        const bool ok = idx < n;
+        k[i] = ok ? kin[idx] : (K)0;
+        v[i] = IOTA ? (uint32_t)idx : (ok ? vin[idx] : 0u);
+        d[i] = ok ? ((uint32_t)(k[i] >> shift) & mask) : RS_BINS;   // RS_BINS: not a key
+    }
+#pragma unroll
+    for (int i = 0; i < RS_I; ++i) {
+        const bool ok = d[i] < RS_BINS;
+        const unsigned peers = __match_any_sync(0xffffffffu, d[i]);
         uint32_t before = 0;
-        if (ok) before = cnt[w][d[i]];
+        if (ok) before = S.cnt[w][d[i]];
         __syncwarp();
-        if (ok && lane == __ffs(peers) - 1) cnt[w][d[i]] = before + __popc(peers);
+        if (ok && lane == __ffs(peers) - 1) S.cnt[w][d[i]] = (uint16_t)(before + __popc(peers));
         __syncwarp();
         r[i] = before + __popc(peers & lt);
     }
     __syncthreads();
-    // digit tid: prefix over warps inside the block, the digit's total, and
-    // the block's first destination for it
+    // digit tid: prefix over the warps, the tile's count, published at once
     uint32_t tot = 0;
 #pragma unroll
-    for (int ww = 0; ww < RS_T / 32; ++ww) {
-        const uint32_t t = cnt[ww][tid];
-        cnt[ww][tid] = tot;
+    for (int q = 0; q < RS_W; ++q) {
+        const uint32_t t = S.cnt[q][tid];
+        S.cnt[q][tid] = (uint16_t)tot;
         tot += t;
     }
-    gof[tid] = offs[(int64_t)tid * nblk + blockIdx.x];
-    // exclusive scan of the digit totals over the block: where each digit's
-    // run starts in the staged tile
-    uint32_t incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) wtot[w] = incl;
-    __syncthreads();
-    uint32_t wbase = 0;
-    for (int ww = 0; ww < w; ++ww) wbase += wtot[ww];
-    loc[tid] = wbase + incl - tot;
+    rs_put(status + tile * RS_BINS + tid, rs_word(epoch, tile == 0 ? 1u : 0u, tot));
+    // where each digit's run starts in the staged tile
+    S.loc[tid] = rs_block_excl(tot, S.wtot);   // ends with a barrier
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < RS_I; ++i) {
         if (d[i] < RS_BINS) {
-            const uint32_t lp = loc[d[i]] + cnt[w][d[i]] + r[i];
-            sk[lp] = k[i];
-            sv[lp] = v[i];
+            const uint32_t lp = S.loc[d[i]] + S.cnt[w][d[i]] + r[i];
+            S.sk[lp] = k[i];
+            S.sv[lp] = v[i];
         }
     }
+    // look back: the counts of the digit in the tiles before this one, RS_LOOK
+    // polls in flight (the tiles of the first wave all publish at once, and
+    // the last of them has to pass half of them one by one)
+    uint32_t excl = 0;
+    if (tile > 0) {
+        unsigned spins = 0;
+        bool found = false;
+        for (int64_t t = tile - 1; !found;) {
+            uint64_t q[RS_LOOK];
+#pragma unroll
+            for (int u = 0; u < RS_LOOK; ++u) q[u] = t >= u ? rs_get(status + (t - u) * RS_BINS + tid) : 0ull;
+            int used = 0;
+#pragma unroll
+            for (int u = 0; u < RS_LOOK; ++u) {
+                const uint32_t tag = (uint32_t)(q[u] >> 32);
+                if (!found && used == u && tag >> 1 == epoch) {
+                    excl += (uint32_t)q[u];
+                    found = tag & 1u;   // tile 0 publishes an inclusive sum
+                    ++used;
+                }
+            }
+            t -= used;
+            if (used == 0 && ++spins > RS_SPIN) {   // the output stays in bounds whatever the offsets (see below)
+                atomicOr(err, ERR_TIMEOUT);
+                break;
+            }
+        }
+        rs_put(status + tile * RS_BINS + tid, rs_word(epoch, 1u, excl + tot));
+    }
+    S.gof[tid] = first + excl;
     __syncthreads();
     const int m = (int)((n - tile0) < RS_TILE ? (n - tile0) : RS_TILE);
     for (int j = tid; j < m; j += RS_T) {
-        const uint64_t kk = sk[j];
+        const K kk = S.sk[j];
         const uint32_t dg = (uint32_t)(kk >> shift) & mask;
-        const uint32_t dst = gof[dg] + (uint32_t)j - loc[dg];
-        kout[dst] = kk;
-        vout[dst] = sv[j];
+        const uint32_t dst = S.gof[dg] + (uint32_t)j - S.loc[dg];
+        if (dst < n) {
+            kout[dst] = kk;
+            vout[dst] = S.sv[j];
+        }
     }
 }
 
+template <class K, int RS_I>
+apcloud_status sort_passes_of(apcloud_ctx *c, K *k0, uint32_t *v0, K *k1, uint32_t *v1, int64_t n, const RadixDigits &dg,
+                           bool counted, bool iota, int *which) {
+    *which = 0;
+    const int ntile = div_up(n, RS_T * RS_I);
+    uint32_t *hist = radix_counts(c, dg);
+    if (!hist) return APCLOUD_E_NOMEM;
+    const size_t words = (size_t)ntile * RS_BINS;
+    const bool fresh = !c->scan.p || c->scan.bytes < words * 8;
+    uint64_t *status = ensure<uint64_t>(c, c->scan, words);
+    if (!status) return APCLOUD_E_NOMEM;
+    if (fresh || c->rs_epoch > 0x7FFFFF00u) {
+        APC_CUDA(c, cudaMemsetAsync(status, 0, c->scan.bytes, c->s));
+        c->rs_epoch = 0;
+    }
+    if (!counted) {
+        APC_TRY(clear_radix_counts(c, dg));
+        const int nb = std::min(div_up(n, RS_T * 4), 608);
+        APC_LAUNCH(c, K_SORT, nb, RS_T, 0, k_rs_hist<K>, (const K *)k0, n, dg, hist);
+        account(c, K_SORT, (double)sizeof(K) * n, 0.0);
+    }
+    uint32_t *ticket = hist + (size_t)dg.passes * RS_BINS;
+    unsigned *derr = ptr<unsigned>(c->derr);
+    const int smem = (int)sizeof(RsShared<K, RS_I>);
+    APC_CUDA(c, cudaFuncSetAttribute(k_rs_pass<K, false, RS_I>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    APC_CUDA(c, cudaFuncSetAttribute(k_rs_pass<K, true, RS_I>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    K *ka = k0, *kb = k1;
+    uint32_t *va = v0, *vb = v1;
+    for (int p = 0; p < dg.passes; ++p) {
+        const int sh = dg.shift[p];
+        const uint32_t mask = (1u << dg.bits[p]) - 1u;
+        const uint32_t *hp = hist + (size_t)p * RS_BINS;
+        const uint32_t epoch = ++c->rs_epoch;
+        if (iota && p == 0)
+            APC_LAUNCH(c, K_SORT, ntile, RS_T, smem, (k_rs_pass<K, true, RS_I>), (const K *)ka, (const uint32_t *)va, kb, vb,
+                       n, sh, mask, hp, ticket + p, status, epoch, derr);
+        else
+            APC_LAUNCH(c, K_SORT, ntile, RS_T, smem, (k_rs_pass<K, false, RS_I>), (const K *)ka, (const uint32_t *)va, kb,
+                       vb, n, sh, mask, hp, ticket + p, status, epoch, derr);
+        account(c, K_SORT, (2.0 * sizeof(K) + (iota && p == 0 ? 4.0 : 8.0)) * n, 0.0);
+        std::swap(ka, kb);
+        std::swap(va, vb);
+    }
+    *which = dg.passes & 1;
+    return cuda_check(c, cudaGetLastError(), "radix_sort");
+}
+
+template <class K>
+apcloud_status sort_passes(apcloud_ctx *c, K *k0, uint32_t *v0, K *k1, uint32_t *v1, int64_t n, const RadixDigits &dg,
+                           bool counted, bool iota, int *which) {
+    return n >= RS_MANY ? sort_passes_of<K, RS_I_MANY>(c, k0, v0, k1, v1, n, dg, counted, iota, which)
+                        : sort_passes_of<K, RS_I_FEW>(c, k0, v0, k1, v1, n, dg, counted, iota, which);
+}
+
 }  // namespace
+
+RadixDigits radix_digits(int nbits) {
+    RadixDigits d{};
+    d.passes = (nbits + RS_BITS - 1) / RS_BITS;
+    for (int p = 0, at = 0; p < d.passes; ++p) {   // digits as equal as they get
+        d.bits[p] = (nbits - at + d.passes - p - 1) / (d.passes - p);
+        d.shift[p] = at;
+        at += d.bits[p];
+    }
+    return d;
+}
+
+uint32_t *radix_counts(apcloud_ctx *c, const RadixDigits &dg) {
+    (void)dg;
+    return ensure<uint32_t>(c, c->flags, RS_MAX_PASS * (RS_BINS + 1));
+}
+
+// zero counts, and the passes' tile counters behind them
+apcloud_status clear_radix_counts(apcloud_ctx *c, const RadixDigits &dg) {
+    uint32_t *h = radix_counts(c, dg);
+    if (!h) return APCLOUD_E_NOMEM;
+    return cuda_check(c, cudaMemsetAsync(h, 0, sizeof(uint32_t) * dg.passes * (RS_BINS + 1), c->s), "radix_sort");
+}
 
 apcloud_status scan_u32(apcloud_ctx *c, const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total) {
     if (n <= 0) {
@@ -218,27 +374,25 @@ apcloud_status radix_sort(apcloud_ctx *c, uint64_t *k0, uint32_t *v0, uint64_t *
                           int nbits, int *which) {
     *which = 0;
     if (n <= 1 || nbits <= 0) return APCLOUD_OK;
-    int nblk = div_up(n, RS_TILE);
-    int64_t nh = (int64_t)RS_BINS * nblk;
-    uint32_t *hist = ensure<uint32_t>(c, c->flags, nh);
-    uint32_t *offs = ensure<uint32_t>(c, c->scan, nh);
-    if (!hist || !offs) return APCLOUD_E_NOMEM;
-    uint64_t *ka = k0, *kb = k1;
-    uint32_t *va = v0, *vb = v1;
-    int cur = 0;
-    for (int shift = 0; shift < nbits; shift += RS_BITS) {
-        int bits = nbits - shift < RS_BITS ? nbits - shift : RS_BITS;
-        uint32_t mask = (1u << bits) - 1u;
-        APC_LAUNCH(c, K_SORT, nblk, RS_T, 0, k_rs_hist, ka, n, shift, mask, hist, nblk);
-        APC_TRY(scan_u32(c, hist, offs, nh, nullptr));
-        APC_LAUNCH(c, K_SORT, nblk, RS_T, 0, k_rs_scatter, ka, va, kb, vb, n, shift, mask, offs, nblk);
-        account(c, K_SORT, 32.0 * n, 0.0);   // key read for the histogram, key+value read and write
-        uint64_t *tk = ka; ka = kb; kb = tk;
-        uint32_t *tv = va; va = vb; vb = tv;
-        cur ^= 1;
-    }
-    *which = cur;
-    return cuda_check(c, cudaGetLastError(), "radix_sort");
+    return sort_passes<uint64_t>(c, k0, v0, k1, v1, n, radix_digits(nbits), false, false, which);
 }
+
+apcloud_status radix_sort(apcloud_ctx *c, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, int64_t n,
+                          int nbits, int *which) {
+    *which = 0;
+    if (n <= 1 || nbits <= 0) return APCLOUD_OK;
+    return sort_passes<uint32_t>(c, k0, v0, k1, v1, n, radix_digits(nbits), false, false, which);
+}
+
+// keys counted already (rs_count / rs_flush into radix_counts), values 0 .. n - 1
+template <class K>
+apcloud_status radix_sort_counted(apcloud_ctx *c, K *k0, uint32_t *v0, K *k1, uint32_t *v1, int64_t n,
+                                  const RadixDigits &dg, int *which) {
+    return sort_passes<K>(c, k0, v0, k1, v1, n, dg, true, true, which);
+}
+template apcloud_status radix_sort_counted<uint32_t>(apcloud_ctx *, uint32_t *, uint32_t *, uint32_t *, uint32_t *,
+                                                     int64_t, const RadixDigits &, int *);
+template apcloud_status radix_sort_counted<uint64_t>(apcloud_ctx *, uint64_t *, uint32_t *, uint64_t *, uint32_t *,
+                                                     int64_t, const RadixDigits &, int *);
 
 }  // namespace apc
