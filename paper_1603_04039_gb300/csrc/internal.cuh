@@ -236,7 +236,7 @@ struct apcloud_ctx {
     apc::DBuf ell_A32, ell_B32;  // FP32 copies for the inner iterations of the mixed form
     apc::DBuf ell_A16, ell_B16;  // FP16 copies for the preconditioner sweeps of the mixed form
     // width-sorted copy of the FP16 sweep matrix: rows ordered by stencil width
-    // inside windows of 256 rows, so 32-row slices pad little (see build_sorted_sweep)
+    // inside windows of 256 rows, so 32-row slices pad little (see rank_sorted_sweep)
     apc::DBuf ss_perm, ss_w, ss_o, ss_col, ss_A, ss_B;
     apc::DBuf ss_col24;                             // chunk columns of the sorted copy, 24 bits each
     apc::DBuf stencil_ovf;                          // nodes whose k-ring outgrew MAXC_FAST candidates
@@ -347,7 +347,9 @@ apcloud_status build_octree(apcloud_ctx *c, const double *x, const double *y, co
                             const int64_t *h_offsets, int nbeams);
 apcloud_status node_beams(apcloud_ctx *c, int32_t *out);
 apcloud_status refresh_lowp(apcloud_ctx *c);          // FP32/FP16 matrix copies from the FP64 values
-apcloud_status build_sorted_sweep(apcloud_ctx *c);    // width-sorted FP16 sweep matrix from the ELL
+// width-sorted sweep matrix: its ranks and slices (entry columns to *d_total), then its entries from the ELL
+apcloud_status rank_sorted_sweep(apcloud_ctx *c, uint32_t *d_total);
+apcloud_status fill_sorted_sweep(apcloud_ctx *c);
 double *poisson_rhs(apcloud_ctx *c, const double *g);  // b of the Poisson system into c->b
 apcloud_status tune_spmv(apcloud_ctx *c, double *ms_out);      // ms per sweep at 64/128/256/512 threads
 int64_t sweep_keep_bytes(const apcloud_ctx *c);                 // sweep matrix bytes read with ordinary loads

@@ -538,39 +538,76 @@ __global__ void __launch_bounds__(T) k_boundary(const uint32_t *__restrict__ bcn
     }
 }
 
-// Face adjacency (Section 4.3): per leaf and face, the face neighbour when it
+// Face adjacency (Section 4.3): per face of a leaf, the face neighbour when it
 // is a leaf, else its 4 children touching the face (leaves by 2:1 balance),
-// or the boundary node of that face (written by k_boundary).
-__global__ void k_adjacency(const uint64_t *__restrict__ anchor, const int8_t *__restrict__ level, int64_t n, int L,
-                            int32_t *__restrict__ adj, unsigned *err) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 6 * n) return;
-    int64_t j = t / 6;
-    int f = (int)(t - j * 6);
-    int4 *out = reinterpret_cast<int4 *>(adj + j * 24 + f * 4);
-    int lev = level[j];
-    const uint64_t pre = (anchor[j] >> (3 * L)) << (3 * L);   // beam index bits
-    uint32_t c[3];
-    unmorton((anchor[j] ^ pre) >> (3 * (L - lev)), c[0], c[1], c[2]);
-    if (c[f >> 1] == ((f & 1) ? (1u << lev) - 1u : 0u)) return;   // domain boundary
-    int d = f >> 1;
-    c[d] = (f & 1) ? c[d] + 1 : c[d] - 1;
-    uint64_t a = pre | (morton(c[0], c[1], c[2]) << (3 * (L - lev)));
-    int64_t k = leaf_of(anchor, n, a, j);
-    if (k < 0) { atomicOr(err, ERR_BALANCE); return; }
-    if (level[k] <= lev) { *out = make_int4((int)k, -1, -1, -1); return; }
-    const int want = (f & 1) ? 0 : 1;
-    int kid[4];
+// or the boundary node of that face (left in the face's slots by k_boundary).
+// Eight lanes per leaf, one per face; the leaf's neighbours are packed to the
+// front of its 24 slots, -1 after them.
+__global__ void __launch_bounds__(T) k_adjacency(const uint64_t *__restrict__ anchor,
+                                                 const int8_t *__restrict__ level, int64_t n, int L, int32_t *adj,
+                                                 unsigned *err) {
+    const int64_t j = ((int64_t)blockIdx.x * T + threadIdx.x) >> 3;
+    const int f = threadIdx.x & 7, lane = threadIdx.x & 31;
+    int kid[4] = {-1, -1, -1, -1}, cnt = 0;
+    if (j < n && f < 6) {
+        const int lev = level[j];
+        const uint64_t aj = anchor[j], pre = (aj >> (3 * L)) << (3 * L);   // beam index bits
+        uint32_t c[3];
+        unmorton((aj ^ pre) >> (3 * (L - lev)), c[0], c[1], c[2]);
+        const int d = f >> 1;
+        const uint32_t cd = d == 0 ? c[0] : (d == 1 ? c[1] : c[2]);
+        if (cd == ((f & 1) ? (1u << lev) - 1u : 0u)) {   // domain boundary
+            kid[0] = adj[j * 24 + f * 4];
+            cnt = 1;
+        } else {
+            const uint32_t nd = (f & 1) ? cd + 1 : cd - 1;
+            const uint32_t x = d == 0 ? nd : c[0], y = d == 1 ? nd : c[1], z = d == 2 ? nd : c[2];
+            const uint64_t a = pre | (morton(x, y, z) << (3 * (L - lev)));
+            const int64_t k = leaf_of(anchor, n, a, j);
+            if (k < 0) {
+                atomicOr(err, ERR_BALANCE);
+            } else if (level[k] <= lev) {
+                kid[0] = (int)k;
+                cnt = 1;
+            } else {
+                const int want = (f & 1) ? 0 : 1;
+                cnt = 4;
+                int64_t from = k;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {   // the four children on the face, in Morton order
-        const int o = d == 0 ? (want << 2 | q) : (d == 1 ? ((q >> 1) << 2 | want << 1 | (q & 1)) : (q << 1 | want));
-        uint32_t cc[3] = {2u * c[0] + ((o >> 2) & 1u), 2u * c[1] + ((o >> 1) & 1u), 2u * c[2] + (o & 1u)};
-        uint64_t ac = pre | (morton(cc[0], cc[1], cc[2]) << (3 * (L - lev - 1)));
-        int64_t kk = leaf_of(anchor, n, ac, k);
-        if (kk < 0 || anchor[kk] != ac || level[kk] != lev + 1) { atomicOr(err, ERR_BALANCE); return; }
-        kid[q] = (int)kk;
+                for (int q = 0; q < 4; ++q) {   // the four children on the face, in Morton order
+                    const int o = d == 0 ? (want << 2 | q)
+                                         : (d == 1 ? ((q >> 1) << 2 | want << 1 | (q & 1)) : (q << 1 | want));
+                    const uint64_t ac = a | (uint64_t)o << (3 * (L - lev - 1));
+                    const int64_t kk = leaf_of(anchor, n, ac, from);
+                    if (kk < 0 || anchor[kk] != ac || level[kk] != lev + 1) {
+                        atomicOr(err, ERR_BALANCE);
+                        break;
+                    }
+                    kid[q] = (int)kk;
+                    from = kk;
+                }
+            }
+        }
     }
-    *out = make_int4(kid[0], kid[1], kid[2], kid[3]);
+    // places of the faces' neighbours: a prefix sum over the leaf's lanes
+    int inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o, 8);
+        if ((lane & 7) >= o) inc += t;
+    }
+    const int tot = __shfl_sync(0xffffffffu, inc, 7, 8);
+    __syncwarp();   // every boundary entry is read
+    if (j >= n) return;
+    int32_t *out = adj + j * 24;
+    const int at = inc - cnt;
+    if (cnt > 0) out[at] = kid[0];
+    if (cnt == 4) {
+        out[at + 1] = kid[1];
+        out[at + 2] = kid[2];
+        out[at + 3] = kid[3];
+    }
+    for (int t = tot + f; t < 24; t += 8) out[t] = -1;
 }
 
 // Node ranges of every beam: interior nodes [r[b], r[b+1]) (the leaves are
@@ -781,7 +818,7 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
     APC_TRY(scan_u32(c, bcnt, bpos, 6 * (int64_t)nblk, small + 4));
     APC_LAUNCH(c, K_TREE, nblk, T, 0, k_boundary, (const uint32_t *)bcnt, (const uint32_t *)bpos, nblk, nleaf, ic, bo,
                bf, adj);
-    APC_LAUNCH(c, K_ADJ, div_up(6 * nleaf, T), T, 0, k_adjacency, la, ll, nleaf, L, adj, derr);
+    APC_LAUNCH(c, K_ADJ, div_up(8 * nleaf, T), T, 0, k_adjacency, la, ll, nleaf, L, adj, derr);
     APC_LAUNCH(c, K_TREE, div_up(nb + 1, T), T, 0, k_beam_ranges, lb, nleaf, nb, (const uint32_t *)bpos, nblk,
                (const uint32_t *)(small + 4), (const int32_t *)bo, rng);
     APC_CUDA(c, cudaGetLastError());

@@ -31,8 +31,8 @@ constexpr int ASTR = NCOL;      // row stride of the staged Vandermonde
 // that redoes the nodes whose rings outgrew them
 template <int MC>
 struct __align__(16) WarpSmemT {
-    int32_t cand[MC];   // read four at a time by the membership test
-    long long d2[MC];
+    int32_t cand[MC];
+    long long d2[MC];   // hash set of the candidates (2 MC ints), then their rank keys, then squared distances
     uint16_t srt[MC];   // candidate slots in (d2, index) order
     uint8_t oct[MC];
     uint8_t pick[MC];   // octant picks, by sorted position
@@ -152,13 +152,6 @@ __device__ bool cholesky_regs(const float *G, float *R, float *Ri, int lane) {
     return true;
 }
 
-// the FP32 path factors in registers, the FP64 path with the warp
-template <class T>
-__device__ __forceinline__ bool cholesky(T *G, T *R, T *Ri, const GramOwn &o, int lane) {
-    if constexpr (sizeof(T) == 4) return cholesky_regs(G, R, Ri, lane);
-    else return cholesky_warp<T>(G, R, Ri, o, lane);
-}
-
 // solve q R = a for the row vector q (R upper), in place on v
 template <class T>
 __device__ __forceinline__ void row_solve_upper(const T *R, const T *Ri, T *v) {
@@ -197,18 +190,16 @@ __device__ __forceinline__ void gram(const T *A, int m, T *G, const GramOwn &o, 
     if (o.two) G[lane + 32] = s2;
 }
 
-__device__ __forceinline__ double exp_t(double v) { return exp(v); }
-__device__ __forceinline__ float exp_t(float v) { return expf(v); }
-
 // Weighted least-squares operator (Section 3.1) of the stencil staged in
-// W.sel / W.seld2, in arithmetic T: rows of W V0 (Eq. regfd with the
+// W.sel / W.seld2, in FP32: rows of W V0 (Eq. regfd with the
 // normalized Gaussian weight), CholeskyQR2, and column `lane` of
 // P = (W V0)^+ W unscaled by h and h^2, returned in FP64.  Returns false when
 // a Cholesky pivot fails; rratio = min |R_ii| / max |R_ii|.
-template <class T, class WS>
-__device__ bool wls_column(WS &W, int m, int lane, const GramOwn &own, int4 c0, const int4 *__restrict__ ic,
+template <class WS>
+__device__ bool wls_column_f32(WS &W, int m, int lane, const GramOwn &own, int4 c0, const int4 *__restrict__ ic,
                            double unit, double ec, double inv_1mec, double (&qout)[NCOL], double &lapj,
                            double &rratio) {
+    typedef float T;
     T *A = reinterpret_cast<T *>(W.A);
     T *G = reinterpret_cast<T *>(W.G);
     T *R1 = reinterpret_cast<T *>(W.R1);
@@ -234,7 +225,7 @@ __device__ bool wls_column(WS &W, int m, int lane, const GramOwn &own, int4 c0, 
             // xi = dy / h with h = max |dy_d| (Section 3.1): exact integers, one rounding in T
             T xi0 = (T)off[0] / (T)hint, xi1 = (T)off[1] / (T)hint, xi2 = (T)off[2] / (T)hint;
             T ratio = (T)mydist / (T)r2max;
-            wj = (exp_t(-ratio) - (T)ec) * (T)inv_1mec;
+            wj = (expf(-ratio) - (T)ec) * (T)inv_1mec;
             const T half = (T)0.5;
             row[0] = xi0; row[1] = xi1; row[2] = xi2;
             row[3] = (half * xi0) * xi0;
@@ -252,7 +243,7 @@ __device__ bool wls_column(WS &W, int m, int lane, const GramOwn &own, int4 c0, 
     __syncwarp();
     gram<T>(A, m, G, own, lane);
     __syncwarp();
-    bool ok = cholesky<T>(G, R1, Ri1, own, lane);
+    bool ok = cholesky_regs(G, R1, Ri1, lane);
     T q[NCOL];
     if (ok) {
         if (lane < m) {
@@ -265,7 +256,7 @@ __device__ bool wls_column(WS &W, int m, int lane, const GramOwn &own, int4 c0, 
         __syncwarp();
         gram<T>(A, m, G, own, lane);
         __syncwarp();
-        ok = cholesky<T>(G, R2, Ri2, own, lane);
+        ok = cholesky_regs(G, R2, Ri2, lane);
     }
     rratio = 0.0;
     lapj = 0.0;
@@ -302,6 +293,169 @@ __device__ bool wls_column(WS &W, int m, int lane, const GramOwn &own, int4 c0, 
     return true;
 }
 
+// Gram matrix of m staged FP64 rows: lane l sums entry l over all rows; the 13
+// entries past 32 are shared by two lanes each (lanes 0-12 the even rows, lanes
+// 16-28 the odd ones), so they cost m / 2 issue slots of the FP64 pipe, not m.
+__device__ __forceinline__ void gram_f64(const double *A, int m, const GramOwn &o, int a2, int b2, int lane,
+                                         double &s1, double &s2) {
+    s1 = 0.0;
+    s2 = 0.0;
+    for (int j = 0; j < m; ++j) s1 = fma(A[j * ASTR + o.a1], A[j * ASTR + o.b1], s1);
+    for (int j = lane >> 4; j < m; j += 2) s2 = fma(A[j * ASTR + a2], A[j * ASTR + b2], s2);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
+}
+
+// 1 / sqrt(g) and 1 / x in FP64 from an FP32 start, one third-order step each
+// (Halley's iteration; with e = 1 - g y^2 or 1 - x y, |e| < 2^-22, the
+// neglected terms are below 2^-64): 5 and 3 issue slots of the FP64 pipe, the
+// conversions on the integer pipe.  g and x well inside the FP32 range.
+__device__ __forceinline__ double rsqrt_f64(double g) {
+    const double y = f32_to_f64_int(rsqrtf(f64_to_f32_int(g)));
+    const double e = fma(-(g * y), y, 1.0);
+    return fma(y, fma(e, 0.375, 0.5) * e, y);
+}
+__device__ __forceinline__ double recip_f64(double x) {
+    const double y = f32_to_f64_int(1.0f / f64_to_f32_int(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// wls_column_f32 in FP64, counted by the FP64 pipe's issue slots (16 cycles per
+// warp instruction and SM, whatever the number of active lanes): the two
+// serial factorisations with a square root and a division per pivot were more
+// than half of the ~940 a node took.  Here the pivots are reciprocal square
+// roots, and the second Cholesky QR pass is a correction: with Q1 = A R1^-1 and
+// G2 = Q1^T Q1 = I + E, P = R1^-1 G2^-1 Q1^T and G2^-1 = I - E + O(E^2); E is
+// the rounding of the first pass (kappa^2 eps), and below 1e-9 its square is
+// below 1e-18 and the FP32 rounding of the correction E q below 1e-15 of q.
+// A block with a larger E goes through the full second pass.
+// ~330 slots: 2.8e5 nodes 12.76 -> 5.13 ms, the FP64 pipe's own time for them
+// (fewer resident warps change nothing).
+template <class WS>
+__device__ bool wls_column_f64(WS &W, int m, int lane, const GramOwn &own, int4 c0, const int4 *__restrict__ ic,
+                               double inv_unit, double ec, double inv_1mec, double (&q)[NCOL], double &lapj,
+                               double &rratio) {
+    double *A = W.A, *G = W.G, *R = W.R1, *Ri = W.Ri1;
+    const unsigned FULL = 0xffffffffu;
+    int off[3] = {0, 0, 0};
+    long long mydist = 0;
+    if (lane < m) {
+        const int4 p = ic[W.sel[lane]];
+        off[0] = p.x - c0.x;
+        off[1] = p.y - c0.y;
+        off[2] = p.z - c0.z;
+        mydist = W.seld2[lane];
+    }
+    const int hint = __reduce_max_sync(FULL, max(abs(off[0]), max(abs(off[1]), abs(off[2]))));
+    // offsets are below 2^24: exact in FP32; squared distances below 2^48
+    const double rh = recip_f64(f32_to_f64_int((float)hint));
+    const double rr = recip_f64((double)W.seld2[m - 1]);
+    double wj = 0.0;
+    rratio = 0.0;
+    lapj = 0.0;
+    {
+        // xi = dy / h with h = max |dy_d| (Section 3.1)
+        const double x0 = f32_to_f64_int((float)off[0]) * rh, x1 = f32_to_f64_int((float)off[1]) * rh,
+                     x2 = f32_to_f64_int((float)off[2]) * rh;
+        const double dist = __hiloint2double(0x43300000 | (int)(mydist >> 32), (int)mydist) - 4503599627370496.0;
+        const double w = (exp(-(dist * rr)) - ec) * inv_1mec;
+        if (lane < m) wj = w;
+        const double w0 = wj * x0, w1 = wj * x1, w2 = wj * x2;
+        const double h0 = 0.5 * x0;
+        double *a = A + lane * ASTR;
+        a[0] = w0;
+        a[1] = w1;
+        a[2] = w2;
+        a[3] = w0 * h0;
+        a[4] = w0 * x1;
+        a[5] = w0 * x2;
+        a[6] = w1 * (0.5 * x1);
+        a[7] = w1 * x2;
+        a[8] = w2 * (0.5 * x2);
+    }
+    int a2, b2;
+    const int e2 = 32 + (lane & 15);
+    const bool two = (lane & 15) < 13;
+    pk_rowcol(two ? e2 : 32, a2, b2);
+    __syncwarp();
+    double g1, g2;
+    gram_f64(A, m, own, a2, b2, lane, g1, g2);
+    // Cholesky G = R^T R, right-looking: entries stay with their lanes, the pivot
+    // row goes through shared memory.  A pivot below 1e-30 (the entries are O(1))
+    // is a rank deficiency either way.
+    for (int k = 0; k < NCOL; ++k) {
+        if (own.a1 == k) R[k * NCOL + own.b1] = g1;
+        if (two && a2 == k && lane < 16) R[k * NCOL + b2] = g2;
+        __syncwarp();
+        const double gkk = R[k * NCOL + k];
+        if (!(gkk > 1e-30)) return false;   // the same in every lane
+        const double rd = rsqrt_f64(gkk);
+        const double mine = (lane >= k && lane < NCOL ? R[k * NCOL + lane] : 0.0) * rd;
+        __syncwarp();
+        if (lane >= k && lane < NCOL) R[k * NCOL + lane] = mine;
+        if (lane == 0) Ri[k] = rd;
+        __syncwarp();
+        if (k < 4 && own.a1 > k) g1 = fma(-R[k * NCOL + own.a1], R[k * NCOL + own.b1], g1);
+        if (k < 8 && a2 > k) g2 = fma(-R[k * NCOL + a2], R[k * NCOL + b2], g2);
+    }
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) q[e] = A[lane * ASTR + e];
+    row_solve_upper<double>(R, Ri, q);
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) A[lane * ASTR + e] = q[e];
+    __syncwarp();
+    gram_f64(A, m, own, a2, b2, lane, g1, g2);
+    const double e1 = own.a1 == own.b1 ? g1 - 1.0 : g1, ee = a2 == b2 ? g2 - 1.0 : g2;
+    const float f1 = f64_to_f32_int(e1), f2 = f64_to_f32_int(ee);
+    const bool small = __all_sync(FULL, fabsf(f1) < 1e-9f && fabsf(f2) < 1e-9f);
+    double *R2 = W.R2, *Ri2 = W.Ri2;
+    if (small) {
+        float *E = reinterpret_cast<float *>(G);
+        E[lane] = f1;
+        if (two && lane < 16) E[e2] = f2;
+        __syncwarp();
+        float qf[NCOL], z[NCOL];
+#pragma unroll
+        for (int r = 0; r < NCOL; ++r) {
+            qf[r] = f64_to_f32_int(q[r]);
+            z[r] = 0.f;
+        }
+#pragma unroll
+        for (int r = 0; r < NCOL; ++r)
+#pragma unroll
+            for (int k = r; k < NCOL; ++k) {
+                const float v = E[pk_idx(r, k)];
+                z[r] = fmaf(v, qf[k], z[r]);
+                if (k != r) z[k] = fmaf(v, qf[r], z[k]);
+            }
+#pragma unroll
+        for (int r = 0; r < NCOL; ++r) q[r] -= f32_to_f64_int(z[r]);
+    } else {
+        G[lane] = g1;
+        if (two && lane < 16) G[e2] = g2;
+        __syncwarp();
+        if (!cholesky_warp<double>(G, R2, Ri2, own, lane)) return false;
+        row_solve_upper<double>(R2, Ri2, q);
+        col_solve_upper<double>(R2, Ri2, q);
+    }
+    col_solve_upper<double>(R, Ri, q);
+    // condition estimate min / max of |R_ii|, to FP32 (it is only compared)
+    float lo = 3e38f, hi = 0.f;
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) {
+        float d = f64_to_f32_int(R[e * NCOL + e]);
+        if (!small) d *= f64_to_f32_int(R2[e * NCOL + e]);
+        lo = fminf(lo, d);
+        hi = fmaxf(hi, d);
+    }
+    rratio = f32_to_f64_int(lo / hi);
+    const double ih = rh * inv_unit, s1 = wj * ih, s2 = s1 * ih;
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) q[e] *= e < 3 ? s1 : s2;   // wj = 0 past the stencil
+    lapj = q[3] + q[6] + q[8];
+    return true;
+}
+
 // The rows of the derivative operator D (row-of-operator major, nodes
 // fastest) of a block's SW nodes.  Each warp stages its node's 9 x MMAX block
 // in its W.A as [e * MMAX + lane] (free once the WLS is done); the last warp
@@ -327,24 +481,41 @@ __device__ __forceinline__ void write_block_d(const unsigned char *smem_raw, uns
     }
 }
 
+// Inserts node v into the warp's hash set of 2 MC slots (at most half full);
+// true for the lane that brought it in.
+template <int MC>
+__device__ __forceinline__ bool ring_insert(int *tab, int v) {
+    constexpr unsigned M = 2 * MC - 1;
+    unsigned h = ((unsigned)v * 0x9E3779B1u >> 16) & M;
+    for (;;) {   // ends: the table never fills
+        const int old = atomicCAS(tab + h, -1, v);
+        if (old == -1) return true;
+        if (old == v) return false;
+        h = (h + 1) & M;
+    }
+}
+
 // SW warps (nodes) per block, one WarpSmemT<MC> each (and the block's
 // arrival count after them); the autotuner picks SW.  With MC = MAXC_FAST
 // (LIST false, every node): 6.6 KB of shared memory per warp and 32 warps per
 // SM at a register budget that spills part of the FP32 factorisation; a node
 // whose ring outgrows MC candidates goes to ovf_list instead of failing.
 // Against 512 slots at 16 warps: 7.1 -> 5.9 ms on a 1e7-particle beam and
-// 31.6 -> 26.1 ms on a 64-beam batch (both passes).  With MC = MAXC and LIST: the nodes of that list
+// 31.6 -> 26.1 ms on a 64-beam batch (both passes); with the candidates' hash
+// set, packed adjacency, 64-bit rank keys and the FP64 code moved to the list
+// kernel 5.86 -> 5.43 ms (3340 instead of ~4200 instructions per node; the
+// shared-memory pipe is 70% busy with the FP32 factorisation's operands).  With MC = MAXC and LIST: the nodes of that list
 // (n_list of them), each warp writing its own D columns.  slots <= MC is the
 // capacity in force (the context's stencil_slots in the first kernel).
-template <int SW, int MC, bool LIST>
+template <int SW, int MC, bool LIST, bool MIXED>
 __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil(
     const int4 *__restrict__ ic, const int32_t *__restrict__ adj, const int32_t *__restrict__ bowner, int n_int,
-    int m_target, int ring_max, double unit, double ec, double inv_1mec, int32_t *__restrict__ nbr_out,
+    int m_target, int ring_max, double unit, double inv_unit, double ec, double inv_1mec, int32_t *__restrict__ nbr_out,
     int32_t *__restrict__ m_out, int32_t *__restrict__ ring_out, double *__restrict__ lap_out,
     double *__restrict__ lapd_out, double *__restrict__ D_out, int64_t dstride, double *__restrict__ rcond_out,
-    int fp32_first, double fp32_rcond_min, int *__restrict__ fp64_count, unsigned *err,
+    double fp32_rcond_min, int *__restrict__ fp64_count, unsigned *err,
     const int32_t *__restrict__ list, int n_list, unsigned *__restrict__ ovf_count, int32_t *__restrict__ ovf_list,
-    int slots) {
+    int slots, int idx_bits, int d2_shift) {
     typedef WarpSmemT<MC> WarpSmem;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -368,67 +539,71 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
     if (lane == 0) W.cand[0] = y0;
     __syncwarp();
     int head = 0, tail = 1;
-    bool done = false, overflow = false;
+    bool done = false, overflow = false, redo = false;   // redo: by the list kernel
     int m = 0, ring = 0;
     double rmin_over_rmax = 0.0;
 
     const GramOwn own = gram_own(lane);
+    int *tab = reinterpret_cast<int *>(W.d2);   // 2 MC slots
+    bool hashed = false;
 
-    for (int k = 1; k <= ring_max && !done; ++k) {
+    for (int k = 1; k <= ring_max && !done && !redo; ++k) {
         // ---- grow the ring by one layer (Section 4.3: (k+1)-ring = k-ring
-        // plus the face neighbours of its nodes).  The frontier [head, tail)
-        // does not change while the layer grows, so the adjacency of up to
-        // eight 32-slot batches is loaded before any of them is merged; the
-        // valid slots (about a quarter: a face with a same-size or coarser
-        // neighbour fills one of its four) are packed densely in the d2 area,
-        // which is free until the candidates are ranked.
-        int32_t *stg = reinterpret_cast<int32_t *>(W.d2);
-        const int nslots = (tail - head) * 24;
-        for (int g0 = 0; g0 < nslots; g0 += 8 * 32) {
-            int vb[8];
-#pragma unroll
-            for (int bt = 0; bt < 8; ++bt) {
-                const int s = g0 + bt * 32 + lane;
-                int v = -1;
-                if (s < nslots) {
-                    const int u = W.cand[head + s / 24];
-                    const int slot = s % 24;
-                    if (u < n_int) v = adj[(int64_t)u * 24 + slot];
-                    else if (slot == 0) v = bowner[u - n_int];
-                }
-                vb[bt] = v;
-            }
-            int nv = 0;
-#pragma unroll
-            for (int bt = 0; bt < 8; ++bt) {
-                const unsigned bv = __ballot_sync(FULL, vb[bt] >= 0);
-                if (vb[bt] >= 0) stg[nv + __popc(bv & lt)] = vb[bt];
-                nv += __popc(bv);
-            }
+        // plus the face neighbours of its nodes).  Eight lanes per frontier
+        // node read its neighbours (packed first in its 24 slots; nearly all
+        // nodes have at most eight), sixteen nodes' loads in flight.  A hash set
+        // of the candidates, in the d2 area until they are ranked, tells the new
+        // ones (a scan of all candidates for each took as long as the search).
+        if (!hashed) {
+            int4 *t4 = reinterpret_cast<int4 *>(tab);
+            for (int t = lane; t < MC / 2; t += 32) t4[t] = make_int4(-1, -1, -1, -1);
             __syncwarp();
-            for (int b0 = 0; b0 < nv; b0 += 32) {
-                const int v = (b0 + lane < nv) ? stg[b0 + lane] : -1;
-                bool fresh = v >= 0;
-                for (int t = 0; fresh && t < nc; t += 4) {
-                    const int4 c4 = *reinterpret_cast<const int4 *>(&W.cand[t]);
-                    if (c4.x == v || (c4.y == v && t + 1 < nc) || (c4.z == v && t + 2 < nc) ||
-                        (c4.w == v && t + 3 < nc))
-                        fresh = false;
+            for (int t = lane; t < nc; t += 32) ring_insert<MC>(tab, W.cand[t]);
+            __syncwarp();
+            hashed = true;
+        }
+        for (int g0 = head; g0 < tail && !overflow; g0 += 16) {
+            int vb[4], ub[4];
+            const int sub = lane & 7;
+#pragma unroll
+            for (int bt = 0; bt < 4; ++bt) {
+                const int t = g0 + bt * 4 + (lane >> 3);
+                ub[bt] = t < tail ? W.cand[t] : -1;
+            }
+#pragma unroll
+            for (int bt = 0; bt < 4; ++bt) {
+                const int u = ub[bt];
+                vb[bt] = u < 0 ? -1 : (u < n_int ? adj[(int64_t)u * 24 + sub] : (sub == 0 ? bowner[u - n_int] : -1));
+            }
+#pragma unroll 1
+            for (int bt = 0; bt < 4 && g0 + bt * 4 < tail && !overflow; ++bt) {
+                int v = vb[0];
+                const int u = ub[0];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    vb[q] = vb[q + 1];
+                    ub[q] = ub[q + 1];
                 }
-                unsigned peers = __match_any_sync(FULL, fresh ? v : -2 - lane);
-                if (fresh && lane != __ffs(peers) - 1) fresh = false;
-                unsigned bal = __ballot_sync(FULL, fresh);
-                int p = nc + __popc(bal & lt);
-                if (fresh) {
-                    if (p < slots) W.cand[p] = v;
-                    else overflow = true;
+                for (int more = 0; more < 24; more += 8) {
+                    if (more > 0) {   // a node with its eight slots full may have more
+                        const bool ask = u >= 0 && u < n_int;
+                        if (!__any_sync(FULL, ask && sub == 7 && v >= 0)) break;
+                        v = ask ? adj[(int64_t)u * 24 + more + sub] : -1;
+                    }
+                    const bool fresh = v >= 0 && ring_insert<MC>(tab, v);
+                    const unsigned bal = __ballot_sync(FULL, fresh);
+                    const int p = nc + __popc(bal & lt);
+                    if (fresh && p < slots) W.cand[p] = v;
+                    nc += __popc(bal);
+                    if (nc > slots) {
+                        overflow = true;   // the same in every lane
+                        break;
+                    }
+                    __syncwarp();
                 }
-                nc += __popc(bal);
-                if (nc > slots) nc = slots;
-                __syncwarp();
             }
         }
-        if (__any_sync(FULL, overflow)) break;
+        if (overflow) break;
         head = tail;
         tail = nc;
         if (k < 2) continue;
@@ -438,41 +613,66 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
 
         // ---- order the candidates by (exact integer squared distance, node
         // index): every later choice is a prefix of this order
-        for (int t = 1 + lane; t < nc; t += 32) {
-            int4 q = ic[W.cand[t]];
-            long long dx = (long long)q.x - c0.x, dy = (long long)q.y - c0.y, dz = (long long)q.z - c0.z;
-            W.d2[t] = dx * dx + dy * dy + dz * dz;
-            W.oct[t] = (uint8_t)(((dx >= 0) << 2) | ((dy >= 0) << 1) | (dz >= 0));
+        // (two candidates per lane and pass over the others).  Offsets are
+        // whole half cells of the deepest level, 2^(d2_shift / 2) units, so
+        // distance and index fit one 64-bit key unless the tree is very deep
+        // and large (idx_bits 0).
+        hashed = false;
+        for (int t0 = 1; t0 < nc; t0 += 64) {   // d2 area: keys of all candidates
+            for (int t = t0 + lane; t < nc && t < t0 + 64; t += 32) {
+                const int id = W.cand[t];
+                int4 q = ic[id];
+                long long dx = (long long)q.x - c0.x, dy = (long long)q.y - c0.y, dz = (long long)q.z - c0.z;
+                const long long dd = dx * dx + dy * dy + dz * dz;
+                W.d2[t] = idx_bits ? (dd >> d2_shift) << idx_bits | id : dd;
+                W.oct[t] = (uint8_t)(((dx >= 0) << 2) | ((dy >= 0) << 1) | (dz >= 0));
+            }
         }
         __syncwarp();
-        for (int t = 1 + lane; t < nc; t += 32) {
-            const long long dt = W.d2[t];
-            const int it = W.cand[t];
-            int r = 0;
-            for (int u = 1; u < nc; ++u) r += key_less(W.d2[u], W.cand[u], dt, it) ? 1 : 0;
-            W.srt[r] = (uint16_t)t;
+        if (idx_bits) {
+            for (int t0 = 1; t0 < nc; t0 += 64) {
+                const int ta = t0 + lane, tb = ta + 32;
+                const unsigned long long ka = ta < nc ? W.d2[ta] : ~0ull, kb = tb < nc ? W.d2[tb] : ~0ull;
+                int ra = 0, rb = 0;
+#pragma unroll 4
+                for (int u = 1; u < nc; ++u) {
+                    const unsigned long long ku = W.d2[u];
+                    ra += ku < ka;
+                    rb += ku < kb;
+                }
+                if (ta < nc) W.srt[ra] = (uint16_t)ta;
+                if (tb < nc) W.srt[rb] = (uint16_t)tb;
+            }
+            __syncwarp();
+            for (int t = 1 + lane; t < nc; t += 32) W.d2[t] = (W.d2[t] >> idx_bits) << d2_shift;
+        } else {
+            for (int t = 1 + lane; t < nc; t += 32) {
+                const long long dt = W.d2[t];
+                const int it = W.cand[t];
+                int r = 0;
+                for (int u = 1; u < nc; ++u) r += key_less(W.d2[u], W.cand[u], dt, it) ? 1 : 0;
+                W.srt[r] = (uint16_t)t;
+            }
         }
         __syncwarp();
         // ---- Section 3.1 quadrant criterion, octants in 3-D: the two nearest
         // in each octant, counted along the order 32 positions at a time
         int nA = 0;
         {
-            int cnt[8];
-#pragma unroll
-            for (int o = 0; o < 8; ++o) cnt[o] = 0;
+            unsigned seen_lo = 0u, seen_hi = 0u;   // counts of octants 0-3 and 4-7, a byte each (capped at 2)
             for (int p0 = 0; p0 < ncand; p0 += 32) {
                 const int pos = p0 + lane;
-                const int o = (pos < ncand) ? (int)W.oct[W.srt[pos]] : -1;
-                int before = 0;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const unsigned bq = __ballot_sync(FULL, o == q);
-                    if (o == q) before = cnt[q] + __popc(bq & lt);
-                    cnt[q] += __popc(bq);
-                }
-                const bool pk = o >= 0 && before < 2;
+                const int o = (pos < ncand) ? (int)W.oct[W.srt[pos]] : 8;
+                const unsigned peers = __match_any_sync(FULL, o);
+                const unsigned word = o < 4 ? seen_lo : seen_hi;
+                const int sh = (o & 3) * 8, rank = __popc(peers & lt);
+                const bool pk = o < 8 && (int)(word >> sh & 255u) + rank < 2;
                 if (pos < ncand) W.pick[pos] = pk ? 1 : 0;
                 nA += __popc(__ballot_sync(FULL, pk));
+                if (p0 + 32 < ncand) {   // picks are what counts towards two per octant
+                    seen_lo += __reduce_add_sync(FULL, pk && o < 4 ? 1u << sh : 0u);
+                    seen_hi += __reduce_add_sync(FULL, pk && o >= 4 ? 1u << sh : 0u);
+                }
             }
         }
         __syncwarp();
@@ -529,12 +729,17 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
         // where FP32 Cholesky QR loses its accuracy)
         double q[NCOL], lapj = 0.0;
         bool ok = false;
-        if (fp32_first) {
-            ok = wls_column<float>(W, m, lane, own, c0, ic, unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
+        if (MIXED) {
+            ok = wls_column_f32(W, m, lane, own, c0, ic, unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
             if (ok && rmin_over_rmax < fp32_rcond_min) ok = false;
+            if (!ok && !LIST) {   // the list kernel holds the FP64 code: here it would cost registers
+                redo = true;
+                break;
+            }
             if (!ok && lane == 0) atomicAdd(fp64_count, 1);
         }
-        if (!ok) ok = wls_column<double>(W, m, lane, own, c0, ic, unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
+        if ((LIST || !MIXED) && !ok)
+            ok = wls_column_f64(W, m, lane, own, c0, ic, inv_unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
         if (ok) ok = rmin_over_rmax >= RANK_TOL;
         if (!ok) lapj = 0.0;
         const double lsum = warp_sum_d(lapj);
@@ -567,9 +772,9 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
         }   // target sizes
     }
     if (!done) {
-        const bool ovf = __any_sync(FULL, overflow);
+        const bool ovf = overflow;
         if (lane == 0) {
-            if (ovf && !LIST) ovf_list[atomicAdd(ovf_count, 1u)] = y0;   // redone with MAXC slots
+            if ((ovf || redo) && !LIST) ovf_list[atomicAdd(ovf_count, 1u)] = y0;   // redone with MAXC slots
             else atomicOr(err, ovf ? (ERR_STENCIL | ERR_OVERFLOW) : ERR_STENCIL);
             m_out[y0] = 0;
             ring_out[y0] = -1;
@@ -611,12 +816,16 @@ __global__ void k_diag(const int32_t *__restrict__ msz, const double *__restrict
     rB[r] = 1.0 / b;
 }
 
-__global__ void k_slice_width(const int32_t *__restrict__ msz, int n_int, int n_tot, int nsl, uint32_t *__restrict__ w) {
+// widths of the 32-row slices; also the sum of the stencil sizes
+__global__ void k_slice_width(const int32_t *__restrict__ msz, int n_int, int n_tot, int nsl, uint32_t *__restrict__ w,
+                              uint32_t *__restrict__ sum_m) {
     int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int lane = threadIdx.x & 31;
     if (s >= nsl) return;
     int r = s * 32 + lane;
     int v = 0;
+    const int sm = __reduce_add_sync(0xffffffffu, r < n_int ? msz[r] : 0);
+    if (lane == 0) atomicAdd(sum_m, (uint32_t)sm);
     if (r < n_int) v = msz[r] + 1;
     else if (r < n_tot) v = 1;
 #pragma unroll
@@ -688,35 +897,54 @@ __global__ void k_values_f32(const double *__restrict__ vA, const double *__rest
     }
 }
 
-template <int SW>
-apcloud_status launch_stencil(apcloud_ctx *c, int n, double unit, double ec, double inv_1mec, int32_t *nbr,
-                              int32_t *msz, int32_t *ring, double *lap, double *lapd, double *D, int64_t dstride,
-                              double *rc, unsigned *derr) {
+template <int SW, bool MIXED>
+apcloud_status launch_stencil_of(apcloud_ctx *c, int n, double unit, double ec, double inv_1mec, int32_t *nbr,
+                                 int32_t *msz, int32_t *ring, double *lap, double *lapd, double *D, int64_t dstride,
+                                 double *rc, unsigned *derr, unsigned *words) {
     // every node with MAXC_FAST candidate slots, then (one read-back of the
     // count) the nodes whose rings outgrew them with MAXC
     int32_t *ovf = ensure<int32_t>(c, c->stencil_ovf, n + 1);
     if (!ovf) return APCLOUD_E_NOMEM;
     APC_CUDA(c, cudaMemsetAsync(derr + 2, 0, sizeof(unsigned), c->s));
+    // rank keys: squared distances in half cells of the deepest level (2 L + 4 bits) over the node index
+    int idx_bits = 1;
+    while ((1ll << idx_bits) < c->n_tot) ++idx_bits;
+    if (2 * c->L + 4 + idx_bits > 63) idx_bits = 0;
+    const int d2_shift = 2 * (KEY_DEPTH - c->L);
     const size_t smem = SW * sizeof(WarpSmemT<MAXC_FAST>) + 16;   // the warps' areas, then the block's arrival count
     // the limit is a per-device property of the function: set on every build
     // (one host call each), so that contexts on other devices get it too
-    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<SW, MAXC_FAST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<SW, MAXC_FAST, false, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
-    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<4, MAXC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<4, MAXC, true, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(4 * sizeof(WarpSmemT<MAXC>) + 16)));
-    APC_LAUNCH(c, K_STENCIL, div_up(n, SW), SW * 32, smem, (k_stencil<SW, MAXC_FAST, false>), ptr<int4>(c->node_ic),
-               ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target, c->P.ring_max, unit, ec, inv_1mec,
-               nbr, msz, ring, lap, lapd, D, dstride, rc, c->P.precision == 1 ? 1 : 0, c->P.fp32_rcond_min,
-               reinterpret_cast<int *>(derr + 1), derr, (const int32_t *)nullptr, 0, derr + 2, ovf, c->P.stencil_slots);
-    unsigned nov = 0;
-    APC_TRY(read_back(c, &nov, derr + 2, sizeof nov));
-    if (nov > 0)
-        APC_LAUNCH(c, K_STENCIL, div_up(nov, 4), 4 * 32, 4 * sizeof(WarpSmemT<MAXC>) + 16, (k_stencil<4, MAXC, true>),
+    APC_LAUNCH(c, K_STENCIL, div_up(n, SW), SW * 32, smem, (k_stencil<SW, MAXC_FAST, false, MIXED>), ptr<int4>(c->node_ic),
+               ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target, c->P.ring_max, unit, 1.0 / unit, ec, inv_1mec,
+               nbr, msz, ring, lap, lapd, D, dstride, rc, c->P.fp32_rcond_min,
+               reinterpret_cast<int *>(derr + 1), derr, (const int32_t *)nullptr, 0, derr + 2, ovf, c->P.stencil_slots,
+               idx_bits, d2_shift);
+    // the overflow count, with the error word and the count of FP64 blocks
+    APC_TRY(read_back(c, words, derr, 3 * sizeof(unsigned)));
+    const unsigned nov = words[2];
+    if (nov > 0) {
+        APC_LAUNCH(c, K_STENCIL, div_up(nov, 4), 4 * 32, 4 * sizeof(WarpSmemT<MAXC>) + 16, (k_stencil<4, MAXC, true, MIXED>),
                    ptr<int4>(c->node_ic), ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target,
-                   c->P.ring_max, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc,
-                   c->P.precision == 1 ? 1 : 0, c->P.fp32_rcond_min, reinterpret_cast<int *>(derr + 1), derr,
-                   (const int32_t *)ovf, (int)nov, derr + 2, ovf, MAXC);
+                   c->P.ring_max, unit, 1.0 / unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc,
+                   c->P.fp32_rcond_min, reinterpret_cast<int *>(derr + 1), derr,
+                   (const int32_t *)ovf, (int)nov, derr + 2, ovf, MAXC, idx_bits, d2_shift);
+        APC_TRY(read_back(c, words, derr, 3 * sizeof(unsigned)));
+    }
     return APCLOUD_OK;
+}
+
+template <int SW>
+apcloud_status launch_stencil(apcloud_ctx *c, int n, double unit, double ec, double inv_1mec, int32_t *nbr,
+                              int32_t *msz, int32_t *ring, double *lap, double *lapd, double *D, int64_t dstride,
+                              double *rc, unsigned *derr, unsigned *words) {
+    return c->P.precision == 1 ? launch_stencil_of<SW, true>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D,
+                                                             dstride, rc, derr, words)
+                               : launch_stencil_of<SW, false>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D,
+                                                              dstride, rc, derr, words);
 }
 
 }  // namespace
@@ -738,37 +966,21 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     const double unit = ldexp(ext, -(KEY_DEPTH + 1));
     const double ec = exp(-c->P.weight_c);
     const double inv_1mec = 1.0 / (1.0 - ec);
+    unsigned words[3];
     switch (c->wls_warps) {
     case 2:
-        APC_TRY(launch_stencil<2>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr));
+        APC_TRY(launch_stencil<2>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr, words));
         break;
     case 8:
-        APC_TRY(launch_stencil<8>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr));
+        APC_TRY(launch_stencil<8>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr, words));
         break;
     default:
-        APC_TRY(launch_stencil<4>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr));
+        APC_TRY(launch_stencil<4>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr, words));
         break;
     }
     APC_CUDA(c, cudaGetLastError());
-    APC_TRY(check_device_errors(c));
-    {
-        unsigned e[2];
-        APC_TRY(read_back(c, e, derr, sizeof e));
-        c->n_fp64_wls = e[1];
-    }
-    {   // total stencil size, for the algorithmic traffic of later kernels
-        uint32_t *tmp = ensure<uint32_t>(c, c->tmp, n + 1);
-        if (!tmp) return APCLOUD_E_NOMEM;
-        uint32_t *small = ptr<uint32_t>(c->dsmall);
-        APC_TRY(scan_u32(c, reinterpret_cast<const uint32_t *>(msz), tmp, n, small + 6));
-        uint32_t sm;
-        APC_TRY(read_back(c, &sm, small + 6, sizeof sm));
-        c->sum_m = sm;
-        // per node: offsets and weights in (28 B per neighbour), Laplacian row and
-        // 9 x m operator out (80 B per neighbour); two 9-column Gram products,
-        // three triangular solves per row and two 9x9 factorizations
-        account(c, K_STENCIL, 108.0 * sm + 8.0 * n, 450.0 * sm + 660.0 * n);
-    }
+    APC_TRY(device_errors(c, words[0]));
+    c->n_fp64_wls = words[1];
 
     // sliced ELL of A and B
     const int nsl = div_up(nt, 32);
@@ -782,12 +994,21 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     double *rA = rd, *rB = rd + nt + 1;
     APC_LAUNCH(c, K_ELL, div_up(nt, 256), 256, 0, k_diag, msz, lapd, ptr<int4>(c->node_ic), n, nt, ext, dA, dB, rA,
                rB);
-    APC_LAUNCH(c, K_ELL, div_up(nsl, 8), 256, 0, k_slice_width, msz, n, nt, nsl, sw);
     uint32_t *small = ptr<uint32_t>(c->dsmall);
+    APC_CUDA(c, cudaMemsetAsync(small + 6, 0, sizeof(uint32_t), c->s));
+    APC_LAUNCH(c, K_ELL, div_up(nsl, 8), 256, 0, k_slice_width, msz, n, nt, nsl, sw, small + 6);
     APC_TRY(scan_u32(c, sw, so, nsl, small + 5));
-    uint32_t tot;
-    APC_TRY(read_back(c, &tot, small + 5, sizeof tot));
-    c->ell_entries = (int64_t)tot * 32;
+    // the width-sorted copy's slices too, so that one read gives every size
+    if (c->P.precision == 1) APC_TRY(rank_sorted_sweep(c, small + 7));
+    uint32_t tot[3];   // ELL columns, stencil sizes, sorted columns
+    APC_TRY(read_back(c, tot, small + 5, sizeof tot));
+    c->ell_entries = (int64_t)tot[0] * 32;
+    c->sum_m = tot[1];
+    c->ss_entries = c->P.precision == 1 ? (int64_t)tot[2] * 32 : 0;
+    // per node: offsets and weights in (28 B per neighbour), Laplacian row and
+    // 9 x m operator out (80 B per neighbour); two 9-column Gram products,
+    // three triangular solves per row and two 9x9 factorizations
+    account(c, K_STENCIL, 108.0 * tot[1] + 8.0 * n, 450.0 * tot[1] + 660.0 * n);
     int32_t *col = ensure<int32_t>(c, c->ell_col, c->ell_entries);
     double *vA = ensure<double>(c, c->ell_A, c->ell_entries);
     double *vB = ensure<double>(c, c->ell_B, c->ell_entries);
@@ -801,7 +1022,7 @@ apcloud_status build_stencils(apcloud_ctx *c) {
         if (!fA || !fB || !hA || !hB) return APCLOUD_E_NOMEM;
         APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_f32, (const double *)vA,
                    (const double *)vB, c->ell_entries, fA, fB, hA, hB);
-        APC_TRY(build_sorted_sweep(c));
+        APC_TRY(fill_sorted_sweep(c));
     }
     return cuda_check(c, cudaGetLastError(), "ell");
 }
@@ -826,6 +1047,7 @@ apcloud_status tune_stencils(apcloud_ctx *c, double *ms_out) {
     const double ec = exp(-c->P.weight_c);
     const double inv_1mec = 1.0 / (1.0 - ec);
     const int shapes[3] = {2, 4, 8};
+    unsigned words[3];
     cudaEvent_t e0, e1;
     APC_CUDA(c, cudaEventCreate(&e0));
     APC_CUDA(c, cudaEventCreate(&e1));
@@ -841,11 +1063,11 @@ apcloud_status tune_stencils(apcloud_ctx *c, double *ms_out) {
             if (st != APCLOUD_OK) break;
             cudaEventRecord(e0, c->s);
             if (shapes[t] == 2)
-                st = launch_stencil<2>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr);
+                st = launch_stencil<2>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr, words);
             else if (shapes[t] == 4)
-                st = launch_stencil<4>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr);
+                st = launch_stencil<4>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr, words);
             else
-                st = launch_stencil<8>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr);
+                st = launch_stencil<8>(c, n, unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc, derr, words);
             cudaEventRecord(e1, c->s);
             if (st == APCLOUD_OK) st = cuda_check(c, cudaEventSynchronize(e1), "autotune stencils");
             if (st == APCLOUD_OK) cudaEventElapsedTime(&ms, e0, e1);
@@ -871,7 +1093,7 @@ apcloud_status refresh_lowp(apcloud_ctx *c) {
     APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_f32, (const double *)ptr<double>(c->ell_A),
                (const double *)ptr<double>(c->ell_B), c->ell_entries, ptr<float>(c->ell_A32), ptr<float>(c->ell_B32),
                ptr<__half>(c->ell_A16), ptr<__half>(c->ell_B16));
-    APC_TRY(build_sorted_sweep(c));
+    APC_TRY(fill_sorted_sweep(c));
     return cuda_check(c, cudaGetLastError(), "refresh_lowp");
 }
 
@@ -975,7 +1197,9 @@ __global__ void k_ss_fill(const uint32_t *__restrict__ sw, const uint32_t *__res
 // the Arnoldi products (also the same bits as the FP32 ELL product), and for
 // the sweeps the chunks' columns packed to 24 bits (while n < 2^24): 20
 // instead of 24 bytes per 4-entry chunk of a bandwidth-bound stream.
-apcloud_status build_sorted_sweep(apcloud_ctx *c) {
+// Ranks and slice widths (their total to *d_total), then the copy itself once
+// ss_entries is known; a refresh of the values needs the second part only.
+apcloud_status rank_sorted_sweep(apcloud_ctx *c, uint32_t *d_total) {
     c->ss_ok = false;
     const int n = c->n_tot;
     if (n == 0) return APCLOUD_OK;
@@ -986,11 +1210,15 @@ apcloud_status build_sorted_sweep(apcloud_ctx *c) {
     uint32_t *w2 = ensure<uint32_t>(c, c->ss_w, nsl2 + 1), *o2 = ensure<uint32_t>(c, c->ss_o, nsl2 + 1);
     if (!perm || !w2 || !o2) return APCLOUD_E_NOMEM;
     APC_LAUNCH(c, K_ELL, nwin, SS_WIN, 0, k_ss_rank, (const int32_t *)ptr<int32_t>(c->msz), c->n_int, n, perm, w2);
-    uint32_t *small = ptr<uint32_t>(c->dsmall);
-    APC_TRY(scan_u32(c, w2, o2, nsl2, small + 13));
-    uint32_t tot;
-    APC_TRY(read_back(c, &tot, small + 13, sizeof tot));
-    c->ss_entries = (int64_t)tot * 32;
+    return scan_u32(c, w2, o2, nsl2, d_total);
+}
+
+apcloud_status fill_sorted_sweep(apcloud_ctx *c) {
+    const int n = c->n_tot;
+    if (n == 0) return APCLOUD_OK;
+    const int64_t nslot = (int64_t)div_up(n, SS_WIN) * SS_WIN;
+    const int32_t *perm = ptr<int32_t>(c->ss_perm);
+    const uint32_t *w2 = ptr<uint32_t>(c->ss_w), *o2 = ptr<uint32_t>(c->ss_o);
     int32_t *col2 = ensure<int32_t>(c, c->ss_col, c->ss_entries + 1);
     __half *A2 = ensure<__half>(c, c->ss_A, c->ss_entries + 1), *B2 = ensure<__half>(c, c->ss_B, c->ss_entries + 1);
     float *A4 = ensure<float>(c, c->ss_A32, c->ss_entries + 1), *B4 = ensure<float>(c, c->ss_B32, c->ss_entries + 1);
@@ -1006,8 +1234,7 @@ apcloud_status build_sorted_sweep(apcloud_ctx *c) {
     APC_LAUNCH(c, K_ELL, div_up(nslot, 256), 256, 0, k_ss_fill, (const uint32_t *)ptr<uint32_t>(c->slice_w),
                (const uint32_t *)ptr<uint32_t>(c->slice_off), (const int32_t *)ptr<int32_t>(c->ell_col),
                (const __half *)ptr<__half>(c->ell_A16), (const __half *)ptr<__half>(c->ell_B16),
-               (const float *)ptr<float>(c->ell_A32), (const float *)ptr<float>(c->ell_B32), (const int32_t *)perm,
-               (const uint32_t *)w2, (const uint32_t *)o2, nslot, col2, A2, B2, A4, B4, col24);
+               (const float *)ptr<float>(c->ell_A32), (const float *)ptr<float>(c->ell_B32), perm, w2, o2, nslot, col2, A2, B2, A4, B4, col24);
     c->ss_ok = true;
     return cuda_check(c, cudaGetLastError(), "sorted sweep matrix");
 }
