@@ -18,6 +18,7 @@
 // signalled through an mbarrier, results read back with tcgen05.ld.  The
 // graph products (P H, P^T G), features, head, loss and Adam run on the CUDA
 // cores.  Every reduction has a fixed order, so a training run is repeatable.
+#include <algorithm>
 #include <atomic>
 #include <cuda_bf16.h>
 
@@ -364,11 +365,13 @@ __global__ void k_wgrad_reduce(const float *__restrict__ part, int nblk, int Kl,
 // ---------------------------------------------------------------- graph
 // ELL entry e of row j with column i != j and a nonzero value: two records,
 // (j, i) carrying Ahat_ji as the row's own entry and (i, j) carrying it as an
-// entry of column i's transpose.  Record value: (ELL index << 1) | direction.
+// entry of column i's transpose.  Record value: (ELL index << 1) | direction;
+// key: row << bits | column, 32 bits wide while both fit.  Keys past the last
+// record stay all ones, which sorts behind every pair of distinct nodes.
+template <class K>
 __global__ void k_edge_emit(const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff,
-                            const int32_t *__restrict__ col, const double *__restrict__ val, int n,
-                            const uint32_t *__restrict__ cnt_off, uint64_t *__restrict__ key,
-                            uint32_t *__restrict__ rec) {
+                            const int32_t *__restrict__ col, const double *__restrict__ val, int n, int bits,
+                            const uint32_t *__restrict__ cnt_off, K *__restrict__ key, uint32_t *__restrict__ rec) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
     const int sl = r >> 5, lane = r & 31;
@@ -379,9 +382,9 @@ __global__ void k_edge_emit(const uint32_t *__restrict__ sw, const uint32_t *__r
         const int64_t e = base + (int64_t)k * 32;
         const int i = col[e];
         if (i == r || val[e] == 0.0) continue;
-        key[2 * o] = ((uint64_t)(uint32_t)r << 32) | (uint32_t)i;
+        key[2 * o] = (K)r << bits | (K)i;
         rec[2 * o] = (uint32_t)(e << 1);
-        key[2 * o + 1] = ((uint64_t)(uint32_t)i << 32) | (uint32_t)r;
+        key[2 * o + 1] = (K)i << bits | (K)r;
         rec[2 * o + 1] = (uint32_t)((e << 1) | 1);
         ++o;
     }
@@ -403,16 +406,18 @@ __global__ void k_edge_count(const uint32_t *__restrict__ sw, const uint32_t *__
     cnt[r] = c;
 }
 
-__global__ void k_run_heads(const uint64_t *__restrict__ key, int64_t m, uint32_t *__restrict__ f) {
+template <class K>
+__global__ void k_run_heads(const K *__restrict__ key, int64_t m, uint32_t *__restrict__ f) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) f[i] = (i == 0 || key[i] != key[i - 1]) ? 1u : 0u;
+    if (i < m) f[i] = (key[i] != (K)~(K)0 && (i == 0 || key[i] != key[i - 1])) ? 1u : 0u;
 }
 
 // unique (row, col) pairs: column, signed out value Ahat_row,col and in value Ahat_col,row
-__global__ void k_edge_merge(const uint64_t *__restrict__ key, const uint32_t *__restrict__ rec, int64_t m,
+template <class K>
+__global__ void k_edge_merge(const K *__restrict__ key, const uint32_t *__restrict__ rec, int64_t m, int bits,
                              const uint32_t *__restrict__ f, const uint32_t *__restrict__ pos,
                              const double *__restrict__ val, int32_t *__restrict__ ecol, float *__restrict__ aout,
-                             float *__restrict__ ain, uint64_t *__restrict__ ukey) {
+                             float *__restrict__ ain, K *__restrict__ ukey) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m || !f[i]) return;
     float o = 0.f, in = 0.f;
@@ -422,20 +427,21 @@ __global__ void k_edge_merge(const uint64_t *__restrict__ key, const uint32_t *_
         if (r & 1u) in = v; else o = v;
     }
     const uint32_t p = pos[i];
-    ecol[p] = (int32_t)(uint32_t)(key[i] & 0xFFFFFFFFull);
+    ecol[p] = (int32_t)(key[i] & (((K)1 << bits) - 1));
     aout[p] = o;
     ain[p] = in;
     ukey[p] = key[i];
 }
 
-__global__ void k_rowptr(const uint64_t *__restrict__ ukey, int64_t m, int n, int32_t *__restrict__ rp) {
+template <class K>
+__global__ void k_rowptr(const K *__restrict__ ukey, const uint32_t *__restrict__ m, int n, int bits,
+                         int32_t *__restrict__ rp) {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j > n) return;
-    const uint64_t v = (uint64_t)(uint32_t)j << 32;
-    int64_t lo = 0, hi = m;
+    int64_t lo = 0, hi = *m;
     while (lo < hi) {
         int64_t mid = (lo + hi) >> 1;
-        if (ukey[mid] < v) lo = mid + 1; else hi = mid;
+        if ((int64_t)(ukey[mid] >> bits) < j) lo = mid + 1; else hi = mid;
     }
     rp[j] = (int32_t)lo;
 }
@@ -642,18 +648,19 @@ __global__ void k_loss_terms(const uint32_t *__restrict__ sw, const uint32_t *__
         for (int q = 0; q < 3; ++q) part[(int64_t)blockIdx.x * 3 + q] = sh[q][0];
 }
 
+// one warp: lane l adds blocks l, l + 32, ..., then a fixed tree (one thread
+// adding 60 blocks took 14 us)
 __global__ void k_loss_final(const double *__restrict__ part, int nblk, int n_int, double *__restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double rr = 0.0, bb = 0.0, lp = 0.0;
-    for (int k = 0; k < nblk; ++k) {
-        rr += part[3 * k];
-        bb += part[3 * k + 1];
-        lp += part[3 * k + 2];
-    }
-    out[1] = n_int > 0 ? lp / n_int : 0.0;
-    out[2] = bb > 0.0 ? rr / bb : 0.0;
+    double v[3] = {0.0, 0.0, 0.0};
+    for (int k = threadIdx.x; k < nblk; k += 32)
+        for (int q = 0; q < 3; ++q) v[q] += part[3 * (int64_t)k + q];
+    for (int o = 16; o > 0; o >>= 1)
+        for (int q = 0; q < 3; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    if (threadIdx.x != 0) return;
+    out[1] = n_int > 0 ? v[2] / n_int : 0.0;
+    out[2] = v[1] > 0.0 ? v[0] / v[1] : 0.0;
     out[0] = out[1] + out[2];
-    out[3] = bb;
+    out[3] = v[1];
 }
 
 // dt from dLp/ds = (2/n)(s c - 1) and dLg/dgamma = -2 b (Ahat^T r) / ||b||^2;
@@ -677,41 +684,47 @@ __global__ void k_head_back(const int32_t *__restrict__ rp, const int32_t *__res
 }
 
 // head weight gradients: dWo = H3^T dt (64 x 2), dbo = sum dt; per-block
-// partials then a fixed-order sum
-__global__ void k_head_wgrad(const __nv_bfloat16 *__restrict__ H3, const float *__restrict__ dt, int n,
-                             float *__restrict__ part) {
-    __shared__ float sh[256];
-    float acc[2 * WD + 2];
+// partials then a fixed-order sum.  Four row groups of 64 threads, a column
+// each, so the rows of H3 are read as they lie (a thread per row with 130
+// sums and a block reduction for each took 128 us on 1.5e4 nodes; 6 us now).
+__global__ void __launch_bounds__(256) k_head_wgrad(const __nv_bfloat16 *__restrict__ H3,
+                                                    const float *__restrict__ dt, int n, float *__restrict__ part) {
+    __shared__ float sh[4][4 * WD];   // sums by column: dWo0, dWo1, dbo0, dbo1
+    const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
+    float a0 = 0.f, a1 = 0.f, s0 = 0.f, s1 = 0.f;
 #pragma unroll 4
-    for (int i = 0; i < 2 * WD + 2; ++i) acc[i] = 0.f;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const float d0 = dt[2 * j], d1 = dt[2 * j + 1];
-        for (int k = 0; k < WD; ++k) {
-            const float h = __bfloat162float(H3[(int64_t)j * WD + k]);
-            acc[2 * k] = fmaf(h, d0, acc[2 * k]);
-            acc[2 * k + 1] = fmaf(h, d1, acc[2 * k + 1]);
-        }
-        acc[2 * WD] += d0;
-        acc[2 * WD + 1] += d1;
+    for (int j = blockIdx.x * 4 + g; j < n; j += gridDim.x * 4) {
+        const float2 d = reinterpret_cast<const float2 *>(dt)[j];
+        const float h = __bfloat162float(H3[(int64_t)j * WD + c]);
+        a0 = fmaf(h, d.x, a0);
+        a1 = fmaf(h, d.y, a1);
+        s0 += d.x;
+        s1 += d.y;
     }
-    for (int q = 0; q < 2 * WD + 2; ++q) {
-        sh[threadIdx.x] = acc[q];
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) part[(int64_t)blockIdx.x * (2 * WD + 2) + q] = sh[0];
-        __syncthreads();
+    sh[g][c] = a0;
+    sh[g][WD + c] = a1;
+    sh[g][2 * WD + c] = s0;
+    sh[g][3 * WD + c] = s1;
+    __syncthreads();
+    if (threadIdx.x < 2 * WD + 2) {
+        const int q = threadIdx.x;   // part holds dWo row by row (k, 2), then dbo
+        const int at = q < 2 * WD ? (q & 1) * WD + (q >> 1) : (2 + q - 2 * WD) * WD;
+        part[(int64_t)blockIdx.x * (2 * WD + 2) + q] = (sh[0][at] + sh[1][at]) + (sh[2][at] + sh[3][at]);
     }
 }
 
-__global__ void k_sum_partials(const float *__restrict__ part, int nblk, int width, float *__restrict__ out) {
-    int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= width) return;
+// out[q] = sum of part[k * width + q] over k: a block per value, a fixed tree
+// (a thread per value adding up to 1024 partials took 45 us)
+__global__ void __launch_bounds__(128) k_sum_partials(const float *__restrict__ part, int nblk, int width,
+                                                      float *__restrict__ out) {
+    __shared__ float sh[4];
+    const int q = blockIdx.x;
     float s = 0.f;
-    for (int k = 0; k < nblk; ++k) s += part[(int64_t)k * width + q];
-    out[q] = s;
+    for (int k = threadIdx.x; k < nblk; k += 128) s += part[(int64_t)k * width + q];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) out[q] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
 }
 
 // dH3 = dt Wo^T, then dZ2 = dH3 * [H3 > 0] in BF16
@@ -802,47 +815,45 @@ T *mp(apcloud_ctx *c, int i) { return ptr<T>(c->mp[i]); }
 
 constexpr int GT1 = 256;
 
-// symmetric stencil graph of the current system (built once per matrix:
-// apcloud_stencils clears mp_graph_n)
-apcloud_status build_graph(apcloud_ctx *c) {
+// Symmetric stencil graph of the current system (built once per matrix:
+// apcloud_stencils clears mp_graph_n).  The buffers are sized by the stored
+// stencil entries, which the records cannot exceed, so nothing waits for
+// their number.
+template <class K>
+apcloud_status build_graph_of(apcloud_ctx *c, int bits) {
     const int n = c->n_tot;
-    if (c->mp_graph_n == n) return APCLOUD_OK;
     const uint32_t *sw = ptr<uint32_t>(c->slice_w), *so = ptr<uint32_t>(c->slice_off);
     const int32_t *col = ptr<int32_t>(c->ell_col);
     const double *val = ptr<double>(c->ell_A);
     uint32_t *cnt = mb<uint32_t>(c, MB_CNT, n + 1), *off = mb<uint32_t>(c, MB_OFF, n + 1);
-    if (!cnt || !off) return APCLOUD_E_NOMEM;
     uint32_t *small = ptr<uint32_t>(c->dsmall);
-    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_edge_count, sw, so, col, val, n, cnt);
-    APC_TRY(scan_u32(c, cnt, off, n, small + 8));
-    uint32_t ne;
-    APC_TRY(read_back(c, &ne, small + 8, sizeof ne));
-    const int64_t m = 2 * (int64_t)ne;
-    uint64_t *k0 = mb<uint64_t>(c, MB_KEY0, m), *k1 = mb<uint64_t>(c, MB_KEY1, m);
+    const int64_t m = 2 * c->sum_m;
+    K *k0 = mb<K>(c, MB_KEY0, m), *k1 = mb<K>(c, MB_KEY1, m);
     uint32_t *r0 = mb<uint32_t>(c, MB_REC0, m), *r1 = mb<uint32_t>(c, MB_REC1, m);
     uint32_t *fl = mb<uint32_t>(c, MB_FLAG, m), *pos = mb<uint32_t>(c, MB_POS, m);
-    if (!k0 || !k1 || !r0 || !r1 || !fl || !pos) return APCLOUD_E_NOMEM;
-    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_edge_emit, sw, so, col, val, n, (const uint32_t *)off, k0,
-               r0);
-    int bits = 0;
-    while ((1ll << bits) < n) ++bits;
-    int which = 0;
-    APC_TRY(radix_sort(c, k0, r0, k1, r1, m, 32 + bits, &which));
-    const uint64_t *sk = which ? k1 : k0;
-    const uint32_t *sr = which ? r1 : r0;
-    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(m, GT1), GT1, 0, k_run_heads, sk, m, fl);
-    APC_TRY(scan_u32(c, fl, pos, m, small + 9));
-    uint32_t nu;
-    APC_TRY(read_back(c, &nu, small + 9, sizeof nu));
-    int32_t *ecol = mb<int32_t>(c, MB_ECOL, nu);
-    float *aout = mb<float>(c, MB_AOUT, nu), *ain = mb<float>(c, MB_AIN, nu);
-    uint64_t *uk = mb<uint64_t>(c, MB_UKEY, nu);
+    int32_t *ecol = mb<int32_t>(c, MB_ECOL, m);
+    float *aout = mb<float>(c, MB_AOUT, m), *ain = mb<float>(c, MB_AIN, m);
+    K *uk = mb<K>(c, MB_UKEY, m);
     int32_t *rp = mb<int32_t>(c, MB_RP, n + 1);
-    float *S = mb<float>(c, MB_S, n), *pf = mb<float>(c, MB_PF, nu), *pb = mb<float>(c, MB_PB, nu);
-    if (!ecol || !aout || !ain || !uk || !rp || !S || !pf || !pb) return APCLOUD_E_NOMEM;
-    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(m, GT1), GT1, 0, k_edge_merge, sk, sr, m, (const uint32_t *)fl,
+    float *S = mb<float>(c, MB_S, n), *pf = mb<float>(c, MB_PF, m), *pb = mb<float>(c, MB_PB, m);
+    if (!cnt || !off || !k0 || !k1 || !r0 || !r1 || !fl || !pos || !ecol || !aout || !ain || !uk || !rp || !S || !pf ||
+        !pb)
+        return APCLOUD_E_NOMEM;
+    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_edge_count, sw, so, col, val, n, cnt);
+    APC_TRY(scan_u32(c, cnt, off, n, nullptr));
+    APC_CUDA(c, cudaMemsetAsync(k0, 0xFF, sizeof(K) * (size_t)m, c->s));
+    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_edge_emit<K>, sw, so, col, val, n, bits,
+               (const uint32_t *)off, k0, r0);
+    int which = 0;
+    APC_TRY(radix_sort(c, k0, r0, k1, r1, m, 2 * bits, &which));
+    const K *sk = which ? k1 : k0;
+    const uint32_t *sr = which ? r1 : r0;
+    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(m, GT1), GT1, 0, k_run_heads<K>, sk, m, fl);
+    APC_TRY(scan_u32(c, fl, pos, m, small + 9));
+    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(m, GT1), GT1, 0, k_edge_merge<K>, sk, sr, m, bits, (const uint32_t *)fl,
                (const uint32_t *)pos, val, ecol, aout, ain, uk);
-    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n + 1, GT1), GT1, 0, k_rowptr, (const uint64_t *)uk, (int64_t)nu, n, rp);
+    APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n + 1, GT1), GT1, 0, k_rowptr<K>, (const K *)uk, (const uint32_t *)(small + 9),
+               n, bits, rp);
     APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_row_sums, (const int32_t *)rp, (const float *)aout,
                (const float *)ain, n, S);
     APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_agg_weights, (const int32_t *)rp, (const int32_t *)ecol,
@@ -850,6 +861,13 @@ apcloud_status build_graph(apcloud_ctx *c) {
     APC_CUDA(c, cudaGetLastError());
     c->mp_graph_n = n;
     return APCLOUD_OK;
+}
+
+apcloud_status build_graph(apcloud_ctx *c) {
+    if (c->mp_graph_n == c->n_tot) return APCLOUD_OK;
+    int bits = 0;
+    while ((1ll << bits) < c->n_tot) ++bits;
+    return 2 * bits <= 32 ? build_graph_of<uint32_t>(c, bits) : build_graph_of<uint64_t>(c, bits);
 }
 
 apcloud_status tc_launch(apcloud_ctx *c, int mode, const TcArgs &a, int grid) {
@@ -919,11 +937,15 @@ apcloud_status forward(apcloud_ctx *c, apcloud_mpnn *m, const double *b) {
     return cuda_check(c, cudaGetLastError(), "mpnn forward");
 }
 
+apcloud_status tc_error(apcloud_ctx *c, unsigned e) {
+    if (e) return fail(c, APCLOUD_E_TIMEOUT, "a tensor-core layer gave up waiting for its MMAs");
+    return APCLOUD_OK;
+}
+
 apcloud_status check_tc(apcloud_ctx *c, apcloud_mpnn *m) {
     unsigned e;
     APC_TRY(read_back(c, &e, m->err, sizeof e));
-    if (e) return fail(c, APCLOUD_E_TIMEOUT, "a tensor-core layer gave up waiting for its MMAs");
-    return APCLOUD_OK;
+    return tc_error(c, e);
 }
 
 // loss (and with backward, every gradient into m->grad)
@@ -934,7 +956,7 @@ apcloud_status loss_grad(apcloud_ctx *c, apcloud_mpnn *m, const double *b, bool 
     const int32_t *col = ptr<int32_t>(c->ell_col);
     const double *val = ptr<double>(c->ell_A);
     float *r = mb<float>(c, MB_R, n);
-    double *lossv = mb<double>(c, MB_LOSS, 4);
+    double *lossv = mb<double>(c, MB_LOSS, 5);
     if (!r || !lossv) return APCLOUD_E_NOMEM;
     const int nb = div_up(n, GT1);
     double *part = mp<double>(c, MB_PART);
@@ -955,9 +977,9 @@ apcloud_status loss_grad(apcloud_ctx *c, apcloud_mpnn *m, const double *b, bool 
                    (const float *)mp<float>(c, MB_T), (const float *)mp<float>(c, MB_CCOL), (const double *)lossv, n,
                    c->n_int, dt);
         const __nv_bfloat16 *H3 = mp<__nv_bfloat16>(c, MB_H3);
-        const int hb = nb < 1024 ? nb : 1024;
-        APC_LAUNCH(c, K_MPNN_GRAPH, hb, GT1, 0, k_head_wgrad, H3, (const float *)dt, n, wpart);
-        APC_LAUNCH(c, K_MPNN_GRAPH, 1, 2 * WD + 2, 0, k_sum_partials, (const float *)wpart, hb, 2 * WD + 2,
+        const int hb = std::min(div_up(n, 64), 608);
+        APC_LAUNCH(c, K_MPNN_GRAPH, hb, 256, 0, k_head_wgrad, H3, (const float *)dt, n, wpart);
+        APC_LAUNCH(c, K_MPNN_GRAPH, 2 * WD + 2, 128, 0, k_sum_partials, (const float *)wpart, hb, 2 * WD + 2,
                    m->grad + OFF_WO);
         APC_LAUNCH(c, K_MPNN_GRAPH, div_up((int64_t)n * WD, GT1), GT1, 0, k_head_dH, (const float *)dt,
                    (const float *)m->theta, H3, n, dZ);
@@ -973,7 +995,7 @@ apcloud_status loss_grad(apcloud_ctx *c, apcloud_mpnn *m, const double *b, bool 
                        m->grad + OFF_W[l]);
             const int cb = div_up(n, 4) < 1024 ? div_up(n, 4) : 1024;
             APC_LAUNCH(c, K_MPNN_GRAPH, cb, 256, 0, k_colsum, (const __nv_bfloat16 *)dZ, n, wpart);
-            APC_LAUNCH(c, K_MPNN_GRAPH, 1, WD, 0, k_sum_partials, (const float *)wpart, cb, WD, m->grad + OFF_B[l]);
+            APC_LAUNCH(c, K_MPNN_GRAPH, WD, 128, 0, k_sum_partials, (const float *)wpart, cb, WD, m->grad + OFF_B[l]);
             if (l == 0) break;
             // dX = dZ W_l^T (tensor cores), dH_l = dX[:, :C] + P^T dX[:, C:], dZ_{l-1} = dH_l * [H_l > 0]
             TcArgs d{};
@@ -987,9 +1009,13 @@ apcloud_status loss_grad(apcloud_ctx *c, apcloud_mpnn *m, const double *b, bool 
         }
     }
     APC_CUDA(c, cudaGetLastError());
-    APC_TRY(check_tc(c, m));
-    double h[4];
+    // the loss and the tensor-core layers' error word in one read
+    APC_CUDA(c, cudaMemcpyAsync(lossv + 4, m->err, sizeof(unsigned), cudaMemcpyDeviceToDevice, c->s));
+    double h[5];
     APC_TRY(read_back(c, h, lossv, sizeof h));
+    unsigned e;
+    memcpy(&e, h + 4, sizeof e);
+    APC_TRY(tc_error(c, e));
     if (h_loss) { h_loss[0] = h[0]; h_loss[1] = h[1]; h_loss[2] = h[2]; }
     return APCLOUD_OK;
 }
