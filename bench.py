@@ -852,11 +852,10 @@ def run_profile(args):
       solve: the 1e7-particle depth-10 beam (1.05e6 nodes): tree, stencils,
              deposit, then --profile-iters Arnoldi steps of the Poisson solve
              (GMRES(30), polynomial degree 16) in --precision; --profile-sorted
-             sweeps and Arnoldi products on the width-sorted matrix at the
-             shape the autotuner picks for it (128 threads, two 4-entry chunks
-             in flight; 4 nodes per stencil block).
+             sweeps and Arnoldi products on the block-local copy of the matrix
+             (4 nodes per stencil block).
       batch: the 64-beam depth-9 batch, then --profile-iters Arnoldi steps
-             (--profile-sorted: 128 threads, two chunks in flight).
+             (--profile-sorted as above, 8 nodes per stencil block).
       mpnn:  --profile-iters training steps of the learned preconditioner on
              a 2e5-particle depth-8 beam.
       small: one whole solve (tree, stencils, deposit, Poisson solve, gather)

@@ -353,11 +353,11 @@ apcloud_status apcloud_set_graphs(apcloud_ctx *ctx, int enable);
  * ones) for every shape of the
  * row-parallel products: 64, 128, 256 and 512 threads per block, each with
  * the loads of 1 or 4 stencil entries issued ahead of their multiply-adds
- * (on the width-sorted copy: 1 or 2 chunks of 4 entries; the sum keeps its
- * order either way), and -- for the FP16 sweeps and FP32 Arnoldi products of
- * the mixed form -- on the sliced ELL and on its width-sorted copy (rows
- * ordered by stencil width inside 256-row windows, so 32-row slices carry
- * little padding; same entries in the same order per row).  The solves run on scratch vectors and the
+ * (the sum keeps its order either way), and -- for the FP16 sweeps and FP32
+ * Arnoldi products of the mixed form -- on the sliced ELL and on its
+ * block-local copy (a block's distinct columns in shared memory, 16-bit
+ * indices; one launch shape; same entries in the same order per row).  The
+ * solves run on scratch vectors and the
  * graphs they capture are released; bit 1 times the stencil build (neighbour
  * search + WLS) at 2, 4 and 8 nodes (warps) per block on the current node
  * set.  The fastest shapes are kept for later calls and written to
@@ -376,17 +376,15 @@ apcloud_status apcloud_autotune(apcloud_ctx *ctx, unsigned what, int *h_spmv_blo
 apcloud_status apcloud_set_launch_shape(apcloud_ctx *ctx, int spmv_block, int spmv_unroll, int sweep_sorted,
                                         int wls_warps);
 
-/* L2 residency of the FP16 sweep matrix (width-sorted copy with packed
- * columns, the mixed form's polynomial preconditioner).  The sweeps of one
- * polynomial application read the whole matrix one after another; a sweep
- * loads its first keep_bytes of matrix bytes (5 per stored entry) as
- * ordinary loads and the rest as streaming loads (ld.global.cs: lines
- * allocated evict-first in L2), so that the streamed part replaces itself in
- * L2 and the kept part is still there for the next sweep.  keep_bytes = -1
- * (the default): 0.4 of the L2 when the matrix and the sweep's vectors (12
- * bytes per row) take between 3/4 of the L2 and twice the L2, else all of
- * the matrix (no streaming loads); 0: every matrix load streaming; larger
- * than the matrix: none.
+/* L2 residency of the FP16 sweep matrix (block-local copy, the mixed form's
+ * polynomial preconditioner).  The sweeps of one polynomial application read
+ * the whole matrix one after another; a sweep loads keep_bytes of matrix bytes
+ * (4 per stored entry, rounded down to sixteenths of the matrix) as ordinary
+ * loads and the rest as evict-first lines, so that the rest replaces itself in
+ * L2 and the kept part, evenly spread over the matrix, is still there for the
+ * next sweep.  keep_bytes = -1 (the default): all of the matrix when it and
+ * the sweep's vectors (12 bytes per row) take at most 3/4 of the L2, else 0.3
+ * of the L2; 0: every matrix load evict-first; larger than the matrix: none.
  * Results are bit-identical for every value (the same loads in the same
  * order).  APCLOUD_E_INVALID for keep_bytes < -1.  The getter writes the
  * value in effect for the current node set (the automatic choice resolved;
@@ -395,7 +393,7 @@ apcloud_status apcloud_set_launch_shape(apcloud_ctx *ctx, int spmv_block, int sp
 /* Programmatic dependent launch of the polynomial's sweeps (on by default):
  * every sweep after the first of an application is launched so that its
  * blocks may start while the sweep before it drains; each row reads its
- * slice, b, the solver state and its first matrix chunks, then waits on the
+ * length, b, the solver state and its matrix entries, then waits on the
  * device (griddepcontrol.wait) for the previous sweep to complete before it
  * reads x or writes y.  enable = 0 launches every sweep in plain stream
  * order.  Results are bit-identical either way.  The paper has no

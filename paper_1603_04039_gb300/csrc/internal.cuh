@@ -180,7 +180,7 @@ struct apcloud_ctx {
     // launch shapes chosen by apcloud_autotune
     int spmv_bs = 256;     // threads per block of the Arnoldi products and sweeps
     int spmv_unroll = 1;   // stencil entries whose loads a thread issues ahead (1 or 4)
-    int sweep_sorted = 0;  // 1: FP16 sweeps on the width-sorted matrix (autotuner's choice)
+    int sweep_sorted = 1;  // 1: FP16 sweeps and FP32 products on the block-local copy (autotuner's choice)
     bool pdl_on = true;        // sweeps after the first of a polynomial application as programmatic dependents
     int64_t sweep_keep = -1;   // bytes of that matrix the sweeps read with ordinary loads, the rest streaming (-1: automatic)
     int jprev[2][2] = {{0, 0}, {0, 0}};   // Arnoldi steps of the last cycle, per system (B, A) and FP64/FP32
@@ -235,13 +235,13 @@ struct apcloud_ctx {
     apc::DBuf slice_w, slice_off, ell_col, ell_A, ell_B, dA, dB;
     apc::DBuf ell_A32, ell_B32;  // FP32 copies for the inner iterations of the mixed form
     apc::DBuf ell_A16, ell_B16;  // FP16 copies for the preconditioner sweeps of the mixed form
-    // width-sorted copy of the FP16 sweep matrix: rows ordered by stencil width
-    // inside windows of 256 rows, so 32-row slices pad little (see rank_sorted_sweep)
-    apc::DBuf ss_perm, ss_w, ss_o, ss_col, ss_A, ss_B;
-    apc::DBuf ss_col24;                             // chunk columns of the sorted copy, 24 bits each
-    apc::DBuf stencil_ovf;                          // nodes whose k-ring outgrew MAXC_FAST candidates
-    bool ss_col24_ok = false;
-    apc::DBuf ss_A32, ss_B32;   // FP32 values in the same layout (Arnoldi products of the mixed form)
+    // block-local copy of the sweep matrix (sweep.cu): slice offsets in chunks, row
+    // lengths, the blocks' lists of other blocks' nodes, 16-bit indices, FP16 and
+    // FP32 values; tried: built since the operators were, ok: every block's list fits
+    apc::DBuf bl_w4, bl_off, bl_len, bl_hlist, bl_hcnt, bl_idx, bl_A, bl_B, bl_A32, bl_B32;
+    int64_t bl_chunks = 0;     // 32-lane chunks of 4 entries
+    bool bl_ok = false, bl_tried = false;
+    apc::DBuf stencil_ovf;     // nodes whose k-ring outgrew MAXC_FAST candidates
     apc::DBuf beam_part;        // per-beam norms: partial sums, BSQ_CH per beam
     apc::DBuf tune_b, tune_x;   // autotuner: right-hand side and iterate of its timed restart cycles
     // ILU(0) comparison solve: factors of system ilu_which while it runs (-1: none)
@@ -249,8 +249,6 @@ struct apcloud_ctx {
     int ilu_which = -1;
     apc::DBuf ilu_lrows, ilu_urows, ilu_lrp, ilu_urp, ilu_lcol, ilu_ucol, ilu_lval, ilu_uval, ilu_dinv;
     apc::DBuf ilu_loff, ilu_uoff;   // level offsets of the two sweeps, for the one-block runs of small levels
-    bool ss_ok = false;
-    int64_t ss_entries = 0;
     // solver
     apc::DBuf V, w0, w1, u, b, partial, gstate, rho_m, rho, phi, nodefield, tmp;
     apc::DBuf nodefield32;   // mixed form: compact node records of the particle pass
@@ -347,9 +345,21 @@ apcloud_status build_octree(apcloud_ctx *c, const double *x, const double *y, co
                             const int64_t *h_offsets, int nbeams);
 apcloud_status node_beams(apcloud_ctx *c, int32_t *out);
 apcloud_status refresh_lowp(apcloud_ctx *c);          // FP32/FP16 matrix copies from the FP64 values
-// width-sorted sweep matrix: its ranks and slices (entry columns to *d_total), then its entries from the ELL
-apcloud_status rank_sorted_sweep(apcloud_ctx *c, uint32_t *d_total);
-apcloud_status fill_sorted_sweep(apcloud_ctx *c);
+// Block-local copy of the sweep matrix (sweep.cu): its chunk count (to
+// *d_total), then, with bl_chunks known, the copy
+apcloud_status count_blocks(apcloud_ctx *c, uint32_t *d_total);
+apcloud_status build_blocks(apcloud_ctx *c);
+// Rows of beams that have converged in a batch (both null outside batches):
+// their Krylov vectors are zero, so the products skip them.
+struct RowSkip {
+    const int32_t *nbo;   // beam of every node
+    const int *bdone;     // 1 once the beam has converged (or finished its cycle)
+    const double *binv;   // per-beam Krylov spaces: 1 / ||w|| of each beam (null: st->inv_norm)
+};
+void block_sweep(apcloud_ctx *c, int which, const float *x, float *y, const float *b, const GmresState *st,
+                 RowSkip skip, int keep, bool pdl);
+void block_product(apcloud_ctx *c, int which, const float *x, float *y, const GmresState *st, RowSkip skip);
+int block_keep(double fraction);   // the `keep` of block_sweep that keeps this fraction of the matrix in L2
 double *poisson_rhs(apcloud_ctx *c, const double *g);  // b of the Poisson system into c->b
 apcloud_status tune_spmv(apcloud_ctx *c, double *ms_out);      // ms per sweep at 64/128/256/512 threads
 int64_t sweep_keep_bytes(const apcloud_ctx *c);                 // sweep matrix bytes read with ordinary loads

@@ -253,162 +253,6 @@ __device__ __forceinline__ float row_dot_h(const __half *__restrict__ val, const
     return acc;
 }
 
-// Resident blocks asked of the width-sorted row kernels: with two chunks in
-// flight (U > 1) they fit 32 registers without spilling, so blocks of up to
-// 256 threads fill the SM's 64 warps (left to itself the compiler takes more
-// registers and fewer warps); the one-chunk form spills at 32 or 40
-// registers and keeps the compiler's choice.  The FP32 product with packed
-// columns needs 40 (48 warps).
-#define SS_MINB(BS, U) (((U) > 1 && (BS) <= 256) ? 2048 / (BS) : 1)
-
-// A row of the width-sorted sweep matrix.  A slice of width w stores its first
-// 4 * floor(w / 4) columns lane-major in 4-entry chunks (chunk j of lane l at
-// entries sbase + 128 j + 4 l .. + 3: one 16-byte column load and one 8-byte
-// value load per chunk) and the last w % 4 columns slice-major as in the ELL.
-// The entries are summed in the same order as row_dot_h.  The columns and
-// values of the next chunk (U = 1) or the next two (U > 1) are in flight
-// while a chunk's x entries are gathered.
-template <int U>
-__device__ __forceinline__ float row_dot_c(const __half *__restrict__ val, const int32_t *__restrict__ col,
-                                           const float *__restrict__ x, int64_t sbase, int lane, int w) {
-    constexpr int AH = (U > 1) ? 2 : 1;   // chunks whose loads are in flight
-    const int4 z4 = make_int4(0, 0, 0, 0);
-    const uint2 z2 = make_uint2(0u, 0u);
-    float acc = 0.f;
-    const int nch = w >> 2;
-    const int4 *c4 = reinterpret_cast<const int4 *>(col + sbase) + lane;
-    const uint2 *v4 = reinterpret_cast<const uint2 *>(val + sbase) + lane;
-    int4 cq[AH];
-    uint2 vq[AH];
-#pragma unroll
-    for (int a = 0; a < AH; ++a) {
-        cq[a] = a < nch ? c4[(int64_t)a * 32] : z4;
-        vq[a] = a < nch ? v4[(int64_t)a * 32] : z2;
-    }
-    for (int j = 0; j < nch; ++j) {
-        const int4 c0 = cq[0];
-        const uint2 v0 = vq[0];
-#pragma unroll
-        for (int a = 0; a + 1 < AH; ++a) {
-            cq[a] = cq[a + 1];
-            vq[a] = vq[a + 1];
-        }
-        cq[AH - 1] = (j + AH < nch) ? c4[(int64_t)(j + AH) * 32] : z4;
-        vq[AH - 1] = (j + AH < nch) ? v4[(int64_t)(j + AH) * 32] : z2;
-        const float x0 = x[c0.x], x1 = x[c0.y], x2 = x[c0.z], x3 = x[c0.w];
-        const float2 f01 = __half22float2(*reinterpret_cast<const __half2 *>(&v0.x));
-        const float2 f23 = __half22float2(*reinterpret_cast<const __half2 *>(&v0.y));
-        acc = fmaf(f01.x, x0, acc);
-        acc = fmaf(f01.y, x1, acc);
-        acc = fmaf(f23.x, x2, acc);
-        acc = fmaf(f23.y, x3, acc);
-    }
-    const int64_t tb = sbase + (int64_t)nch * 128 + lane;
-    for (int k = 0; k < (w & 3); ++k) acc = fmaf(__half2float(val[tb + (int64_t)k * 32]), x[col[tb + (int64_t)k * 32]], acc);
-    return acc;
-}
-
-// Programmatic dependent launch (APC_LAUNCH_PDL).  A kernel launched with the
-// attribute may start while the kernel before it in the stream is running,
-// once every block of that kernel has executed griddepcontrol.launch_dependents
-// (or exited); griddepcontrol.wait returns once that kernel has completed and
-// its writes are visible.  Without the attribute the wait returns at once.
-// A sweep lets the next one start only after its own wait: so sweep i + 1
-// never runs beside sweep i - 1, which read the buffer (through the SM's
-// read-only cache) that sweep i rewrites and sweep i + 1 reads.  With the
-// release at block start, small grids ran three sweeps side by side and
-// sweep i + 1 read lines that sweep i - 1 had cached: wrong results.
-__device__ __forceinline__ void grid_dep_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-// L2 eviction priority of the sweep's matrix loads.  The polynomial's sweeps
-// follow one another, each reading the whole width-sorted matrix, so what
-// the L2 still holds of one sweep's matrix the next one reads from there.
-// A matrix larger than the L2 read as a plain cyclic stream leaves nothing
-// to reuse (every line is evicted before its next read); with the slices
-// past a threshold read as streaming data (ld.global.cs, __ldcs: lines
-// allocated evict-first in L1 and L2), those lines replace one another and
-// the slices below it stay resident.  The cache operator only steers the
-// caches: the loads, and the results, are the same.
-
-// row_dot_c with the chunks' columns packed to 24 bits: chunk j of lane l is
-// three words at pbase + 96 j + 32 p + l (p = 0, 1, 2), read by three
-// coalesced 4-byte loads; the last w % 4 columns stay in the 32-bit array.
-// Same entries in the same order: the same bits as row_dot_c.  With EF the
-// matrix loads are streaming loads; the two forms are separate
-// instantiations, chosen per row, so each keeps the 32-register bound.  The
-// grid-dependency wait (grid_dep_wait) comes after the first chunks' loads
-// are issued and before any x is read; xr receives x[r].
-template <int U, bool EF>
-__device__ __forceinline__ float row_dot_c24(const __half *__restrict__ val, const int32_t *__restrict__ col,
-                                             const uint32_t *__restrict__ col24, const float *__restrict__ x,
-                                             int64_t sbase, int64_t pbase, int lane, int w, int r, float &xr) {
-    constexpr int AH = (U > 1) ? 2 : 1;   // chunks whose loads are in flight
-    float acc = 0.f;
-    const int nch = w >> 2;
-    const uint32_t *p0 = col24 + pbase + lane;
-    const uint2 *v4 = reinterpret_cast<const uint2 *>(val + sbase) + lane;
-    uint3 cq[AH];
-    uint2 vq[AH];
-    auto load = [&](int a, uint3 &c, uint2 &v) {
-        if (a >= nch) {
-            c = make_uint3(0u, 0u, 0u);
-            v = make_uint2(0u, 0u);
-        } else {
-            const uint32_t *q = p0 + (int64_t)a * 96;
-            const uint2 *u = v4 + (int64_t)a * 32;
-            if (EF) {
-                c = make_uint3(__ldcs(q), __ldcs(q + 32), __ldcs(q + 64));
-                v = __ldcs(u);
-            } else {
-                c = make_uint3(q[0], q[32], q[64]);
-                v = *u;
-            }
-        }
-    };
-#pragma unroll
-    for (int a = 0; a < AH; ++a) load(a, cq[a], vq[a]);
-    grid_dep_wait();
-    xr = x[r];
-    for (int j = 0; j < nch; ++j) {
-        const uint3 c0 = cq[0];
-        const uint2 v0 = vq[0];
-#pragma unroll
-        for (int a = 0; a + 1 < AH; ++a) {
-            cq[a] = cq[a + 1];
-            vq[a] = vq[a + 1];
-        }
-        load(j + AH, cq[AH - 1], vq[AH - 1]);
-        const uint32_t i0 = c0.x & 0xFFFFFFu, i1 = (c0.x >> 24) | ((c0.y & 0xFFFFu) << 8),
-                       i2 = (c0.y >> 16) | ((c0.z & 0xFFu) << 16), i3 = c0.z >> 8;
-        const float x0 = x[i0], x1 = x[i1], x2 = x[i2], x3 = x[i3];
-        const float2 f01 = __half22float2(*reinterpret_cast<const __half2 *>(&v0.x));
-        const float2 f23 = __half22float2(*reinterpret_cast<const __half2 *>(&v0.y));
-        acc = fmaf(f01.x, x0, acc);
-        acc = fmaf(f01.y, x1, acc);
-        acc = fmaf(f23.x, x2, acc);
-        acc = fmaf(f23.y, x3, acc);
-    }
-    const int64_t tb = sbase + (int64_t)nch * 128 + lane;
-    for (int k = 0; k < (w & 3); ++k) {
-        const __half *hv = val + tb + (int64_t)k * 32;
-        const int32_t *hc = col + tb + (int64_t)k * 32;
-        const float fv = __half2float(EF ? __ldcs(hv) : *hv);
-        acc = fmaf(fv, x[EF ? __ldcs(hc) : *hc], acc);
-    }
-    return acc;
-}
-
-// Rows of beams that have converged in a batch (both null outside batches):
-// their Krylov vectors are zero, so the products skip them.
-struct RowSkip {
-    const int32_t *nbo;   // beam of every node
-    const int *bdone;     // 1 once the beam has converged (or finished its cycle)
-    const double *binv;   // per-beam Krylov spaces: 1 / ||w|| of each beam (null: st->inv_norm)
-};
-
 // BS: threads per block (one row each; mode 2 strides over the rows with a
 // grid of resid_blocks(n) blocks of RT threads: one block per row block put
 // 4118 same-address ticket atomics on the last-block test of a 1.05e6-row
@@ -499,247 +343,32 @@ __global__ void __launch_bounds__(BS) k_sweep_h(const uint32_t *__restrict__ sw,
     y[r] = fmaf(om, b[r] - acc, x[r]);
 }
 
-// The same sweep on the width-sorted copy: thread = slot of a 32-slot slice,
-// its row from the window's permutation (entries in the same order, so the
-// same bits as k_sweep_h).  With packed columns and KS, slices stored from
-// entry `keep` on are read as streaming (evict-first) loads; without KS
-// (no threshold in effect) the kernel holds the ordinary form alone, whose
-// code the branch slows by 5% (98 against 103 us per sweep of a 64-beam
-// batch).
-template <int BS, int U = 1, bool P24 = false, bool KS = false>
-__global__ void __launch_bounds__(BS, SS_MINB(BS, U)) k_sweep_s(const int32_t *__restrict__ perm, const uint32_t *__restrict__ sw,
-                                                const uint32_t *__restrict__ soff, const int32_t *__restrict__ col,
-                                                const __half *__restrict__ val, int64_t nslot,
-                                                const float *__restrict__ x, float *__restrict__ y,
-                                                const float *__restrict__ b, const GmresState *__restrict__ st,
-                                                RowSkip skip, const uint32_t *__restrict__ col24, int64_t keep) {
-    // Sweeps after the first of a polynomial application are launched as
-    // programmatic dependents of the sweep before them, whose y is their x:
-    // a row reads its slice, b, the state and its first chunks before the
-    // grid-dependency wait (none of them is written by a sweep), x and y only
-    // after it.  The row's own loads are issued before the state is read (in
-    // batches after the test for a converged beam, whose rows read nothing
-    // more).
-    const int64_t sl_ = (int64_t)blockIdx.x * BS + threadIdx.x;
-    if (sl_ >= nslot) return;
-    const int r = perm[sl_];
-    const int sl = (int)(sl_ >> 5), lane = (int)(sl_ & 31);
-    const int w = (int)sw[sl];
-    const int64_t sb = (int64_t)soff[sl] * 32;
-    float br, xr;
-    if (!skip.nbo) {
-        br = b[r < 0 ? 0 : r];
-        if (st->done || r < 0) return;
-    } else {
-        if (st->done || r < 0) return;
-        if (skip.bdone[skip.nbo[r]]) {
-            grid_dep_wait();
-            y[r] = 0.f;
-            return;
-        }
-        br = b[r];
-    }
-    const float om = (float)st->omega;
-    float acc;
-    if (!P24) {
-        grid_dep_wait();
-        xr = x[r];
-        acc = row_dot_c<U>(val, col, x, sb, lane, w);
-    } else if (KS && sb >= keep) {
-        acc = row_dot_c24<U, true>(val, col, col24, x, sb, (int64_t)soff[sl] * 24, lane, w, r, xr);
-    } else {
-        acc = row_dot_c24<U, false>(val, col, col24, x, sb, (int64_t)soff[sl] * 24, lane, w, r, xr);
-    }
-    y[r] = fmaf(om, br - acc, xr);
-}
-
-// A row of the width-sorted copy with FP32 values: the same chunked layout as
-// row_dot_c (one 16-byte column load and one 16-byte value load per 4-entry
-// chunk, one or two chunks in flight), the entries in their stored order.
-template <int U>
-__device__ __forceinline__ float row_dot_cf(const float *__restrict__ val, const int32_t *__restrict__ col,
-                                            const float *__restrict__ x, int64_t sbase, int lane, int w) {
-    constexpr int AH = (U > 1) ? 2 : 1;
-    const int4 z4 = make_int4(0, 0, 0, 0);
-    const float4 zf = make_float4(0.f, 0.f, 0.f, 0.f);
-    float acc = 0.f;
-    const int nch = w >> 2;
-    const int4 *c4 = reinterpret_cast<const int4 *>(col + sbase) + lane;
-    const float4 *v4 = reinterpret_cast<const float4 *>(val + sbase) + lane;
-    int4 cq[AH];
-    float4 vq[AH];
-#pragma unroll
-    for (int a = 0; a < AH; ++a) {
-        cq[a] = a < nch ? c4[(int64_t)a * 32] : z4;
-        vq[a] = a < nch ? v4[(int64_t)a * 32] : zf;
-    }
-    for (int j = 0; j < nch; ++j) {
-        const int4 c0 = cq[0];
-        const float4 v0 = vq[0];
-#pragma unroll
-        for (int a = 0; a + 1 < AH; ++a) {
-            cq[a] = cq[a + 1];
-            vq[a] = vq[a + 1];
-        }
-        cq[AH - 1] = (j + AH < nch) ? c4[(int64_t)(j + AH) * 32] : z4;
-        vq[AH - 1] = (j + AH < nch) ? v4[(int64_t)(j + AH) * 32] : zf;
-        const float x0 = x[c0.x], x1 = x[c0.y], x2 = x[c0.z], x3 = x[c0.w];
-        acc = fmaf(v0.x, x0, acc);
-        acc = fmaf(v0.y, x1, acc);
-        acc = fmaf(v0.z, x2, acc);
-        acc = fmaf(v0.w, x3, acc);
-    }
-    const int64_t tb = sbase + (int64_t)nch * 128 + lane;
-    for (int k = 0; k < (w & 3); ++k) acc = fmaf(val[tb + (int64_t)k * 32], x[col[tb + (int64_t)k * 32]], acc);
-    return acc;
-}
-
-// row_dot_cf with the chunks' columns packed to 24 bits (see row_dot_c24):
-// the same entries in the same order, the same bits
-template <int U>
-__device__ __forceinline__ float row_dot_cf24(const float *__restrict__ val, const int32_t *__restrict__ col,
-                                              const uint32_t *__restrict__ col24, const float *__restrict__ x,
-                                              int64_t sbase, int64_t pbase, int lane, int w) {
-    constexpr int AH = (U > 1) ? 2 : 1;
-    const uint3 z3 = make_uint3(0u, 0u, 0u);
-    const float4 zf = make_float4(0.f, 0.f, 0.f, 0.f);
-    float acc = 0.f;
-    const int nch = w >> 2;
-    const uint32_t *p0 = col24 + pbase + lane;
-    const float4 *v4 = reinterpret_cast<const float4 *>(val + sbase) + lane;
-    uint3 cq[AH];
-    float4 vq[AH];
-#pragma unroll
-    for (int a = 0; a < AH; ++a) {
-        cq[a] = a < nch ? make_uint3(p0[a * 96], p0[a * 96 + 32], p0[a * 96 + 64]) : z3;
-        vq[a] = a < nch ? v4[(int64_t)a * 32] : zf;
-    }
-    for (int j = 0; j < nch; ++j) {
-        const uint3 c0 = cq[0];
-        const float4 v0 = vq[0];
-#pragma unroll
-        for (int a = 0; a + 1 < AH; ++a) {
-            cq[a] = cq[a + 1];
-            vq[a] = vq[a + 1];
-        }
-        const int64_t jn = (int64_t)(j + AH) * 96;
-        cq[AH - 1] = (j + AH < nch) ? make_uint3(p0[jn], p0[jn + 32], p0[jn + 64]) : z3;
-        vq[AH - 1] = (j + AH < nch) ? v4[(int64_t)(j + AH) * 32] : zf;
-        const uint32_t i0 = c0.x & 0xFFFFFFu, i1 = (c0.x >> 24) | ((c0.y & 0xFFFFu) << 8),
-                       i2 = (c0.y >> 16) | ((c0.z & 0xFFu) << 16), i3 = c0.z >> 8;
-        const float x0 = x[i0], x1 = x[i1], x2 = x[i2], x3 = x[i3];
-        acc = fmaf(v0.x, x0, acc);
-        acc = fmaf(v0.y, x1, acc);
-        acc = fmaf(v0.z, x2, acc);
-        acc = fmaf(v0.w, x3, acc);
-    }
-    const int64_t tb = sbase + (int64_t)nch * 128 + lane;
-    for (int k = 0; k < (w & 3); ++k) acc = fmaf(val[tb + (int64_t)k * 32], x[col[tb + (int64_t)k * 32]], acc);
-    return acc;
-}
-
-// y = Ahat x on the width-sorted FP32 copy, skipped once the cycle is done
-// (the Arnoldi product of k_spmv<4, float> with the same bits)
-template <int BS, int U = 1, bool P24 = false>
-__global__ void __launch_bounds__(BS, (P24 && SS_MINB(BS, U) > 1) ? 1536 / BS : SS_MINB(BS, U)) k_spmv_s(const int32_t *__restrict__ perm, const uint32_t *__restrict__ sw,
-                                               const uint32_t *__restrict__ soff, const int32_t *__restrict__ col,
-                                               const float *__restrict__ val, int64_t nslot,
-                                               const float *__restrict__ x, float *__restrict__ y,
-                                               const GmresState *__restrict__ st, RowSkip skip,
-                                               const uint32_t *__restrict__ col24) {
-    const int64_t sl_ = (int64_t)blockIdx.x * BS + threadIdx.x;
-    if (sl_ >= nslot) return;
-    const int r = perm[sl_];
-    const int sl = (int)(sl_ >> 5), lane = (int)(sl_ & 31);
-    const int w = (int)sw[sl];
-    const int64_t sb = (int64_t)soff[sl] * 32;
-    if (st->done || r < 0) return;
-    if (skip.nbo && skip.bdone[skip.nbo[r]]) {
-        y[r] = 0.f;
-        return;
-    }
-    y[r] = P24 ? row_dot_cf24<U>(val, col, col24, x, sb, (int64_t)soff[sl] * 24, lane, w)
-               : row_dot_cf<U>(val, col, x, sb, lane, w);
-}
-
-// r = b - Ahat u and ||r||^2 (the restart residual, MODE 2 of k_spmv) on the
-// width-sorted FP32 copy with 24-bit chunk columns: every row's entries in the
-// same order as on the ELL (the same r), the norm summed over the sorted slots
-// by a grid of resid_blocks blocks striding over them
-template <int U>
-__global__ void __launch_bounds__(RT) k_resid_s(const int32_t *__restrict__ perm, const uint32_t *__restrict__ sw,
-                                                const uint32_t *__restrict__ soff, const int32_t *__restrict__ col,
-                                                const float *__restrict__ val, const uint32_t *__restrict__ col24,
-                                                int64_t nslot, const float *__restrict__ x, float *__restrict__ y,
-                                                const float *__restrict__ b, GmresState *st,
-                                                double *__restrict__ partial) {
-    __shared__ double sm[RT + RT / 32 + 8];
-    double yv = 0.0;
-    for (int64_t sl_ = (int64_t)blockIdx.x * RT + threadIdx.x; sl_ < nslot; sl_ += (int64_t)gridDim.x * RT) {
-        const int r = perm[sl_];
-        if (r >= 0) {
-            const int sl = (int)(sl_ >> 5), lane = (int)(sl_ & 31);
-            const int w = (int)sw[sl];
-            const int64_t sb = (int64_t)soff[sl] * 32;
-            const float acc = row_dot_cf24<U>(val, col, col24, x, sb, (int64_t)soff[sl] * 24, lane, w);
-            const float t = b[r] - acc;
-            y[r] = t;
-            yv = fma((double)t, (double)t, yv);
-        }
-    }
-    double a[1] = {yv};
-    double tot = 0.0;
-    block_reduce_many<1>(a, 1, sm, &tot);
-    if (threadIdx.x == 0) partial[blockIdx.x * 64] = tot;
-    if (last_block(&st->ticket)) {
-        __shared__ double fs[1];
-        final_sums(partial, gridDim.x, 1, sm, fs);
-        if (threadIdx.x == 0) {
-            const double beta = sqrt(fs[0]);
-            st->beta = beta;
-            st->g[0] = beta;
-            for (int i = 1; i <= MAX_RESTART; ++i) st->g[i] = 0.0;
-            st->jend = 0;
-            st->done = (beta <= st->rtol * st->bnorm) ? 1 : 0;
-            st->inv_norm = beta > 0.0 ? 1.0 / beta : 0.0;
-            st->ticket = 0;
-        }
-    }
-}
-
 // Row-parallel products of the Arnoldi steps and sweeps at the block size the
 // autotuner chose (64, 128, 256 or 512 threads).
-#define APC_ROWS_BS_WITH(LAUNCH, c, kind, n, KERNEL_OF, ...)                                                \
-    do {                                                                                                    \
-        if ((c)->spmv_unroll == 4) {                                                                        \
-            switch ((c)->spmv_bs) {                                                                         \
-            case 64: LAUNCH(c, kind, div_up(n, 64), 64, 0, KERNEL_OF(64, 4), __VA_ARGS__); break;         \
-            case 128: LAUNCH(c, kind, div_up(n, 128), 128, 0, KERNEL_OF(128, 4), __VA_ARGS__); break;     \
-            case 512: LAUNCH(c, kind, div_up(n, 512), 512, 0, KERNEL_OF(512, 4), __VA_ARGS__); break;     \
-            default: LAUNCH(c, kind, div_up(n, 256), 256, 0, KERNEL_OF(256, 4), __VA_ARGS__); break;      \
-            }                                                                                               \
-        } else {                                                                                            \
-            switch ((c)->spmv_bs) {                                                                         \
-            case 64: LAUNCH(c, kind, div_up(n, 64), 64, 0, KERNEL_OF(64, 1), __VA_ARGS__); break;         \
-            case 128: LAUNCH(c, kind, div_up(n, 128), 128, 0, KERNEL_OF(128, 1), __VA_ARGS__); break;     \
-            case 512: LAUNCH(c, kind, div_up(n, 512), 512, 0, KERNEL_OF(512, 1), __VA_ARGS__); break;     \
-            default: LAUNCH(c, kind, div_up(n, 256), 256, 0, KERNEL_OF(256, 1), __VA_ARGS__); break;      \
-            }                                                                                               \
-        }                                                                                                   \
+#define APC_ROWS_BS(c, kind, n, KERNEL_OF, ...)                                                                 \
+    do {                                                                                                        \
+        if ((c)->spmv_unroll == 4) {                                                                            \
+            switch ((c)->spmv_bs) {                                                                             \
+            case 64: APC_LAUNCH(c, kind, div_up(n, 64), 64, 0, KERNEL_OF(64, 4), __VA_ARGS__); break;         \
+            case 128: APC_LAUNCH(c, kind, div_up(n, 128), 128, 0, KERNEL_OF(128, 4), __VA_ARGS__); break;     \
+            case 512: APC_LAUNCH(c, kind, div_up(n, 512), 512, 0, KERNEL_OF(512, 4), __VA_ARGS__); break;     \
+            default: APC_LAUNCH(c, kind, div_up(n, 256), 256, 0, KERNEL_OF(256, 4), __VA_ARGS__); break;      \
+            }                                                                                                   \
+        } else {                                                                                                \
+            switch ((c)->spmv_bs) {                                                                             \
+            case 64: APC_LAUNCH(c, kind, div_up(n, 64), 64, 0, KERNEL_OF(64, 1), __VA_ARGS__); break;         \
+            case 128: APC_LAUNCH(c, kind, div_up(n, 128), 128, 0, KERNEL_OF(128, 1), __VA_ARGS__); break;     \
+            case 512: APC_LAUNCH(c, kind, div_up(n, 512), 512, 0, KERNEL_OF(512, 1), __VA_ARGS__); break;     \
+            default: APC_LAUNCH(c, kind, div_up(n, 256), 256, 0, KERNEL_OF(256, 1), __VA_ARGS__); break;      \
+            }                                                                                                   \
+        }                                                                                                       \
     } while (0)
-#define APC_ROWS_BS(c, kind, n, KERNEL_OF, ...) APC_ROWS_BS_WITH(APC_LAUNCH, c, kind, n, KERNEL_OF, __VA_ARGS__)
 #define APC_SPMV_BS(c, n, KERNEL_OF, ...) APC_ROWS_BS(c, K_SPMV, n, KERNEL_OF, __VA_ARGS__)
 #define APC_SWEEP_BS(c, n, KERNEL_OF, ...) APC_ROWS_BS(c, K_SWEEP, n, KERNEL_OF, __VA_ARGS__)
-#define APC_SWEEP_BS_PDL(c, n, KERNEL_OF, ...) APC_ROWS_BS_WITH(APC_LAUNCH_PDL, c, K_SWEEP, n, KERNEL_OF, __VA_ARGS__)
 #define APC_SPMV1(B, U) (k_spmv<1, T, B, U>)
 #define APC_SPMV3(B, U) (k_spmv<3, T, B, U>)
 #define APC_SPMV4(B, U) (k_spmv<4, T, B, U>)
 #define APC_SWEEPH(B, U) (k_sweep_h<B, U>)
-#define APC_SWEEPS(B, U) (k_sweep_s<B, U, false>)
-#define APC_SWEEPS24(B, U) (k_sweep_s<B, U, true>)
-#define APC_SWEEPS24K(B, U) (k_sweep_s<B, U, true, true>)
-#define APC_SPMVS(B, U) (k_spmv_s<B, U, false>)
-#define APC_SPMVS24(B, U) (k_spmv_s<B, U, true>)
 
 
 // ---------------------------------------------------------------- Gram-Schmidt passes
@@ -1544,6 +1173,8 @@ int sm_count() {
     return sms > 0 ? sms : 152;
 }
 
+constexpr double KEEP_ALL = 0.75, KEEP_PART = 0.3;   // sweep_keep_bytes
+
 int64_t l2_bytes() {
     int b = 0, dev = 0;
     cudaGetDevice(&dev);
@@ -1551,35 +1182,33 @@ int64_t l2_bytes() {
     return b > 0 ? b : (int64_t)126 << 20;
 }
 
-// Bytes a sweep reads per stored entry of the packed width-sorted matrix (a
-// 2-byte value and 3 bytes of packed column) and per row (x and b read, y
-// written, FP32).
-constexpr double SWEEP_ENTRY_BYTES = 5.0, SWEEP_ROW_BYTES = 12.0;
+// Bytes a sweep reads per stored entry of the block-local copy (FP16 value and
+// 16-bit index) and per row (x and b read, y written, FP32).
+constexpr double SWEEP_ENTRY_BYTES = 4.0, SWEEP_ROW_BYTES = 12.0;
+
+double sweep_matrix_bytes(const apcloud_ctx *c) { return SWEEP_ENTRY_BYTES * 128.0 * (double)c->bl_chunks; }
 
 }  // namespace
 
 // Matrix bytes the sweeps read with ordinary loads when left to the library:
-// all of them when the matrix and the sweep's vectors fit in 3/4 of the L2;
-// 0.4 of the L2 when they take up to twice the L2 (the rest of the L2 holds
-// the vectors and the streamed lines; on the 1.05e6-row, 145 MB matrix of a
-// 1e7-particle beam at depth 10 kept sizes of 0.2 to 0.5 of the L2 gave
-// 30.5 to 31.2 us per sweep against 35.3 us with no streaming loads and
-// 33.0 us with streaming loads only); all of them again beyond (a 650 MB
-// matrix of a 64-beam batch gained nothing from the 8% that can stay and
-// lost 2% to the streaming loads).
+// all of them when the matrix and the sweep's vectors fit in KEEP_ALL of the
+// L2; else KEEP_PART of the L2 (the rest holds the vectors and the streamed
+// lines).  Solve times with 0, 20, 40, 50 MB and all of it kept: 21.3, 19.4,
+// 18.8, 18.6, 18.4 ms at 4.9e5 rows; 48.9, 46.9, 45.5, 45.9, 55.5 ms at 1.05e6;
+// 127.6, 127.6, 129.3, 129.2, 130.6 ms at 4.5e6.
 int64_t sweep_keep_bytes(const apcloud_ctx *c) {
     if (c->sweep_keep >= 0) return c->sweep_keep;
     const double l2 = (double)l2_bytes();
-    const double tot = SWEEP_ENTRY_BYTES * (double)c->ss_entries + SWEEP_ROW_BYTES * (double)c->n_tot;
-    return (tot <= 0.75 * l2 || tot > 2.0 * l2) ? INT64_MAX : (int64_t)(0.4 * l2);
+    const double tot = sweep_matrix_bytes(c) + SWEEP_ROW_BYTES * (double)c->n_tot;
+    return tot <= KEEP_ALL * l2 ? INT64_MAX : (int64_t)(KEEP_PART * l2);
 }
 
 namespace {
 
-// the same as the entry of the sorted matrix from which slices are hinted
-int64_t sweep_keep_entries(const apcloud_ctx *c) {
+// the same for block_sweep
+int sweep_keep_blocks(const apcloud_ctx *c) {
     const int64_t kb = sweep_keep_bytes(c);
-    return kb == INT64_MAX ? INT64_MAX : (int64_t)((double)kb / SWEEP_ENTRY_BYTES);
+    return block_keep(kb == INT64_MAX ? 1.0 : (double)kb / (sweep_matrix_bytes(c) + 1.0));
 }
 
 // dot kernels: 2 fat blocks per SM (few partials for the last block to sum)
@@ -2255,14 +1884,8 @@ struct Krylov {
     int pdeg = 1;                   // degree of the Jacobi-Neumann polynomial (1 = Jacobi)
     double omega = 1.0;
     const __half *hval = nullptr;   // FP16 copy of the matrix for the sweeps (FP32 vectors only)
-    // width-sorted FP16 sweep matrix (null: sweep on the ELL)
-    const int32_t *sperm = nullptr, *scol = nullptr;
-    const uint32_t *ssw = nullptr, *sso = nullptr;
-    const __half *sval = nullptr;
-    const float *sval32 = nullptr;  // FP32 values of the same copy (Arnoldi products)
-    const uint32_t *scol24 = nullptr;   // its chunk columns packed to 24 bits (sweeps), or null
-    int64_t skeep = INT64_MAX;          // sweeps: slices from this entry on are read with streaming loads
-    int64_t nslot = 0;
+    int blocks = -1;                // sweeps and products on the block-local copy of system `blocks` (-1: on the ELL)
+    int skeep = INT_MAX;            // how much of it the sweeps keep in L2 (block_sweep)
     T *z0 = nullptr, *z1 = nullptr, *t = nullptr;   // sweep ping-pong and cycle-end combination
     // flexible basis: Z_j = p(Ahat) v_j kept from step j, so that the cycle ends
     // with u += Z y instead of applying the polynomial to V y once more
@@ -2294,30 +1917,11 @@ T *poly_apply(apcloud_ctx *c, const T *val, const T *v, T *z_first, const Krylov
     for (int i = 1; i < K.pdeg; ++i) {
         if (last && i + 1 == K.pdeg) nxt = last;   // the last sweep writes where the caller keeps z
         if constexpr (sizeof(T) == 4) {
-            if (K.hval && K.sperm) {
+            if (K.blocks >= 0) {
                 // the first sweep follows the kernel that wrote v and the
                 // state; each later one follows a sweep (APC_LAUNCH_PDL)
-                const bool pdl = i > 1 && c->pdl_on;
-                const float *xc = (const float *)cur;
-                float *yn = (float *)nxt;
-                const GmresState *sc = (const GmresState *)st;
-                if (K.scol24 && K.skeep < c->ss_entries) {
-                    if (pdl) APC_SWEEP_BS_PDL(c, K.nslot, APC_SWEEPS24K, K.sperm, K.ssw, K.sso, K.scol, K.sval,
-                                              K.nslot, xc, yn, (const float *)v, sc, skip, K.scol24, K.skeep);
-                    else APC_SWEEP_BS(c, K.nslot, APC_SWEEPS24K, K.sperm, K.ssw, K.sso, K.scol, K.sval, K.nslot,
-                                      xc, yn, (const float *)v, sc, skip, K.scol24, K.skeep);
-                } else if (K.scol24) {
-                    if (pdl) APC_SWEEP_BS_PDL(c, K.nslot, APC_SWEEPS24, K.sperm, K.ssw, K.sso, K.scol, K.sval,
-                                              K.nslot, xc, yn, (const float *)v, sc, skip, K.scol24, K.skeep);
-                    else APC_SWEEP_BS(c, K.nslot, APC_SWEEPS24, K.sperm, K.ssw, K.sso, K.scol, K.sval, K.nslot,
-                                      xc, yn, (const float *)v, sc, skip, K.scol24, K.skeep);
-                } else {
-                    if (pdl) APC_SWEEP_BS_PDL(c, K.nslot, APC_SWEEPS, K.sperm, K.ssw, K.sso, K.scol, K.sval,
-                                              K.nslot, xc, yn, (const float *)v, sc, skip,
-                                              (const uint32_t *)nullptr, (int64_t)0);
-                    else APC_SWEEP_BS(c, K.nslot, APC_SWEEPS, K.sperm, K.ssw, K.sso, K.scol, K.sval, K.nslot,
-                                      xc, yn, (const float *)v, sc, skip, (const uint32_t *)nullptr, (int64_t)0);
-                }
+                block_sweep(c, K.blocks, (const float *)cur, (float *)nxt, (const float *)v, (const GmresState *)st,
+                            skip, K.skeep, i > 1 && c->pdl_on);
                 T *tmp = cur; cur = nxt; nxt = tmp;
                 continue;
             }
@@ -2335,23 +1939,10 @@ T *poly_apply(apcloud_ctx *c, const T *val, const T *v, T *z_first, const Krylov
     return cur;
 }
 
-// the restart residual r = b - Ahat u into K.wraw with beta = ||r||: on the
-// packed sorted FP32 copy when the cycle has it, else on the ELL
+// the restart residual r = b - Ahat u into K.wraw with beta = ||r||
 template <class T>
 void residual_launch(apcloud_ctx *c, const T *val, const Krylov<T> &K, const T *u, const T *b, GmresState *st) {
     const int n = c->n_tot;
-    if constexpr (sizeof(T) == 4) {
-        if (K.pdeg > 1 && K.sval32 && K.sperm && K.scol24) {
-            const int nb = resid_blocks(K.nslot);
-            if (c->spmv_unroll == 4)
-                APC_LAUNCH(c, K_SPMV, nb, RT, 0, k_resid_s<4>, K.sperm, K.ssw, K.sso, K.scol, K.sval32, K.scol24,
-                           K.nslot, (const float *)u, (float *)K.wraw, (const float *)b, st, K.partial);
-            else
-                APC_LAUNCH(c, K_SPMV, nb, RT, 0, k_resid_s<1>, K.sperm, K.ssw, K.sso, K.scol, K.sval32, K.scol24,
-                           K.nslot, (const float *)u, (float *)K.wraw, (const float *)b, st, K.partial);
-            return;
-        }
-    }
     const uint32_t *sw = ptr<uint32_t>(c->slice_w), *so = ptr<uint32_t>(c->slice_off);
     const int32_t *col = ptr<int32_t>(c->ell_col);
     APC_LAUNCH(c, K_SPMV, resid_blocks(n), RT, 0, (k_spmv<2, T>), sw, so, col, val, n, u, K.wraw, (T *)nullptr, b, st,
@@ -2359,20 +1950,14 @@ void residual_launch(apcloud_ctx *c, const T *val, const Krylov<T> &K, const T *
 }
 
 // w = Ahat z of a polynomial-preconditioned Arnoldi step (skipped once the
-// cycle is done): on the width-sorted FP32 copy when the sweeps use it, else
-// on the ELL
+// cycle is done): on the block-local copy when the sweeps use it, else on the
+// ELL
 template <class T>
 void arnoldi_product(apcloud_ctx *c, const T *val, const Krylov<T> &K, const T *z, GmresState *st, RowSkip skip) {
     const int n = c->n_tot;
     if constexpr (sizeof(T) == 4) {
-        if (K.sval32 && K.sperm && K.scol24) {
-            APC_SPMV_BS(c, K.nslot, APC_SPMVS24, K.sperm, K.ssw, K.sso, K.scol, K.sval32, K.nslot, (const float *)z,
-                        (float *)K.w, (const GmresState *)st, skip, K.scol24);
-            return;
-        }
-        if (K.sval32 && K.sperm) {
-            APC_SPMV_BS(c, K.nslot, APC_SPMVS, K.sperm, K.ssw, K.sso, K.scol, K.sval32, K.nslot, (const float *)z,
-                        (float *)K.w, (const GmresState *)st, skip, (const uint32_t *)nullptr);
+        if (K.blocks >= 0) {
+            block_product(c, K.blocks, (const float *)z, (float *)K.w, (const GmresState *)st, skip);
             return;
         }
     }
@@ -2623,8 +2208,12 @@ apcloud_status run_cycle(apcloud_ctx *c, const T *val, const T *b, T *u, const K
                            c->slice_w.p, c->slice_off.p, c->ell_col.p, K.skip.nbo, K.skip.bdone, K.tact,
                            K.mask ? K.mask->r2 : nullptr, K.bk ? K.bk->items : nullptr,
                            K.bk ? K.bk->H : nullptr, K.bk ? K.bk->done : nullptr,
-                           K.bk ? (const void *)(intptr_t)K.bk->nitems : nullptr, K.sperm, K.sval, K.scol, K.ssw,
-                           K.sso, K.Z, K.sval32, K.scol24};
+                           K.bk ? (const void *)(intptr_t)K.bk->nitems : nullptr, K.Z,
+                           (const void *)(intptr_t)(K.blocks + 1), K.blocks >= 0 ? c->bl_idx.p : nullptr,
+                           K.blocks >= 0 ? c->bl_hlist.p : nullptr, K.blocks >= 0 ? c->bl_off.p : nullptr,
+                           K.blocks >= 0 ? c->bl_len.p : nullptr, K.blocks >= 0 ? c->bl_hcnt.p : nullptr,
+                           K.blocks >= 0 ? (K.blocks ? c->bl_A.p : c->bl_B.p) : nullptr,
+                           K.blocks >= 0 ? (K.blocks ? c->bl_A32.p : c->bl_B32.p) : nullptr};
         static_assert(sizeof p <= sizeof key.p, "graph key holds every buffer address");
         for (size_t i = 0; i < sizeof p / sizeof p[0]; ++i) key.p[i] = p[i];
         GraphEntry *g = find_graph(c, key);
@@ -2696,9 +2285,8 @@ apcloud_status gmres_core(apcloud_ctx *c, const T *val, const T *b, T *u, double
             const double sweeps = (K.pdeg <= 1 || K.ilu) ? 0.0 : (double)(K.pdeg - 1) * (je + (K.Z ? 0 : 1));
             const double prods = je + 1.0;
             const double sb = K.hval ? 2.0 : vb;
-            const double cb = K.scol24 ? 3.0 : 4.0;   // column bytes per entry read by a sweep
-            // Arnoldi products and the restart residual (24-bit columns on the packed sorted copy)
-            const double pcb = (K.pdeg > 1 && K.sval32 && K.scol24) ? 3.0 : 4.0;
+            const double cb = K.blocks >= 0 ? 2.0 : 4.0;   // index bytes per entry of a sweep or product
+            const double pcb = K.blocks >= 0 ? (2.0 * je + 4.0) / prods : 4.0;   // the residual's are 4
             account(c, K_SPMV, ((vb + pcb) * nnz + 2.0 * vb * dn) * prods, 2.0 * nnz * prods);
             account(c, K_SWEEP, ((sb + cb) * nnz + 3.0 * vb * dn) * sweeps, 2.0 * nnz * sweeps);
         }
@@ -2926,16 +2514,13 @@ apcloud_status gmres_solve(apcloud_ctx *c, int which, const double *b, double *x
             K.pdeg = c->P.poly_degree;
             K.omega = c->P.poly_omega;
             K.hval = ptr<__half>(which ? c->ell_A16 : c->ell_B16);
-            if (c->ss_ok && c->sweep_sorted) {
-                K.sperm = ptr<int32_t>(c->ss_perm);
-                K.ssw = ptr<uint32_t>(c->ss_w);
-                K.sso = ptr<uint32_t>(c->ss_o);
-                K.scol = ptr<int32_t>(c->ss_col);
-                K.sval = ptr<__half>(which ? c->ss_A : c->ss_B);
-                K.sval32 = ptr<float>(which ? c->ss_A32 : c->ss_B32);
-                if (c->ss_col24_ok) K.scol24 = ptr<uint32_t>(c->ss_col24);
-                K.skeep = sweep_keep_entries(c);
-                K.nslot = (int64_t)div_up(c->n_tot, 256) * 256;
+            if (c->sweep_sorted) {
+                // systems meant for the resident solve have no copy yet: this one did not fit
+                if (!c->bl_tried && c->bl_chunks > 0) APC_TRY(build_blocks(c));
+                if (c->bl_ok) {
+                    K.blocks = which;
+                    K.skeep = sweep_keep_blocks(c);
+                }
             }
             K.z0 = ensure<float>(c, c->pz0, ldv + 1);
             K.z1 = ensure<float>(c, c->pz1, ldv + 1);
@@ -3021,8 +2606,8 @@ apcloud_status tune_spmv(apcloud_ctx *c, double *ms_out) {
     const int sizes[4] = {64, 128, 256, 512}, unrolls[2] = {1, 4};
     const int saved = c->spmv_bs, saved_u = c->spmv_unroll, saved_s = c->sweep_sorted;
     int pick = saved, pick_u = saved_u, pick_s = saved_s;
-    // the width-sorted sweep matrix is a third dimension when it exists
-    const int nvar = (mixed && c->P.poly_degree > 1 && c->ss_ok) ? 16 : 8;
+    // the block-local copy is a third dimension
+    const int nvar = (mixed && c->P.poly_degree > 1) ? 16 : 8;
     cudaEvent_t e0, e1;
     APC_CUDA(c, cudaEventCreate(&e0));
     APC_CUDA(c, cudaEventCreate(&e1));

@@ -998,13 +998,17 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     APC_CUDA(c, cudaMemsetAsync(small + 6, 0, sizeof(uint32_t), c->s));
     APC_LAUNCH(c, K_ELL, div_up(nsl, 8), 256, 0, k_slice_width, msz, n, nt, nsl, sw, small + 6);
     APC_TRY(scan_u32(c, sw, so, nsl, small + 5));
-    // the width-sorted copy's slices too, so that one read gives every size
-    if (c->P.precision == 1) APC_TRY(rank_sorted_sweep(c, small + 7));
-    uint32_t tot[3];   // ELL columns, stencil sizes, sorted columns
+    // the block-local copy's size too, so that one read gives every size; systems
+    // the resident solve takes do not need the copy
+    c->ell_entries = 0;
+    c->bl_ok = c->bl_tried = false;
+    const bool blocks = c->P.precision == 1 && c->P.poly_degree > 1;
+    if (blocks) APC_TRY(count_blocks(c, small + 7));
+    uint32_t tot[3];   // ELL columns, stencil sizes, chunks
     APC_TRY(read_back(c, tot, small + 5, sizeof tot));
     c->ell_entries = (int64_t)tot[0] * 32;
     c->sum_m = tot[1];
-    c->ss_entries = c->P.precision == 1 ? (int64_t)tot[2] * 32 : 0;
+    c->bl_chunks = blocks ? tot[2] : 0;
     // per node: offsets and weights in (28 B per neighbour), Laplacian row and
     // 9 x m operator out (80 B per neighbour); two 9-column Gram products,
     // three triangular solves per row and two 9x9 factorizations
@@ -1022,7 +1026,7 @@ apcloud_status build_stencils(apcloud_ctx *c) {
         if (!fA || !fB || !hA || !hB) return APCLOUD_E_NOMEM;
         APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_f32, (const double *)vA,
                    (const double *)vB, c->ell_entries, fA, fB, hA, hB);
-        APC_TRY(fill_sorted_sweep(c));
+        if (blocks && !resident_ok(c, 1)) APC_TRY(build_blocks(c));
     }
     return cuda_check(c, cudaGetLastError(), "ell");
 }
@@ -1093,150 +1097,8 @@ apcloud_status refresh_lowp(apcloud_ctx *c) {
     APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_f32, (const double *)ptr<double>(c->ell_A),
                (const double *)ptr<double>(c->ell_B), c->ell_entries, ptr<float>(c->ell_A32), ptr<float>(c->ell_B32),
                ptr<__half>(c->ell_A16), ptr<__half>(c->ell_B16));
-    APC_TRY(fill_sorted_sweep(c));
+    if (c->bl_tried) APC_TRY(build_blocks(c));
     return cuda_check(c, cudaGetLastError(), "refresh_lowp");
-}
-
-namespace {
-
-constexpr int SS_WIN = 256;   // rows per sorting window (8 slices)
-
-// one block per window: rank the window's rows by stored width (descending,
-// ties by row index), perm[slot] = row (-1 past the last row), and the width
-// of each of the window's 8 slices
-__global__ void __launch_bounds__(SS_WIN) k_ss_rank(const int32_t *__restrict__ msz, int n_int, int n_tot,
-                                                  int32_t *__restrict__ perm, uint32_t *__restrict__ w) {
-    __shared__ int wd[SS_WIN];
-    __shared__ int sorted_w[SS_WIN];
-    const int base = blockIdx.x * SS_WIN, t = threadIdx.x, r = base + t;
-    const int my = r < n_int ? msz[r] + 1 : (r < n_tot ? 1 : -1);
-    wd[t] = my;
-    __syncthreads();
-    int rank = 0;
-    for (int k = 0; k < SS_WIN; ++k) {
-        const int o = wd[k];
-        rank += (o > my) || (o == my && k < t);
-    }
-    perm[base + rank] = my >= 0 ? r : -1;
-    sorted_w[rank] = my > 0 ? my : 0;
-    __syncthreads();
-    if ((t & 31) == 0) w[blockIdx.x * (SS_WIN / 32) + (t >> 5)] = (uint32_t)sorted_w[t];   // max of the slice
-}
-
-// entry k of lane `lane` in a sorted slice of width w starting at entry sb:
-// 4-entry chunks lane-major for the first 4 * floor(w / 4) columns, the rest
-// slice-major
-__device__ __forceinline__ int64_t ss_slot(int64_t sb, int w, int k, int lane) {
-    const int kf = w & ~3;
-    return (k < kf) ? sb + (int64_t)(k >> 2) * 128 + lane * 4 + (k & 3)
-                    : sb + (int64_t)kf * 32 + (int64_t)(k - kf) * 32 + lane;
-}
-
-// copy every row's stored entries (in their order) into its slot of the sorted layout
-__global__ void k_ss_fill(const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff,
-                          const int32_t *__restrict__ col, const __half *__restrict__ hA, const __half *__restrict__ hB,
-                          const float *__restrict__ fA, const float *__restrict__ fB,
-                          const int32_t *__restrict__ perm, const uint32_t *__restrict__ w2,
-                          const uint32_t *__restrict__ o2, int64_t nslot, int32_t *__restrict__ col2,
-                          __half *__restrict__ A2, __half *__restrict__ B2, float *__restrict__ A4,
-                          float *__restrict__ B4, uint32_t *__restrict__ col24) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nslot) return;
-    const int sl2 = (int)(s >> 5), lane2 = (int)(s & 31);
-    const int64_t b2 = (int64_t)o2[sl2] * 32;
-    const int wid2 = (int)w2[sl2];
-    const int r = perm[s];
-    int k = 0;
-    if (r >= 0) {
-        const int sl = r >> 5, lane = r & 31;
-        const int w = (int)sw[sl];
-        const int64_t base = (int64_t)soff[sl] * 32 + lane;
-        for (; k < wid2 && k < w; ++k) {
-            const int64_t e = base + (int64_t)k * 32, q = ss_slot(b2, wid2, k, lane2);
-            col2[q] = col[e];
-            A2[q] = hA[e];
-            B2[q] = hB[e];
-            A4[q] = fA[e];
-            B4[q] = fB[e];
-        }
-    }
-    for (; k < wid2; ++k) {   // padding: the row itself (or row 0) with value 0
-        const int64_t q = ss_slot(b2, wid2, k, lane2);
-        col2[q] = r >= 0 ? r : 0;
-        A2[q] = __float2half(0.f);
-        B2[q] = __float2half(0.f);
-        A4[q] = 0.f;
-        B4[q] = 0.f;
-    }
-    if (col24) {
-        // the columns of the 4-entry chunks again, 24 bits each: a chunk's four
-        // columns in three words, word p of lane l at 24 o + 96 j + 32 p + l
-        const int64_t pw = (int64_t)o2[sl2] * 24 + lane2;
-        for (int j = 0; j < (wid2 >> 2); ++j) {
-            uint32_t cc[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) cc[t] = (uint32_t)col2[ss_slot(b2, wid2, 4 * j + t, lane2)];
-            col24[pw + (int64_t)j * 96] = cc[0] | (cc[1] << 24);
-            col24[pw + (int64_t)j * 96 + 32] = (cc[1] >> 8) | (cc[2] << 16);
-            col24[pw + (int64_t)j * 96 + 64] = (cc[2] >> 16) | (cc[3] << 8);
-        }
-    }
-}
-
-}  // namespace
-
-// The FP16 preconditioner sweeps stream the whole matrix 15 times per Arnoldi
-// step; in 32-row slices of consecutive rows the slice width is that of its
-// widest stencil and 14% of the stored entries are padding.  This copy orders
-// the rows of every 256-row window by stored width (SELL-C-sigma, C = 32,
-// sigma = 256): slices then hold rows of nearly equal width.  Within a slice
-// the entries are grouped in 4-entry chunks per row (16-byte column loads),
-// the last width % 4 columns as in the ELL.  Each row keeps its entries in
-// their stored order, so a sweep on this copy gives the same bits as on the
-// ELL.  The copy carries the FP16 values of the sweeps and the FP32 values of
-// the Arnoldi products (also the same bits as the FP32 ELL product), and for
-// the sweeps the chunks' columns packed to 24 bits (while n < 2^24): 20
-// instead of 24 bytes per 4-entry chunk of a bandwidth-bound stream.
-// Ranks and slice widths (their total to *d_total), then the copy itself once
-// ss_entries is known; a refresh of the values needs the second part only.
-apcloud_status rank_sorted_sweep(apcloud_ctx *c, uint32_t *d_total) {
-    c->ss_ok = false;
-    const int n = c->n_tot;
-    if (n == 0) return APCLOUD_OK;
-    const int nwin = div_up(n, SS_WIN);
-    const int64_t nslot = (int64_t)nwin * SS_WIN;
-    const int nsl2 = (int)(nslot / 32);
-    int32_t *perm = ensure<int32_t>(c, c->ss_perm, nslot);
-    uint32_t *w2 = ensure<uint32_t>(c, c->ss_w, nsl2 + 1), *o2 = ensure<uint32_t>(c, c->ss_o, nsl2 + 1);
-    if (!perm || !w2 || !o2) return APCLOUD_E_NOMEM;
-    APC_LAUNCH(c, K_ELL, nwin, SS_WIN, 0, k_ss_rank, (const int32_t *)ptr<int32_t>(c->msz), c->n_int, n, perm, w2);
-    return scan_u32(c, w2, o2, nsl2, d_total);
-}
-
-apcloud_status fill_sorted_sweep(apcloud_ctx *c) {
-    const int n = c->n_tot;
-    if (n == 0) return APCLOUD_OK;
-    const int64_t nslot = (int64_t)div_up(n, SS_WIN) * SS_WIN;
-    const int32_t *perm = ptr<int32_t>(c->ss_perm);
-    const uint32_t *w2 = ptr<uint32_t>(c->ss_w), *o2 = ptr<uint32_t>(c->ss_o);
-    int32_t *col2 = ensure<int32_t>(c, c->ss_col, c->ss_entries + 1);
-    __half *A2 = ensure<__half>(c, c->ss_A, c->ss_entries + 1), *B2 = ensure<__half>(c, c->ss_B, c->ss_entries + 1);
-    float *A4 = ensure<float>(c, c->ss_A32, c->ss_entries + 1), *B4 = ensure<float>(c, c->ss_B32, c->ss_entries + 1);
-    if (!col2 || !A2 || !B2 || !A4 || !B4) return APCLOUD_E_NOMEM;
-    // 24-bit columns for the sweeps while every node index fits
-    uint32_t *col24 = nullptr;
-    c->ss_col24_ok = false;
-    if (n < (1 << 24)) {
-        col24 = ensure<uint32_t>(c, c->ss_col24, c->ss_entries / 4 * 3 + 1);
-        if (!col24) return APCLOUD_E_NOMEM;
-        c->ss_col24_ok = true;
-    }
-    APC_LAUNCH(c, K_ELL, div_up(nslot, 256), 256, 0, k_ss_fill, (const uint32_t *)ptr<uint32_t>(c->slice_w),
-               (const uint32_t *)ptr<uint32_t>(c->slice_off), (const int32_t *)ptr<int32_t>(c->ell_col),
-               (const __half *)ptr<__half>(c->ell_A16), (const __half *)ptr<__half>(c->ell_B16),
-               (const float *)ptr<float>(c->ell_A32), (const float *)ptr<float>(c->ell_B32), perm, w2, o2, nslot, col2, A2, B2, A4, B4, col24);
-    c->ss_ok = true;
-    return cuda_check(c, cudaGetLastError(), "sorted sweep matrix");
 }
 
 }  // namespace apc
