@@ -26,7 +26,12 @@ constexpr int NF = 12;  // per-node record: phi, 9 derivatives, 2 pad
 // words: phi and the node centre (FP64, words 0-7), gradient and Hessian
 // fx fy fz fxx fxy fxz fyy fyz fzz (FP32, words 8-16), pad
 constexpr int NF32 = 20;
+constexpr int GT = 256;  // threads of the mixed form's particle pass
 
+// Ten FP64 instructions per stencil entry keep the FP64 pipe busy four fifths of
+// the time; the operator's 72 bytes per entry take about as long as it leaves.
+// Two entries per step put the second's loads behind the first's arithmetic:
+// 141 us for 265186 nodes (150 one at a time, 183 with four: registers).
 __global__ void k_derivs(const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff,
                          const int32_t *__restrict__ col, const double *__restrict__ D, int64_t dstride,
                          const double *__restrict__ phi, int n_int, double *__restrict__ nf,
@@ -41,6 +46,7 @@ __global__ void k_derivs(const uint32_t *__restrict__ sw, const uint32_t *__rest
     double acc[NCOL];
 #pragma unroll
     for (int r = 0; r < NCOL; ++r) acc[r] = 0.0;
+#pragma unroll 2
     for (int k = 1; k < w; ++k) {
         const int cj = col[base + (int64_t)k * 32];
         const double diff = phi[cj] - p0;
@@ -91,48 +97,77 @@ __device__ __forceinline__ void taylor(const double *__restrict__ nf, int j, dou
     ez = g2 + hr2;
 }
 
-template <bool F32>
 __global__ void __launch_bounds__(256) k_gather_leaf(
     const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z, int64_t n,
     double lo0, double lo1, double lo2, double unit, const int32_t *__restrict__ pleaf, const int4 *__restrict__ ic,
-    const double *__restrict__ nf, const float *__restrict__ nf32, double *__restrict__ php, double *__restrict__ ex,
-    double *__restrict__ ey, double *__restrict__ ez) {
+    const double *__restrict__ nf, double *__restrict__ php, double *__restrict__ ex, double *__restrict__ ey,
+    double *__restrict__ ez) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int j = __ldcs(pleaf + i);
     const double p0 = __ldcs(x + i), p1 = __ldcs(y + i), p2 = __ldcs(z + i);
     double v, gx, gy, gz;
-    if (F32) {
-        // the mixed form: corrections (g.r, H r, r.H.r) in FP32 around the FP64
-        // node potential, from the compact record; its node derivatives carry
-        // FP32 accuracy already (FP32 stencils).  The pass stays off the slow
-        // FP64 pipe but for the offsets from the centre and the potential's
-        // add: the seven double/float conversions run on the integer pipe
-        const double2 *c2 = reinterpret_cast<const double2 *>(nf32 + (int64_t)j * NF32);
-        const float4 *f4 = reinterpret_cast<const float4 *>(nf32 + (int64_t)j * NF32 + 8);
-        const double2 pc = c2[0], cc = c2[1];
-        const float4 u = f4[0], w = f4[1], t = f4[2];
-        const float r0 = f64_to_f32_int(p0 - pc.y), r1 = f64_to_f32_int(p1 - cc.x), r2 = f64_to_f32_int(p2 - cc.y);
-        // u = (fx, fy, fz, fxx), w = (fxy, fxz, fyy, fyz), t.x = fzz
-        const float hr0 = fmaf(w.y, r2, fmaf(w.x, r1, u.w * r0));
-        const float hr1 = fmaf(w.w, r2, fmaf(w.z, r1, w.x * r0));
-        const float hr2 = fmaf(t.x, r2, fmaf(w.w, r1, w.y * r0));
-        const float corr = fmaf(u.z, r2, fmaf(u.y, r1, u.x * r0)) + 0.5f * fmaf(r2, hr2, fmaf(r1, hr1, r0 * hr0));
-        v = pc.x + f32_to_f64_int(corr);
-        gx = f32_to_f64_int(u.x + hr0);
-        gy = f32_to_f64_int(u.y + hr1);
-        gz = f32_to_f64_int(u.z + hr2);
-    } else {
-        const int4 q = ic[j];
-        const double r0 = p0 - __dadd_rn(lo0, __dmul_rn((double)q.x, unit));
-        const double r1 = p1 - __dadd_rn(lo1, __dmul_rn((double)q.y, unit));
-        const double r2 = p2 - __dadd_rn(lo2, __dmul_rn((double)q.z, unit));
-        taylor(nf, j, r0, r1, r2, v, gx, gy, gz);
-    }
+    const int4 q = ic[j];
+    const double r0 = p0 - __dadd_rn(lo0, __dmul_rn((double)q.x, unit));
+    const double r1 = p1 - __dadd_rn(lo1, __dmul_rn((double)q.y, unit));
+    const double r2 = p2 - __dadd_rn(lo2, __dmul_rn((double)q.z, unit));
+    taylor(nf, j, r0, r1, r2, v, gx, gy, gz);
     if (php) __stcs(php + i, v);
     if (ex) __stcs(ex + i, gx);
     if (ey) __stcs(ey + i, gy);
     if (ez) __stcs(ez + i, gz);
+}
+
+// The mixed form: corrections (g.r, H r, r.H.r) in FP32 around the FP64 node
+// potential, from the compact record; its node derivatives carry FP32 accuracy
+// already (FP32 stencils).  The pass stays off the slow FP64 pipe but for the
+// offsets from the centre and the potential's add: the seven double/float
+// conversions run on the integer pipe.
+//
+// Particles come in any order, so a record per lane costs five loads of 32
+// different lines each, 160 L1 look-ups a warp: 312 us at 2e7 particles, twice
+// what the bytes take.  Here a warp fetches its 32 records together, the five
+// 16-byte parts of a record by neighbouring lanes (a third of the look-ups),
+// and hands them over through shared memory (rows of 80 bytes: no bank
+// conflicts): 297 us.  Records of 96 or 128 bytes change nothing, loads past L1
+// (358 us: a tenth of the leaves hold most particles) and asynchronous copies
+// into shared memory (310 us) lose.
+__global__ void __launch_bounds__(GT) k_gather_leaf32(
+    const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z, int64_t n,
+    const int32_t *__restrict__ pleaf, const float *__restrict__ nf32, double *__restrict__ php,
+    double *__restrict__ ex, double *__restrict__ ey, double *__restrict__ ez) {
+    __shared__ float4 rec[GT * 5];
+    const int64_t i = (int64_t)blockIdx.x * GT + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const bool live = i < n;
+    const int j = live ? __ldcs(pleaf + i) : 0;
+    const double p0 = live ? __ldcs(x + i) : 0.0, p1 = live ? __ldcs(y + i) : 0.0, p2 = live ? __ldcs(z + i) : 0.0;
+    float4 *mine = rec + (threadIdx.x - lane) * 5;
+    float4 part[5];
+#pragma unroll
+    for (int t = 0; t < 5; ++t) {
+        const int e = t * 32 + lane, o = e / 5;
+        const int jo = __shfl_sync(0xFFFFFFFFu, j, o);
+        part[t] = __ldg(reinterpret_cast<const float4 *>(nf32 + (int64_t)jo * NF32) + (e - o * 5));
+    }
+#pragma unroll
+    for (int t = 0; t < 5; ++t) mine[t * 32 + lane] = part[t];
+    __syncwarp();
+    if (!live) return;
+    const double2 pc = *reinterpret_cast<const double2 *>(mine + lane * 5);
+    const double2 cc = *reinterpret_cast<const double2 *>(mine + lane * 5 + 1);
+    const float4 u = mine[lane * 5 + 2], w = mine[lane * 5 + 3];
+    const float fzz = mine[lane * 5 + 4].x;
+    const float r0 = f64_to_f32_int(p0 - pc.y), r1 = f64_to_f32_int(p1 - cc.x), r2 = f64_to_f32_int(p2 - cc.y);
+    // u = (fx, fy, fz, fxx), w = (fxy, fxz, fyy, fyz)
+    const float hr0 = fmaf(w.y, r2, fmaf(w.x, r1, u.w * r0));
+    const float hr1 = fmaf(w.w, r2, fmaf(w.z, r1, w.x * r0));
+    const float hr2 = fmaf(fzz, r2, fmaf(w.w, r1, w.y * r0));
+    const float corr = fmaf(u.z, r2, fmaf(u.y, r1, u.x * r0)) + 0.5f * fmaf(r2, hr2, fmaf(r1, hr1, r0 * hr0));
+    if (php) __stcs(php + i, pc.x + f32_to_f64_int(corr));
+    if (ex) __stcs(ex + i, f32_to_f64_int(u.x + hr0));
+    if (ey) __stcs(ey + i, f32_to_f64_int(u.y + hr1));
+    if (ez) __stcs(ez + i, f32_to_f64_int(u.z + hr2));
 }
 
 __global__ void k_gather(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
@@ -188,13 +223,12 @@ apcloud_status gather_field(apcloud_ctx *c, double *phi_p, double *ex, double *e
                ptr<int32_t>(c->ell_col), ptr<double>(c->D), dstride, ptr<double>(c->phi), n, nf,
                ptr<int4>(c->node_ic), c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, nf32);
     if (mixed)
-        APC_LAUNCH(c, K_GATHER, div_up(c->N, 256), 256, 0, k_gather_leaf<true>, c->px, c->py, c->pz, c->N,
-                   c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, (const int32_t *)ptr<int32_t>(c->pleaf),
-                   ptr<int4>(c->node_ic), (const double *)nf, (const float *)nf32, phi_p, ex, ey, ez);
+        APC_LAUNCH(c, K_GATHER, div_up(c->N, GT), GT, 0, k_gather_leaf32, c->px, c->py, c->pz, c->N,
+                   (const int32_t *)ptr<int32_t>(c->pleaf), (const float *)nf32, phi_p, ex, ey, ez);
     else
-        APC_LAUNCH(c, K_GATHER, div_up(c->N, 256), 256, 0, k_gather_leaf<false>, c->px, c->py, c->pz, c->N,
+        APC_LAUNCH(c, K_GATHER, div_up(c->N, 256), 256, 0, k_gather_leaf, c->px, c->py, c->pz, c->N,
                    c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, (const int32_t *)ptr<int32_t>(c->pleaf),
-                   ptr<int4>(c->node_ic), (const double *)nf, (const float *)nullptr, phi_p, ex, ey, ez);
+                   ptr<int4>(c->node_ic), (const double *)nf, phi_p, ex, ey, ez);
     // node pass: operator (72 B), column (4 B) and neighbour value (8 B) per
     // stencil entry plus the 96 B record (and the 80 B compact record of the
     // mixed form); particle pass: leaf index and position in (28 B), phi and E
