@@ -2,21 +2,21 @@
 // search of Section 4.3, and assembly of the density matrix B and the
 // Poisson matrix A of Section 3.2 in sliced ELL.
 //
-// One warp per node.  The warp grows the k-ring (k = 2..ring_max) by BFS over
+// One warp per node grows the k-ring (k = 2..ring_max) by BFS over
 // the face adjacency with the candidate set in shared memory, sorts the
-// candidates once by (exact integer squared distance, node index), takes the
+// candidates once by (exact integer squared distance, node index) and takes the
 // octant picks, the nearest fill and the ties as prefix counts (ballots) along
-// that order, and builds the weighted scaled Vandermonde W V0 with one lane per
-// neighbour (lane j = row j, m <= 32).  The least-squares operator
-// P = (W V0)^+ W is formed by Cholesky QR applied twice (CholeskyQR2): the
-// 9x9 Gram matrices come from shared memory and are factored by the whole
-// warp, Q = A R^-1 is lane-local, and column j of P is R^-1 q_j^T W_j, again
-// lane-local.  This replaces the column-by-column Householder reductions of a
-// CPU QR (9 dependent cross-lane reductions) with two Gram products, two
-// 9-step warp factorisations and lane-private triangular solves.
+// that order.  The least-squares operator P = (W V0)^+ W of the weighted scaled
+// Vandermonde W V0 (a row per neighbour, m <= 32) is formed by Cholesky QR
+// applied twice (CholeskyQR2): two 9x9 Gram matrices, their factorisations, and
+// triangular solves row by row, column j of P being R^-1 q_j^T W_j.  In FP64 the
+// same warp goes on with it, one lane per neighbour; in the mixed form a second
+// kernel does, four nodes per warp (k_wls32), and the few nodes that its FP32
+// factorisation cannot certify start again in a third (the list kernel).
 #include <cuda_fp16.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "fpconv.cuh"
 #include "internal.cuh"
@@ -30,7 +30,7 @@ constexpr int ASTR = NCOL;      // row stride of the staged Vandermonde
 // MC candidate slots: MAXC_FAST in the kernel over all nodes, MAXC in the one
 // that redoes the nodes whose rings outgrew them
 template <int MC>
-struct __align__(16) WarpSmemT {
+struct __align__(16) SelectSmemT {
     int32_t cand[MC];
     long long d2[MC];   // hash set of the candidates (2 MC ints), then their rank keys, then squared distances
     uint16_t srt[MC];   // candidate slots in (d2, index) order
@@ -38,6 +38,9 @@ struct __align__(16) WarpSmemT {
     uint8_t pick[MC];   // octant picks, by sorted position
     int32_t sel[MMAX];
     long long seld2[MMAX];
+};
+template <int MC>
+struct __align__(16) WarpSmemT : SelectSmemT<MC> {
     double A[MMAX * ASTR];
     double G[48];
     double R1[NCOL * NCOL];
@@ -45,18 +48,8 @@ struct __align__(16) WarpSmemT {
     double Ri1[NCOL], Ri2[NCOL];   // reciprocal diagonals of R1, R2
 };
 
-
 __device__ __forceinline__ bool key_less(long long da, int ia, long long db, int ib) {
     return da < db || (da == db && ia < ib);
-}
-
-__device__ __forceinline__ long long warp_max_ll(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        long long t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = t > v ? t : v;
-    }
-    return v;
 }
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -113,17 +106,21 @@ __device__ bool cholesky_warp(T *G, T *R, T *Ri, const GramOwn &o, int lane) {
     return true;
 }
 
-// FP32 Cholesky of the packed Gram matrix computed by every lane at once in
-// registers (the 45 entries are broadcast from shared memory, the nine pivot
-// steps run without any exchange between lanes); lane 0 stores R and the
-// reciprocal pivots for the triangular solves.  The reciprocal square root of
-// each pivot gives both R_kk = g * rsqrt(g) and 1 / R_kk.  Returns false on a
-// non-positive pivot, the same decision in every lane.
-__device__ bool cholesky_regs(const float *G, float *R, float *Ri, int lane) {
-    float g[45];
+// FP32 Cholesky G = R^T R of the packed Gram matrix, computed by every lane at
+// once in registers (the 45 entries are broadcast from shared memory, the nine
+// pivot steps run without any exchange between lanes): g becomes R, rd the
+// reciprocals of its diagonal.  The reciprocal square root of each pivot gives
+// both R_kk = g * rsqrt(g) and 1 / R_kk.  Returns false on a non-positive pivot,
+// the same decision in every lane.
+__device__ __forceinline__ bool cholesky_regs(const float *G, float (&g)[48], float (&rd)[NCOL]) {
 #pragma unroll
-    for (int e = 0; e < 45; ++e) g[e] = G[e];
-    float rd[NCOL];
+    for (int e = 0; e < 12; ++e) {
+        const float4 v = reinterpret_cast<const float4 *>(G)[e];
+        g[4 * e] = v.x;
+        g[4 * e + 1] = v.y;
+        g[4 * e + 2] = v.z;
+        g[4 * e + 3] = v.w;
+    }
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < NCOL; ++k) {
@@ -139,17 +136,7 @@ __device__ bool cholesky_regs(const float *G, float *R, float *Ri, int lane) {
 #pragma unroll
             for (int j = i; j < NCOL; ++j) g[pk_idx(i, j)] = fmaf(-g[pk_idx(k, i)], g[pk_idx(k, j)], g[pk_idx(i, j)]);
     }
-    if (!ok) return false;
-    if (lane == 0) {
-#pragma unroll
-        for (int a = 0; a < NCOL; ++a) {
-            Ri[a] = rd[a];
-#pragma unroll
-            for (int b = a; b < NCOL; ++b) R[a * NCOL + b] = g[pk_idx(a, b)];
-        }
-    }
-    __syncwarp();
-    return true;
+    return ok;
 }
 
 // solve q R = a for the row vector q (R upper), in place on v
@@ -176,46 +163,116 @@ __device__ __forceinline__ void col_solve_upper(const T *R, const T *Ri, T *v) {
     }
 }
 
-// Gram matrix of the m staged rows, the lane's two owned entries accumulated
-// side by side
-template <class T>
-__device__ __forceinline__ void gram(const T *A, int m, T *G, const GramOwn &o, int lane) {
-    T s1 = (T)0, s2 = (T)0;
-    for (int j = 0; j < m; ++j) {
-        const T *r = A + j * ASTR;
-        s1 = fma(r[o.a1], r[o.b1], s1);
-        s2 = fma(r[o.a2], r[o.b2], s2);
+// solve q R = a for the row vector q (R upper, packed), in place on v
+__device__ __forceinline__ void row_solve_upper(const float (&R)[48], const float (&Ri)[NCOL], float *v) {
+#pragma unroll
+    for (int c = 0; c < NCOL; ++c) {
+        float s = v[c];
+#pragma unroll
+        for (int k = 0; k < c; ++k) s -= v[k] * R[pk_idx(k, c)];
+        v[c] = s * Ri[c];
+    }
+}
+
+// solve R z = v for the column vector z (R upper, packed), in place
+__device__ __forceinline__ void col_solve_upper(const float (&R)[48], const float (&Ri)[NCOL], float *v) {
+#pragma unroll
+    for (int c = NCOL - 1; c >= 0; --c) {
+        float s = v[c];
+#pragma unroll
+        for (int k = c + 1; k < NCOL; ++k) s -= R[pk_idx(c, k)] * v[k];
+        v[c] = s * Ri[c];
+    }
+}
+
+// col_solve_upper in the place of the first (open) and the second (tail) of two
+// solves one after another, with a stop between them: the first entry is handed
+// over before its division by R_00 (rd00 its reciprocal), which the second
+// rounds together with the first term, as the compiler contracts the two
+// written in one piece (wls_column_f32).
+__device__ __forceinline__ void col_solve_rows(const float (&R)[48], const float (&Ri)[NCOL], float *v) {
+#pragma unroll
+    for (int c = NCOL - 1; c > 0; --c) {
+        float s = v[c];
+#pragma unroll
+        for (int k = c + 1; k < NCOL; ++k) s -= R[pk_idx(c, k)] * v[k];
+        v[c] = s * Ri[c];
+    }
+}
+__device__ __forceinline__ void col_solve_open(const float (&R)[48], const float (&Ri)[NCOL], float *v) {
+    col_solve_rows(R, Ri, v);
+#pragma unroll
+    for (int k = 1; k < NCOL; ++k) v[0] -= R[pk_idx(0, k)] * v[k];
+}
+__device__ __forceinline__ void col_solve_tail(const float (&R)[48], const float (&Ri)[NCOL], float *v, float rd00) {
+    col_solve_rows(R, Ri, v);
+    float s = __fmaf_rn(v[0], rd00, -__fmul_rn(R[pk_idx(0, 1)], v[1]));
+#pragma unroll
+    for (int k = 2; k < NCOL; ++k) s -= R[pk_idx(0, k)] * v[k];
+    v[0] = s * Ri[0];
+}
+
+// Gram matrix of the m rows staged by columns (entry e of row j at e * FSTR + j,
+// zeros in rows m to 31), the lane's two owned entries accumulated side by side
+// in row order, four rows to a load
+constexpr int FSTR = 36;
+__device__ __forceinline__ void gram_f32(const float *A, int m, float *G, const GramOwn &o, int lane) {
+    float s1 = 0.f, s2 = 0.f;
+    const float *a1 = A + o.a1 * FSTR, *b1 = A + o.b1 * FSTR, *a2 = A + o.a2 * FSTR, *b2 = A + o.b2 * FSTR;
+    for (int j = 0; j < m; j += 4) {
+        const float4 p = *reinterpret_cast<const float4 *>(a1 + j), q = *reinterpret_cast<const float4 *>(b1 + j);
+        const float4 r = *reinterpret_cast<const float4 *>(a2 + j), t = *reinterpret_cast<const float4 *>(b2 + j);
+        s1 = fmaf(p.x, q.x, s1);
+        s2 = fmaf(r.x, t.x, s2);
+        s1 = fmaf(p.y, q.y, s1);
+        s2 = fmaf(r.y, t.y, s2);
+        s1 = fmaf(p.z, q.z, s1);
+        s2 = fmaf(r.z, t.z, s2);
+        s1 = fmaf(p.w, q.w, s1);
+        s2 = fmaf(r.w, t.w, s2);
     }
     G[lane] = s1;
     if (o.two) G[lane + 32] = s2;
 }
 
+// The FP32 column's constants: the weight's, and the least condition estimates
+// (min / max of |R_ii|) that it takes and that any column needs, each the least
+// FP32 number not below the FP64 one (r < the one exactly when r < the other).
+struct Fp32Args {
+    float ec, inv_1mec, rcond_min, rank_min;
+};
+float fp32_not_below(double v) {
+    const float f = (float)v;
+    return (double)f < v ? std::nextafter(f, INFINITY) : f;
+}
+
 // Weighted least-squares operator (Section 3.1) of the stencil staged in
 // W.sel / W.seld2, in FP32: rows of W V0 (Eq. regfd with the
 // normalized Gaussian weight), CholeskyQR2, and column `lane` of
-// P = (W V0)^+ W unscaled by h and h^2, returned in FP64.  Returns false when
+// P = (W V0)^+ W unscaled by h and h^2.  Returns false when
 // a Cholesky pivot fails; rratio = min |R_ii| / max |R_ii|.
+// Conversions to and from 64-bit types run on the narrow FP64 pipe: offsets
+// are 32-bit integers here, the squared distances too (in half cells of the
+// deepest level, unless they need more), and h takes the one FP64 product.
 template <class WS>
 __device__ bool wls_column_f32(WS &W, int m, int lane, const GramOwn &own, int4 c0, const int4 *__restrict__ ic,
-                           double unit, double ec, double inv_1mec, double (&qout)[NCOL], double &lapj,
-                           double &rratio) {
+                               double unit, const Fp32Args &fa, int d2_shift, float (&qout)[NCOL],
+                               float &lapj, float &rratio) {
     typedef float T;
     T *A = reinterpret_cast<T *>(W.A);
     T *G = reinterpret_cast<T *>(W.G);
     T *R1 = reinterpret_cast<T *>(W.R1);
-    T *R2 = reinterpret_cast<T *>(W.R2);
-    T *Ri1 = reinterpret_cast<T *>(W.Ri1);
-    T *Ri2 = reinterpret_cast<T *>(W.Ri2);
-    long long off[3] = {0, 0, 0};
-    long long mydist = 0, amax = 0;
+    int off[3] = {0, 0, 0};
+    int amax = 0;
+    unsigned long long mydist = 0;
     if (lane < m) {
         int4 q = ic[W.sel[lane]];
-        off[0] = (long long)q.x - c0.x; off[1] = (long long)q.y - c0.y; off[2] = (long long)q.z - c0.z;
-        mydist = W.seld2[lane];
-        for (int d = 0; d < 3; ++d) { long long a = off[d] < 0 ? -off[d] : off[d]; amax = a > amax ? a : amax; }
+        off[0] = q.x - c0.x; off[1] = q.y - c0.y; off[2] = q.z - c0.z;
+        mydist = (unsigned long long)W.seld2[lane] >> d2_shift;
+        for (int d = 0; d < 3; ++d) amax = max(amax, abs(off[d]));
     }
-    const long long hint = warp_max_ll(amax);
-    const long long r2max = W.seld2[m - 1];
+    const int hint = __reduce_max_sync(0xffffffffu, amax);
+    const unsigned long long r2max = (unsigned long long)W.seld2[m - 1] >> d2_shift;
     T wj = (T)0;
     {
         T row[NCOL];
@@ -224,8 +281,8 @@ __device__ bool wls_column_f32(WS &W, int m, int lane, const GramOwn &own, int4 
         if (lane < m) {
             // xi = dy / h with h = max |dy_d| (Section 3.1): exact integers, one rounding in T
             T xi0 = (T)off[0] / (T)hint, xi1 = (T)off[1] / (T)hint, xi2 = (T)off[2] / (T)hint;
-            T ratio = (T)mydist / (T)r2max;
-            wj = (expf(-ratio) - (T)ec) * (T)inv_1mec;
+            T ratio = (r2max >> 32) ? (T)mydist / (T)r2max : (T)(unsigned)mydist / (T)(unsigned)r2max;
+            wj = (expf(-ratio) - fa.ec) * fa.inv_1mec;
             const T half = (T)0.5;
             row[0] = xi0; row[1] = xi1; row[2] = xi2;
             row[3] = (half * xi0) * xi0;
@@ -238,57 +295,78 @@ __device__ bool wls_column_f32(WS &W, int m, int lane, const GramOwn &own, int4 
             for (int e = 0; e < NCOL; ++e) row[e] = wj * row[e];
         }
 #pragma unroll
-        for (int e = 0; e < NCOL; ++e) A[lane * ASTR + e] = row[e];
+        for (int e = 0; e < NCOL; ++e) A[e * FSTR + lane] = row[e];
     }
     __syncwarp();
-    gram<T>(A, m, G, own, lane);
+    gram_f32(A, m, G, own, lane);
     __syncwarp();
-    bool ok = cholesky_regs(G, R1, Ri1, lane);
+    // the factors stay in registers for the solves that follow them; the first,
+    // needed again at the end, waits in shared memory
+    T R[48], Ri[NCOL];
+    bool ok = cholesky_regs(G, R, Ri);
     T q[NCOL];
+    T dr[NCOL];   // diagonal of R1, then of R1 R2
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) dr[e] = R[pk_idx(e, e)];
     if (ok) {
-        if (lane < m) {
+        if (lane == 0) {
 #pragma unroll
-            for (int e = 0; e < NCOL; ++e) q[e] = A[lane * ASTR + e];
-            row_solve_upper<T>(R1, Ri1, q);
+            for (int e = 0; e < 12; ++e)
+                reinterpret_cast<float4 *>(R1)[e] = make_float4(R[4 * e], R[4 * e + 1], R[4 * e + 2], R[4 * e + 3]);
 #pragma unroll
-            for (int e = 0; e < NCOL; ++e) A[lane * ASTR + e] = q[e];
+            for (int e = 0; e < NCOL; ++e) R1[48 + e] = Ri[e];
         }
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) q[e] = A[e * FSTR + lane];   // zeros past the rows
+        row_solve_upper(R, Ri, q);
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) A[e * FSTR + lane] = q[e];
         __syncwarp();
-        gram<T>(A, m, G, own, lane);
+        gram_f32(A, m, G, own, lane);
         __syncwarp();
-        ok = cholesky_regs(G, R2, Ri2, lane);
+        ok = cholesky_regs(G, R, Ri);
     }
-    rratio = 0.0;
-    lapj = 0.0;
+    rratio = 0.f;
+    lapj = 0.f;
     if (!ok) return false;
     T dmin = (T)1e30, dmax = (T)0;
 #pragma unroll
     for (int e = 0; e < NCOL; ++e) {
-        T r = fabs(R1[e * NCOL + e] * R2[e * NCOL + e]);
+        T r = fabs(dr[e] * R[pk_idx(e, e)]);
         dmin = fmin(dmin, r);
         dmax = fmax(dmax, r);
     }
-    rratio = (double)(dmin / dmax);
+    rratio = dmin / dmax;
     // unscale rows by 1/h and 1/h^2 (h = max |dy_d|), in T
-    const T h = (T)((double)hint * unit);
+    const T h = (T)((double)hint * unit);   // hint < 2^23: exact in FP32
     const T ih = (T)1 / h, ih2 = ih * ih;
     if (lane < m) {
 #pragma unroll
-        for (int e = 0; e < NCOL; ++e) q[e] = A[lane * ASTR + e];
-        row_solve_upper<T>(R2, Ri2, q);
-        col_solve_upper<T>(R2, Ri2, q);
-        col_solve_upper<T>(R1, Ri1, q);
+        for (int e = 0; e < NCOL; ++e) q[e] = A[e * FSTR + lane];
+        row_solve_upper(R, Ri, q);
+        col_solve_upper(R, Ri, q);
+#pragma unroll
+        for (int e = 0; e < 12; ++e) {
+            const float4 v = reinterpret_cast<const float4 *>(R1)[e];
+            R[4 * e] = v.x;
+            R[4 * e + 1] = v.y;
+            R[4 * e + 2] = v.z;
+            R[4 * e + 3] = v.w;
+        }
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) Ri[e] = R1[48 + e];
+        col_solve_upper(R, Ri, q);
         T lj = (T)0;
 #pragma unroll
         for (int e = 0; e < NCOL; ++e) {
             const T v = (q[e] * wj) * (e < 3 ? ih : ih2);
-            qout[e] = (double)v;
+            qout[e] = v;
             if (e == 3 || e == 6 || e == 8) lj += v;
         }
-        lapj = (double)lj;
+        lapj = lj;
     } else {
 #pragma unroll
-        for (int e = 0; e < NCOL; ++e) qout[e] = 0.0;
+        for (int e = 0; e < NCOL; ++e) qout[e] = 0.f;
     }
     return true;
 }
@@ -496,27 +574,28 @@ __device__ __forceinline__ bool ring_insert(int *tab, int v) {
 }
 
 // SW warps (nodes) per block, one WarpSmemT<MC> each (and the block's
-// arrival count after them); the autotuner picks SW.  With MC = MAXC_FAST
-// (LIST false, every node): 6.6 KB of shared memory per warp and 32 warps per
-// SM at a register budget that spills part of the FP32 factorisation; a node
-// whose ring outgrows MC candidates goes to ovf_list instead of failing.
-// Against 512 slots at 16 warps: 7.1 -> 5.9 ms on a 1e7-particle beam and
-// 31.6 -> 26.1 ms on a 64-beam batch (both passes); with the candidates' hash
-// set, packed adjacency, 64-bit rank keys and the FP64 code moved to the list
-// kernel 5.86 -> 5.43 ms (3340 instead of ~4200 instructions per node; the
-// shared-memory pipe is 70% busy with the FP32 factorisation's operands).  With MC = MAXC and LIST: the nodes of that list
-// (n_list of them), each warp writing its own D columns.  slots <= MC is the
+// arrival count after them); the autotuner picks SW.  Three forms:
+//   FP64, every node (MC = MAXC_FAST): 6.6 KB of shared memory per warp and 32
+//     warps per SM; a node whose ring outgrows MC candidates goes to ovf_list
+//     instead of failing (against 512 slots at 16 warps a fifth faster);
+//   SELECT, every node of the mixed form: ring and selection only, 2.4 KB and
+//     40 registers, 48 warps per SM (0.29 ms for 2.8e5 nodes, bound by
+//     instructions: 91% of the issue slots);
+//   LIST (MC = MAXC): the n_list nodes of list, each warp writing its own D
+//     columns.
+// One kernel for the mixed form's every node took 1.22 ms at 2.8e5 nodes and
+// 5.13 at 1.05e6, SELECT, k_wls32 and LIST 0.66 and 2.57.  slots <= MC is the
 // capacity in force (the context's stencil_slots in the first kernel).
-template <int SW, int MC, bool LIST, bool MIXED>
-__global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil(
+template <int SW, int MC, bool LIST, bool MIXED, bool SELECT>
+__global__ void __launch_bounds__(SW * 32, SELECT ? 48 / SW : (MC < MAXC ? 32 : 16) / SW) k_stencil(
     const int4 *__restrict__ ic, const int32_t *__restrict__ adj, const int32_t *__restrict__ bowner, int n_int,
     int m_target, int ring_max, double unit, double inv_unit, double ec, double inv_1mec, int32_t *__restrict__ nbr_out,
     int32_t *__restrict__ m_out, int32_t *__restrict__ ring_out, double *__restrict__ lap_out,
     double *__restrict__ lapd_out, double *__restrict__ D_out, int64_t dstride, double *__restrict__ rcond_out,
     double fp32_rcond_min, int *__restrict__ fp64_count, unsigned *err,
     const int32_t *__restrict__ list, int n_list, unsigned *__restrict__ ovf_count, int32_t *__restrict__ ovf_list,
-    int slots, int idx_bits, int d2_shift) {
-    typedef WarpSmemT<MC> WarpSmem;
+    int slots, int idx_bits, int d2_shift, Fp32Args fa) {
+    typedef typename std::conditional<SELECT, SelectSmemT<MC>, WarpSmemT<MC>>::type WarpSmem;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     WarpSmem &W = reinterpret_cast<WarpSmem *>(smem_raw)[wid];
@@ -525,12 +604,13 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
     const unsigned FULL = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
     unsigned *arrived = reinterpret_cast<unsigned *>(reinterpret_cast<WarpSmem *>(smem_raw) + SW);
-    if (!LIST) {
+    (void)arrived;
+    if (!LIST && !SELECT) {
         if (threadIdx.x == 0) *arrived = 0u;
         __syncthreads();
     }
     if (y0 >= n_int) {
-        if (!LIST) write_block_d<SW, WarpSmem>(smem_raw, arrived, lane, blockIdx.x * SW, n_int, D_out, dstride);
+        if constexpr (!LIST && !SELECT) write_block_d<SW, WarpSmem>(smem_raw, arrived, lane, blockIdx.x * SW, n_int, D_out, dstride);
         return;
     }
 
@@ -539,7 +619,7 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
     if (lane == 0) W.cand[0] = y0;
     __syncwarp();
     int head = 0, tail = 1;
-    bool done = false, overflow = false, redo = false;   // redo: by the list kernel
+    bool done = false, overflow = false;
     int m = 0, ring = 0;
     double rmin_over_rmax = 0.0;
 
@@ -547,7 +627,7 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
     int *tab = reinterpret_cast<int *>(W.d2);   // 2 MC slots
     bool hashed = false;
 
-    for (int k = 1; k <= ring_max && !done && !redo; ++k) {
+    for (int k = 1; k <= ring_max && !done; ++k) {
         // ---- grow the ring by one layer (Section 4.3: (k+1)-ring = k-ring
         // plus the face neighbours of its nodes).  Eight lanes per frontier
         // node read its neighbours (packed first in its 24 slots; nearly all
@@ -723,23 +803,32 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
         __syncwarp();
         m = nsel;
 
+        if constexpr (SELECT) {   // the operators are the next kernel's
+            nbr_out[(int64_t)y0 * MMAX + lane] = (lane < m) ? W.sel[lane] : -1;
+            if (lane == 0) {
+                m_out[y0] = m;
+                ring_out[y0] = k;
+            }
+            done = true;
+        } else {
         // ---- weighted least squares: FP32 first when asked, FP64 for blocks the
         // FP32 factorisation cannot certify (Cholesky failure or condition
         // estimate min|R_ii|/max|R_ii| below fp32_rcond_min, by default 1e-3,
         // where FP32 Cholesky QR loses its accuracy)
         double q[NCOL], lapj = 0.0;
         bool ok = false;
-        if (MIXED) {
-            ok = wls_column_f32(W, m, lane, own, c0, ic, unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
-            if (ok && rmin_over_rmax < fp32_rcond_min) ok = false;
-            if (!ok && !LIST) {   // the list kernel holds the FP64 code: here it would cost registers
-                redo = true;
-                break;
-            }
+        if constexpr (MIXED) {
+            float qf[NCOL], lf, rf;
+            ok = wls_column_f32(W, m, lane, own, c0, ic, unit, fa, d2_shift, qf, lf, rf) && !(rf < fa.rcond_min);
             if (!ok && lane == 0) atomicAdd(fp64_count, 1);
+            if (ok) {
+                rmin_over_rmax = (double)rf;
+                lapj = (double)lf;
+#pragma unroll
+                for (int e = 0; e < NCOL; ++e) q[e] = (double)qf[e];
+            }
         }
-        if ((LIST || !MIXED) && !ok)
-            ok = wls_column_f64(W, m, lane, own, c0, ic, inv_unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
+        if (!ok) ok = wls_column_f64(W, m, lane, own, c0, ic, inv_unit, ec, inv_1mec, q, lapj, rmin_over_rmax);
         if (ok) ok = rmin_over_rmax >= RANK_TOL;
         if (!ok) lapj = 0.0;
         const double lsum = warp_sum_d(lapj);
@@ -769,12 +858,13 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
         }
         ring = k;
         done = true;
+        }
         }   // target sizes
     }
     if (!done) {
         const bool ovf = overflow;
         if (lane == 0) {
-            if ((ovf || redo) && !LIST) ovf_list[atomicAdd(ovf_count, 1u)] = y0;   // redone with MAXC slots
+            if (ovf && !LIST) ovf_list[atomicAdd(ovf_count, 1u)] = y0;   // redone with MAXC slots
             else atomicOr(err, ovf ? (ERR_STENCIL | ERR_OVERFLOW) : ERR_STENCIL);
             m_out[y0] = 0;
             ring_out[y0] = -1;
@@ -784,16 +874,256 @@ __global__ void __launch_bounds__(SW * 32, (MC < MAXC ? 32 : 16) / SW) k_stencil
         nbr_out[(int64_t)y0 * MMAX + lane] = -1;
         lap_out[(int64_t)y0 * MMAX + lane] = 0.0;
         __syncwarp();
-        if (LIST) {
+        if constexpr (LIST) {
 #pragma unroll
             for (int e = 0; e < NCOL; ++e) D_out[((int64_t)e * MMAX + lane) * dstride + y0] = 0.0;
-        } else {
+        } else if constexpr (!SELECT) {
 #pragma unroll
             for (int e = 0; e < NCOL; ++e) W.A[e * MMAX + lane] = 0.0;
         }
     }
     (void)ring;
-    if (!LIST) write_block_d<SW, WarpSmem>(smem_raw, arrived, lane, blockIdx.x * SW, n_int, D_out, dstride);
+    if constexpr (!LIST && !SELECT) write_block_d<SW, WarpSmem>(smem_raw, arrived, lane, blockIdx.x * SW, n_int, D_out, dstride);
+}
+
+// The mixed form's operators of the selected stencils: wls_column_f32, four
+// nodes per warp.  With a warp per node, both 9x9 factorisations run in every
+// lane at once, 450 of 1700 instructions 32 times over; the loads of their
+// operands keep the shared-memory pipe busy; and the kernel that also selects
+// outgrows the instruction cache (1.9 of 10 cycles between instructions waited
+// for the next one).  Here a lane builds the rows of its neighbour for the four
+// nodes; then eight lanes have one node each: 3 x 3 blocks of its Gram matrix, the
+// factor in registers, every eighth row in the solves.  The same operations in
+// the same order: the same bits.  0.35 ms for 2.8e5 nodes, of which the operator's
+// 663 MB take 0.1 (with an entry of the Gram matrix per lane and the factors read
+// back from shared memory for every node 0.48: the load/store pipe 88% busy).
+// Conversions stay on the FP64 pipe: it is a third busy, and the integer ones
+// cost more issue slots than it has to spare.  Nodes the FP32
+// factorisation cannot certify, and those that need more neighbours, go to the
+// list kernel, which starts them again.
+constexpr int WN = 4;   // nodes per warp
+constexpr int WLS_SW = 4;                      // warps per block
+struct __align__(16) Wls32Smem {
+    float A[WN][(NCOL + 1) * FSTR];   // rows by columns, then the weights; at the end the operator, [e * MMAX + lane]
+    unsigned good, pad[3];
+    float G[WN][48], R1[WN][60];      // Gram matrix, then R2; R1: 45 packed entries, from 48 on the reciprocal diagonal
+};
+
+__device__ __forceinline__ void load_factor(const float *F, float (&R)[48], float (&Ri)[NCOL]) {
+#pragma unroll
+    for (int e = 0; e < 12; ++e) {
+        const float4 v = reinterpret_cast<const float4 *>(F)[e];
+        R[4 * e] = v.x;
+        R[4 * e + 1] = v.y;
+        R[4 * e + 2] = v.z;
+        R[4 * e + 3] = v.w;
+    }
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) Ri[e] = F[48 + e];
+}
+__device__ __forceinline__ void store_factor(float *F, const float (&R)[48], const float (&Ri)[NCOL]) {
+#pragma unroll
+    for (int e = 0; e < 12; ++e)
+        reinterpret_cast<float4 *>(F)[e] = make_float4(R[4 * e], R[4 * e + 1], R[4 * e + 2], R[4 * e + 3]);
+#pragma unroll
+    for (int e = 0; e < NCOL; ++e) F[48 + e] = Ri[e];
+}
+
+// Gram matrix of one node's rows by eight lanes, six of them a 3 x 3 block each
+// (what falls below the diagonal is not stored): six loads of four rows for 36
+// multiply-adds, where an entry per lane takes four for eight.  Rows m to
+// mmax (below 32) are zeros; every entry is summed in row order.
+__device__ __forceinline__ void gram_blocks(const float *A, int mmax, float *G, int blk) {
+    const int br = blk < 3 ? 0 : (blk < 5 ? 1 : 2), bc = blk < 3 ? blk : (blk < 5 ? blk - 2 : 2);
+    const float *pa = A + 3 * br * FSTR, *pb = A + 3 * bc * FSTR;
+    float s[3][3] = {};
+#pragma unroll 1
+    for (int j = 0; j < mmax; j += 4) {
+        float4 a[3], b[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            a[i] = *reinterpret_cast<const float4 *>(pa + i * FSTR + j);
+            b[i] = *reinterpret_cast<const float4 *>(pb + i * FSTR + j);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                float t = s[i][k];
+                t = fmaf(a[i].x, b[k].x, t);
+                t = fmaf(a[i].y, b[k].y, t);
+                t = fmaf(a[i].z, b[k].z, t);
+                s[i][k] = fmaf(a[i].w, b[k].w, t);
+            }
+    }
+    if (blk < 6) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (br < bc || i <= k) G[pk_idx(3 * br + i, 3 * bc + k)] = s[i][k];
+    }
+}
+
+template <int SW>
+__global__ void __launch_bounds__(SW * 32, 24 / SW) k_wls32(
+    const int4 *__restrict__ ic, int n_int, double unit, Fp32Args fa, int d2_shift, const int32_t *__restrict__ nbr,
+    const int32_t *__restrict__ msz, double *__restrict__ lap_out, double *__restrict__ lapd_out,
+    double *__restrict__ D_out, int64_t dstride, double *__restrict__ rcond_out, unsigned *__restrict__ list_count,
+    int32_t *__restrict__ list) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    Wls32Smem &W = reinterpret_cast<Wls32Smem *>(smem_raw)[wid];
+    const int w0 = (blockIdx.x * SW + wid) * WN;   // past the last node: empty stencils
+    const unsigned FULL = 0xffffffffu;
+    // ---- rows, a lane per neighbour; lane q < WN keeps node q's size and h in units
+    const int my_m = lane < WN && w0 + lane < n_int ? msz[w0 + lane] : 0;
+    float my_hint = 1.f;
+    int4 p[WN], c0[WN];
+#pragma unroll
+    for (int q = 0; q < WN; ++q) {
+        const int m = __shfl_sync(FULL, my_m, q);
+        const int id = lane < m ? nbr[(int64_t)(w0 + q) * MMAX + lane] : -1;
+        c0[q] = m > 0 ? ic[w0 + q] : make_int4(0, 0, 0, 0);
+        p[q] = id >= 0 ? ic[id] : c0[q];
+    }
+#pragma unroll
+    for (int q = 0; q < WN; ++q) {
+        const int m = __shfl_sync(FULL, my_m, q);
+        const int o0 = p[q].x - c0[q].x, o1 = p[q].y - c0[q].y, o2 = p[q].z - c0[q].z;
+        const int hint = __reduce_max_sync(FULL, max(abs(o0), max(abs(o1), abs(o2))));
+        // offsets are whole multiples of 2^(d2_shift / 2), half cells of the deepest level
+        const int h0 = o0 >> (d2_shift >> 1), h1 = o1 >> (d2_shift >> 1), h2 = o2 >> (d2_shift >> 1);
+        const unsigned long long d = (unsigned long long)((long long)h0 * h0 + (long long)h1 * h1 + (long long)h2 * h2);
+        const unsigned long long r2max = __shfl_sync(FULL, d, m - 1);   // the last is the farthest
+        if (lane == q) my_hint = (float)hint;
+        float row[NCOL], wj = 0.f;
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) row[e] = 0.f;
+        if (lane < m) {
+            const float fh = (float)hint;
+            const float xi0 = (float)o0 / fh, xi1 = (float)o1 / fh, xi2 = (float)o2 / fh;
+            const float ratio = (r2max >> 32) ? (float)d / (float)r2max : (float)(unsigned)d / (float)(unsigned)r2max;
+            wj = (expf(-ratio) - fa.ec) * fa.inv_1mec;
+            row[0] = xi0; row[1] = xi1; row[2] = xi2;
+            row[3] = (0.5f * xi0) * xi0;
+            row[4] = xi0 * xi1;
+            row[5] = xi0 * xi2;
+            row[6] = (0.5f * xi1) * xi1;
+            row[7] = xi1 * xi2;
+            row[8] = (0.5f * xi2) * xi2;
+#pragma unroll
+            for (int e = 0; e < NCOL; ++e) row[e] = wj * row[e];
+        }
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) W.A[q][e * FSTR + lane] = row[e];
+        W.A[q][NCOL * FSTR + lane] = wj;
+    }
+    __syncwarp();
+    // ---- from here on lanes 8 q to 8 q + 7 have node q: a 3 x 3 block of its Gram
+    // matrix each, its factor in the registers of all eight, every eighth row
+    const int sub = lane >> 3, r0 = lane & 7, mmax = __reduce_max_sync(FULL, my_m), m = __shfl_sync(FULL, my_m, sub);
+    float *A = W.A[sub] + r0;
+    gram_blocks(W.A[sub], mmax, W.G[sub], r0);
+    __syncwarp();
+    float R[48], Ri[NCOL];
+    bool ok = cholesky_regs(W.G[sub], R, Ri);
+    if (r0 == 0) store_factor(W.R1[sub], R, Ri);
+#pragma unroll 1
+    for (int i = 0; i < MMAX; i += 8) {
+        float v[NCOL];
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) v[e] = A[e * FSTR + i];
+        row_solve_upper(R, Ri, v);
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) A[e * FSTR + i] = v[e];
+    }
+    __syncwarp();
+    gram_blocks(W.A[sub], mmax, W.G[sub], r0);
+    __syncwarp();
+    ok = cholesky_regs(W.G[sub], R, Ri) && ok;
+    float rf;
+    {
+        float dmin = 1e30f, dmax = 0.f;
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) {
+            const float r = fabsf(W.R1[sub][pk_idx(e, e)] * R[pk_idx(e, e)]);
+            dmin = fminf(dmin, r);
+            dmax = fmaxf(dmax, r);
+        }
+        rf = dmin / dmax;
+    }
+    ok = ok && !(rf < fa.rcond_min) && rf >= fa.rank_min;
+#pragma unroll 1
+    for (int i = 0; i < MMAX; i += 8) {
+        float v[NCOL];
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) v[e] = A[e * FSTR + i];
+        row_solve_upper(R, Ri, v);
+        col_solve_open(R, Ri, v);
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) A[e * FSTR + i] = v[e];
+    }
+    const float rd20 = Ri[0];
+    // columns of P, unscaled by 1/h and 1/h^2, and the Laplacian's in place of the weights
+    load_factor(W.R1[sub], R, Ri);
+    const float h = (float)((double)__shfl_sync(FULL, my_hint, sub) * unit), ih = 1.f / h, ih2 = ih * ih;
+#pragma unroll 1
+    for (int i = 0; i < MMAX; i += 8) {
+        float v[NCOL], lj = 0.f;
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) v[e] = A[e * FSTR + i];
+        col_solve_tail(R, Ri, v, rd20);
+        const float wj = A[NCOL * FSTR + i];
+        const bool live = ok && r0 + i < m;
+#pragma unroll
+        for (int e = 0; e < NCOL; ++e) {
+            v[e] = live ? (v[e] * wj) * (e < 3 ? ih : ih2) : 0.f;
+            if (e == 3 || e == 6 || e == 8) lj += v[e];
+            A[e * FSTR + i] = v[e];
+        }
+        A[NCOL * FSTR + i] = lj;
+    }
+    __syncwarp();
+    // sums of the Laplacian columns: warp_sum_d's tree for the four nodes at
+    // once, one after the first two steps in each quarter of the warp
+    double lsum;
+    {
+        float l[WN];
+#pragma unroll
+        for (int q = 0; q < WN; ++q) l[q] = W.A[q][NCOL * FSTR + lane];
+        const bool up = lane & 16, odd = lane & 8;
+        const double a = (double)(up ? l[2] : l[0]) + (double)__shfl_xor_sync(FULL, up ? l[0] : l[2], 16);
+        const double b = (double)(up ? l[3] : l[1]) + (double)__shfl_xor_sync(FULL, up ? l[1] : l[3], 16);
+        lsum = (odd ? b : a) + __shfl_xor_sync(FULL, odd ? a : b, 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) lsum += __shfl_xor_sync(FULL, lsum, o);
+    }
+    // lanes 8 q to 8 q + 7 hold node q's sum (and its ok and rf)
+    const bool good = ok && -lsum < 0.0;
+    const unsigned gmask = __ballot_sync(FULL, good);
+    if (r0 == 0 && w0 + sub < n_int) {
+        lapd_out[w0 + sub] = good ? -lsum : 0.0;
+        rcond_out[w0 + sub] = good ? (double)rf : 0.0;
+        if (!good && m > 0) list[atomicAdd(list_count, 1u)] = w0 + sub;   // m = 0: listed when selected
+    }
+#pragma unroll
+    for (int q = 0; q < WN; ++q)
+        if (w0 + q < n_int)
+            lap_out[(int64_t)(w0 + q) * MMAX + lane] =
+                gmask >> (8 * q) & 1u ? (double)W.A[q][NCOL * FSTR + lane] : 0.0;
+    // the block's nodes' columns side by side
+    if (lane == 0) W.good = gmask;
+    __syncthreads();
+    constexpr int NB = SW * WN;
+    const int nd = threadIdx.x % NB, y = blockIdx.x * NB + nd;
+    const Wls32Smem &V = reinterpret_cast<const Wls32Smem *>(smem_raw)[nd / WN];
+    if (y < n_int) {
+        const bool g = V.good >> (8 * (nd % WN)) & 1u;
+#pragma unroll 4
+        for (int row = threadIdx.x / NB; row < NCOL * MMAX; row += SW * 32 / NB)
+            D_out[(int64_t)row * dstride + y] = g ? (double)V.A[nd % WN][row + (FSTR - MMAX) * (row / MMAX)] : 0.0;
+    }
 }
 
 // ---------------------------------------------------------------- matrices
@@ -911,27 +1241,43 @@ apcloud_status launch_stencil_of(apcloud_ctx *c, int n, double unit, double ec, 
     while ((1ll << idx_bits) < c->n_tot) ++idx_bits;
     if (2 * c->L + 4 + idx_bits > 63) idx_bits = 0;
     const int d2_shift = 2 * (KEY_DEPTH - c->L);
-    const size_t smem = SW * sizeof(WarpSmemT<MAXC_FAST>) + 16;   // the warps' areas, then the block's arrival count
-    // the limit is a per-device property of the function: set on every build
-    // (one host call each), so that contexts on other devices get it too
-    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<SW, MAXC_FAST, false, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
-    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<4, MAXC, true, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const Fp32Args fa{(float)ec, (float)inv_1mec, fp32_not_below(c->P.fp32_rcond_min), fp32_not_below(RANK_TOL)};
+    // the limits are per-device properties of the functions: set on every build
+    // (one host call each), so that contexts on other devices get them too
+    APC_CUDA(c, cudaFuncSetAttribute(k_stencil<4, MAXC, true, MIXED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)(4 * sizeof(WarpSmemT<MAXC>) + 16)));
-    APC_LAUNCH(c, K_STENCIL, div_up(n, SW), SW * 32, smem, (k_stencil<SW, MAXC_FAST, false, MIXED>), ptr<int4>(c->node_ic),
-               ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target, c->P.ring_max, unit, 1.0 / unit, ec, inv_1mec,
-               nbr, msz, ring, lap, lapd, D, dstride, rc, c->P.fp32_rcond_min,
-               reinterpret_cast<int *>(derr + 1), derr, (const int32_t *)nullptr, 0, derr + 2, ovf, c->P.stencil_slots,
-               idx_bits, d2_shift);
+    if constexpr (MIXED) {
+        const size_t smem = SW * sizeof(SelectSmemT<MAXC_FAST>) + 16, wsmem = WLS_SW * sizeof(Wls32Smem);
+        APC_CUDA(c, cudaFuncSetAttribute(k_stencil<SW, MAXC_FAST, false, true, true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        APC_CUDA(c, cudaFuncSetAttribute(k_wls32<WLS_SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem));
+        APC_LAUNCH(c, K_STENCIL, div_up(n, SW), SW * 32, smem, (k_stencil<SW, MAXC_FAST, false, true, true>),
+                   ptr<int4>(c->node_ic), ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target,
+                   c->P.ring_max, unit, 1.0 / unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc,
+                   c->P.fp32_rcond_min, reinterpret_cast<int *>(derr + 1), derr, (const int32_t *)nullptr, 0, derr + 2,
+                   ovf, c->P.stencil_slots, idx_bits, d2_shift, fa);
+        APC_LAUNCH(c, K_STENCIL, div_up(n, WLS_SW * WN), WLS_SW * 32, wsmem, (k_wls32<WLS_SW>), (const int4 *)ptr<int4>(c->node_ic),
+                   n, unit, fa, d2_shift, (const int32_t *)nbr, (const int32_t *)msz, lap, lapd, D, dstride, rc, derr + 2,
+                   ovf);
+    } else {
+        const size_t smem = SW * sizeof(WarpSmemT<MAXC_FAST>) + 16;   // the warps' areas, then the block's arrival count
+        APC_CUDA(c, cudaFuncSetAttribute(k_stencil<SW, MAXC_FAST, false, false, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        APC_LAUNCH(c, K_STENCIL, div_up(n, SW), SW * 32, smem, (k_stencil<SW, MAXC_FAST, false, false, false>),
+                   ptr<int4>(c->node_ic), ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target,
+                   c->P.ring_max, unit, 1.0 / unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc,
+                   c->P.fp32_rcond_min, reinterpret_cast<int *>(derr + 1), derr, (const int32_t *)nullptr, 0, derr + 2,
+                   ovf, c->P.stencil_slots, idx_bits, d2_shift, fa);
+    }
     // the overflow count, with the error word and the count of FP64 blocks
     APC_TRY(read_back(c, words, derr, 3 * sizeof(unsigned)));
     const unsigned nov = words[2];
     if (nov > 0) {
-        APC_LAUNCH(c, K_STENCIL, div_up(nov, 4), 4 * 32, 4 * sizeof(WarpSmemT<MAXC>) + 16, (k_stencil<4, MAXC, true, MIXED>),
+        APC_LAUNCH(c, K_STENCIL, div_up(nov, 4), 4 * 32, 4 * sizeof(WarpSmemT<MAXC>) + 16, (k_stencil<4, MAXC, true, MIXED, false>),
                    ptr<int4>(c->node_ic), ptr<int32_t>(c->adj), ptr<int32_t>(c->bowner), n, c->P.m_target,
                    c->P.ring_max, unit, 1.0 / unit, ec, inv_1mec, nbr, msz, ring, lap, lapd, D, dstride, rc,
                    c->P.fp32_rcond_min, reinterpret_cast<int *>(derr + 1), derr,
-                   (const int32_t *)ovf, (int)nov, derr + 2, ovf, MAXC, idx_bits, d2_shift);
+                   (const int32_t *)ovf, (int)nov, derr + 2, ovf, MAXC, idx_bits, d2_shift, fa);
         APC_TRY(read_back(c, words, derr, 3 * sizeof(unsigned)));
     }
     return APCLOUD_OK;
