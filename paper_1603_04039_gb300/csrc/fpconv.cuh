@@ -1,4 +1,4 @@
-// fpconv.cuh -- binary64 <-> binary32 conversions, and the floor, clamp and
+// fpconv.cuh -- binary64 <-> binary32 and binary64 -> binary16 conversions, and the floor, clamp and
 // range test of the Morton-key quantisation, on the integer pipe.
 //
 // GB300 runs FP64 arithmetic, and the conversions between double and float,
@@ -16,6 +16,8 @@
 // bit against the hardware conversions and the FP64 floor / fmin / fmax /
 // comparison forms by tests/test_gpu_fpconv.py (NaNs compare as NaNs).
 #pragma once
+
+#include <cuda_fp16.h>
 
 #include <cstdint>
 
@@ -66,6 +68,32 @@ __device__ __forceinline__ double f32_to_f64_int(float f) {
         lo = (uint32_t)fr;
     }
     return __hiloint2double((int)hi, (int)lo);
+}
+
+// double -> half (binary16: 5 exponent bits, bias 15, 10 fraction bits), round
+// to nearest even, the steps of f64_to_f32_int with 42 dropped bits
+__device__ __forceinline__ __half f64_to_f16_int(double d) {
+    const uint64_t b = (uint64_t)__double_as_longlong(d);
+    const uint32_t sign = (uint32_t)(b >> 48) & 0x8000u;
+    const int E = (int)((b >> 52) & 0x7FFu), e = E - 1023 + 15;
+    const uint64_t frac = b & 0xFFFFFFFFFFFFFull;
+    uint32_t r;
+    if (E == 0x7FF) {
+        r = frac ? 0x7FFFu : 0x7C00u;
+    } else if (e >= 31) {
+        r = 0x7C00u;
+    } else {
+        const uint64_t sig = (E ? (1ull << 52) : 0ull) | frac;
+        const int drop = e > 0 ? 42 : 42 + 1 - e;
+        if (drop >= 64) {
+            r = 0u;
+        } else {
+            const uint64_t keep = sig >> drop, rest = sig & ((1ull << drop) - 1ull), half = 1ull << (drop - 1);
+            const uint32_t up = (rest > half || (rest == half && (keep & 1ull))) ? 1u : 0u;
+            r = (e > 0 ? (uint32_t)(e - 1) << 10 : 0u) + (uint32_t)keep + up;
+        }
+    }
+    return __ushort_as_half((unsigned short)(sign | r));
 }
 
 // min(max(floor(t), 0), maxv) as an unsigned integer, for maxv < 2^31; NaN

@@ -1130,7 +1130,7 @@ __global__ void __launch_bounds__(SW * 32, 24 / SW) k_wls32(
 // diagonals of A and B (the Jacobi scaling) and their reciprocals
 __global__ void k_diag(const int32_t *__restrict__ msz, const double *__restrict__ lapd, const int4 *__restrict__ ic,
                        int n_int, int n_tot, double ext, double *__restrict__ dA, double *__restrict__ dB,
-                       double *__restrict__ rA, double *__restrict__ rB) {
+                       double2 *__restrict__ rAB) {
     int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_tot) return;
     double a = 1.0, b = 1.0;
@@ -1142,8 +1142,7 @@ __global__ void k_diag(const int32_t *__restrict__ msz, const double *__restrict
     }
     dA[r] = a;
     dB[r] = b;
-    rA[r] = 1.0 / a;
-    rB[r] = 1.0 / b;
+    rAB[r] = make_double2(1.0 / a, 1.0 / b);
 }
 
 // widths of the 32-row slices; also the sum of the stencil sizes
@@ -1167,64 +1166,89 @@ __global__ void k_slice_width(const int32_t *__restrict__ msz, int n_int, int n_
 // and (h_j^2/24) l_ji (Section 3.2 with the cell-indicator moments); boundary
 // rows are identity rows.  Values are stored right-scaled by the inverse
 // diagonal of the column (Jacobi preconditioning folded into the matrix).
-__global__ void k_ell_fill(const int32_t *__restrict__ msz, const int32_t *__restrict__ nbr,
-                           const double *__restrict__ lap, const double *__restrict__ lapd, const int4 *__restrict__ ic,
-                           const double *__restrict__ dA, const double *__restrict__ dB, const double *__restrict__ rA,
-                           const double *__restrict__ rB, int n_int, int n_tot, double ext,
-                           const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff,
-                           int32_t *__restrict__ col, double *__restrict__ vA, double *__restrict__ vB) {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
-    int s = r >> 5, lane = r & 31;
+//
+// The FP64 pipe's three products per entry and 44 bytes of it take about as
+// long.  The mixed form's FP32 and FP16 copies are written along (a pass of their
+// own read the values again and converted to FP16 on the FP64 pipe), a row's
+// four next columns and values come in three loads and a column's two
+// reciprocals in one: at 2.5e7 entries 290 us, fill and copies 262 + 190 before.
+struct LowCopies {   // null without the mixed form
+    float *fA, *fB;
+    __half *hA, *hB;
+};
+template <bool MIXED>
+__device__ __forceinline__ void put_low(const LowCopies &c, int64_t e, double a, double b) {
+    if constexpr (MIXED) {
+        c.fA[e] = f64_to_f32_int(a);
+        c.fB[e] = f64_to_f32_int(b);
+        c.hA[e] = f64_to_f16_int(a);
+        c.hB[e] = f64_to_f16_int(b);
+    }
+}
+
+template <bool MIXED>
+__global__ void __launch_bounds__(256) k_ell_fill(
+    const int32_t *__restrict__ msz, const int32_t *__restrict__ nbr, const double *__restrict__ lap,
+    const double *__restrict__ lapd, const int4 *__restrict__ ic, const double *__restrict__ dA,
+    const double *__restrict__ dB, const double2 *__restrict__ rAB, int n_int, int n_tot, double ext,
+    const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff, int32_t *__restrict__ col,
+    double *__restrict__ vA, double *__restrict__ vB, LowCopies low) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = r >> 5, lane = r & 31;
     if (s * 32 >= n_tot) return;
-    int w = (int)sw[s];
-    int64_t base = (int64_t)soff[s] * 32 + lane;
-    if (r >= n_tot) {
-        for (int k = 0; k < w; ++k) { col[base + k * 32] = 0; vA[base + k * 32] = 0.0; vB[base + k * 32] = 0.0; }
-        return;
+    const int w = (int)sw[s];
+    const int64_t base = (int64_t)soff[s] * 32 + lane;
+    const bool real = r < n_tot, inner = r < n_int;
+    const int m = inner ? msz[r] : 0, own = real ? r : 0;
+    double a0 = 0.0, b0 = 0.0, sc = 0.0;
+    if (inner) {
+        const double h = ldexp(ext, -ic[r].w), l = lapd[r];
+        sc = h * h / 24.0;
+        a0 = l / dA[r];
+        b0 = (1.0 + sc * l) / dB[r];
+    } else if (real) {
+        a0 = 1.0 / dA[r];
+        b0 = 1.0 / dB[r];
     }
-    if (r >= n_int) {
-        col[base] = r; vA[base] = 1.0 / dA[r]; vB[base] = 1.0 / dB[r];
-        for (int k = 1; k < w; ++k) { col[base + k * 32] = r; vA[base + k * 32] = 0.0; vB[base + k * 32] = 0.0; }
-        return;
-    }
-    int m = msz[r];
-    double h = ldexp(ext, -ic[r].w);
-    double sc = h * h / 24.0;
-    col[base] = r;
-    vA[base] = lapd[r] / dA[r];
-    vB[base] = (1.0 + sc * lapd[r]) / dB[r];
-    for (int k = 1; k < w; ++k) {
-        int64_t e = base + (int64_t)k * 32;
-        if (k <= m) {
-            int cj = nbr[(int64_t)r * MMAX + k - 1];
-            double l = lap[(int64_t)r * MMAX + k - 1];
+    col[base] = own;
+    vA[base] = a0;
+    vB[base] = b0;
+    put_low<MIXED>(low, base, a0, b0);
+    for (int k0 = 0; k0 + 1 < w; k0 += 4) {
+        int id[4] = {own, own, own, own};
+        double l[4] = {0.0, 0.0, 0.0, 0.0};
+        if (k0 < m) {   // MMAX entries per row: aligned, and never past the row's end
+            const int4 q = *reinterpret_cast<const int4 *>(nbr + (int64_t)r * MMAX + k0);
+            const double2 x = *reinterpret_cast<const double2 *>(lap + (int64_t)r * MMAX + k0);
+            const double2 y = *reinterpret_cast<const double2 *>(lap + (int64_t)r * MMAX + k0 + 2);
+            id[0] = q.x; id[1] = q.y; id[2] = q.z; id[3] = q.w;
+            l[0] = x.x; l[1] = x.y; l[2] = y.x; l[3] = y.y;
+        }
+        double2 rc[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) rc[t] = k0 + t < m ? rAB[id[t]] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (k0 + t + 1 >= w) break;
+            const int64_t e = base + (int64_t)(k0 + t + 1) * 32;
             // off-diagonal entries times the column's reciprocal diagonal (an
             // FP64 division per entry would make this pass FP64-bound; the
             // diagonal entries above keep their exact division, so they stay 1)
-            col[e] = cj;
-            vA[e] = l * rA[cj];
-            vB[e] = (sc * l) * rB[cj];
-        } else {
-            col[e] = r;
-            vA[e] = 0.0;
-            vB[e] = 0.0;
+            const bool in = k0 + t < m;
+            const double a = in ? l[t] * rc[t].x : 0.0, b = in ? (sc * l[t]) * rc[t].y : 0.0;
+            col[e] = in ? id[t] : own;
+            vA[e] = a;
+            vB[e] = b;
+            put_low<MIXED>(low, e, a, b);
         }
     }
 }
 
-// FP32 copies of the stored (Jacobi-scaled) matrix values for the mixed form
-__global__ void k_values_f32(const double *__restrict__ vA, const double *__restrict__ vB, int64_t n,
-                             float *__restrict__ fA, float *__restrict__ fB, __half *__restrict__ hA,
-                             __half *__restrict__ hB) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        // the FP32 copies on the integer pipe (bit-exact); the FP16 ones keep
-        // the hardware conversion (a direct rounding from FP64)
-        fA[i] = f64_to_f32_int(vA[i]);
-        fB[i] = f64_to_f32_int(vB[i]);
-        hA[i] = __double2half(vA[i]);
-        hB[i] = __double2half(vB[i]);
-    }
+// FP32 and FP16 copies of the stored (Jacobi-scaled) matrix values for the mixed
+// form, when those have changed
+__global__ void k_values_low(const double *__restrict__ vA, const double *__restrict__ vB, int64_t n, LowCopies low) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) put_low<true>(low, i, vA[i], vB[i]);
 }
 
 template <int SW, bool MIXED>
@@ -1335,11 +1359,9 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     uint32_t *so = ensure<uint32_t>(c, c->slice_off, nsl + 1);
     double *dA = ensure<double>(c, c->dA, nt + 1);
     double *dB = ensure<double>(c, c->dB, nt + 1);
-    double *rd = ensure<double>(c, c->ell_rd, 2 * ((int64_t)nt + 1));   // reciprocals, for the fill only
+    double2 *rd = ensure<double2>(c, c->ell_rd, (int64_t)nt + 1);   // reciprocals, for the fill only
     if (!sw || !so || !dA || !dB || !rd) return APCLOUD_E_NOMEM;
-    double *rA = rd, *rB = rd + nt + 1;
-    APC_LAUNCH(c, K_ELL, div_up(nt, 256), 256, 0, k_diag, msz, lapd, ptr<int4>(c->node_ic), n, nt, ext, dA, dB, rA,
-               rB);
+    APC_LAUNCH(c, K_ELL, div_up(nt, 256), 256, 0, k_diag, msz, lapd, ptr<int4>(c->node_ic), n, nt, ext, dA, dB, rd);
     uint32_t *small = ptr<uint32_t>(c->dsmall);
     APC_CUDA(c, cudaMemsetAsync(small + 6, 0, sizeof(uint32_t), c->s));
     APC_LAUNCH(c, K_ELL, div_up(nsl, 8), 256, 0, k_slice_width, msz, n, nt, nsl, sw, small + 6);
@@ -1363,15 +1385,15 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     double *vA = ensure<double>(c, c->ell_A, c->ell_entries);
     double *vB = ensure<double>(c, c->ell_B, c->ell_entries);
     if (!col || !vA || !vB) return APCLOUD_E_NOMEM;
-    APC_LAUNCH(c, K_ELL, div_up((int64_t)nsl * 32, 256), 256, 0, k_ell_fill, msz, nbr, lap, lapd,
-               ptr<int4>(c->node_ic), dA, dB, (const double *)rA, (const double *)rB, n, nt, ext, sw, so, col, vA,
-               vB);
-    if (c->P.precision == 1) {
-        float *fA = ensure<float>(c, c->ell_A32, c->ell_entries), *fB = ensure<float>(c, c->ell_B32, c->ell_entries);
-        __half *hA = ensure<__half>(c, c->ell_A16, c->ell_entries), *hB = ensure<__half>(c, c->ell_B16, c->ell_entries);
-        if (!fA || !fB || !hA || !hB) return APCLOUD_E_NOMEM;
-        APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_f32, (const double *)vA,
-                   (const double *)vB, c->ell_entries, fA, fB, hA, hB);
+    if (c->P.precision == 0) {
+        APC_LAUNCH(c, K_ELL, div_up((int64_t)nsl * 32, 256), 256, 0, k_ell_fill<false>, msz, nbr, lap, lapd,
+                   ptr<int4>(c->node_ic), dA, dB, (const double2 *)rd, n, nt, ext, sw, so, col, vA, vB, LowCopies{});
+    } else {
+        const LowCopies low{ensure<float>(c, c->ell_A32, c->ell_entries), ensure<float>(c, c->ell_B32, c->ell_entries),
+                            ensure<__half>(c, c->ell_A16, c->ell_entries), ensure<__half>(c, c->ell_B16, c->ell_entries)};
+        if (!low.fA || !low.fB || !low.hA || !low.hB) return APCLOUD_E_NOMEM;
+        APC_LAUNCH(c, K_ELL, div_up((int64_t)nsl * 32, 256), 256, 0, k_ell_fill<true>, msz, nbr, lap, lapd,
+                   ptr<int4>(c->node_ic), dA, dB, (const double2 *)rd, n, nt, ext, sw, so, col, vA, vB, low);
         if (blocks && !resident_ok(c, 1)) APC_TRY(build_blocks(c));
     }
     return cuda_check(c, cudaGetLastError(), "ell");
@@ -1440,9 +1462,9 @@ namespace apc {
 // FP32/FP16 copies of the stored values again (after the FP64 values changed)
 apcloud_status refresh_lowp(apcloud_ctx *c) {
     if (c->P.precision != 1 || c->ell_entries == 0) return APCLOUD_OK;
-    APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_f32, (const double *)ptr<double>(c->ell_A),
-               (const double *)ptr<double>(c->ell_B), c->ell_entries, ptr<float>(c->ell_A32), ptr<float>(c->ell_B32),
-               ptr<__half>(c->ell_A16), ptr<__half>(c->ell_B16));
+    APC_LAUNCH(c, K_ELL, div_up(c->ell_entries, 256), 256, 0, k_values_low, (const double *)ptr<double>(c->ell_A),
+               (const double *)ptr<double>(c->ell_B), c->ell_entries,
+               LowCopies{ptr<float>(c->ell_A32), ptr<float>(c->ell_B32), ptr<__half>(c->ell_A16), ptr<__half>(c->ell_B16)});
     if (c->bl_tried) APC_TRY(build_blocks(c));
     return cuda_check(c, cudaGetLastError(), "refresh_lowp");
 }

@@ -53,6 +53,9 @@ constexpr int BB_T = 512, BB_TAB = 8192;   // threads and hash slots of the buil
 // One block's columns outside its rows, sorted, and its entries in the layout
 // above.  A block with more than BL_HMAX such columns, or a diagonal that is not
 // 1, sets *bad: the system then stays on the ELL.
+// 281 us at 1.05e6 rows, most of it latency (350 with one column and one chunk's
+// values in flight per lane): three blocks per SM, a bitonic sort of some 1200
+// nodes each.
 __global__ void __launch_bounds__(BB_T) k_block_build(
     const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff, const int32_t *__restrict__ col,
     const __half *__restrict__ hA, const __half *__restrict__ hB, const float *__restrict__ fA,
@@ -71,21 +74,30 @@ __global__ void __launch_bounds__(BB_T) k_block_build(
     for (int i = tid; i < BB_TAB; i += BB_T) key[i] = -1;
     if (tid == 0) cnt = 0;
     __syncthreads();
-    volatile int *vc = &cnt;
+    volatile int *vc = &cnt, *vkey = key;
     const int64_t e0 = (int64_t)soff[s0] * 32, e1 = ((int64_t)soff[s1 - 1] + sw[s1 - 1]) * 32;
-    for (int64_t e = e0 + tid; e < e1; e += BB_T) {
-        const int c = col[e];
-        if ((c >= r0 && c < r1) || *vc > BL_HMAX) continue;   // the table never fills: at most BL_HMAX + BB_T entries
-        unsigned h = (unsigned)c * 0x9E3779B1u >> 19;
-        for (;;) {
-            const int old = atomicCAS(key + h, -1, c);
-            if (old == c) break;
-            if (old == -1) {
-                const int p = atomicAdd(&cnt, 1);
-                if (p < BL_HMAX) list[p] = c;
-                break;
+    for (int64_t e = e0 + tid; e < e1; e += 8 * BB_T) {   // eight columns in flight
+        int cc[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) cc[t] = e + t * BB_T < e1 ? col[e + t * BB_T] : r0;
+#pragma unroll 1
+        for (int t = 0; t < 8; ++t) {
+            const int c = cc[0];
+#pragma unroll
+            for (int u = 0; u < 7; ++u) cc[u] = cc[u + 1];
+            if ((c >= r0 && c < r1) || *vc > BL_HMAX) continue;   // the table never fills: at most BL_HMAX + BB_T entries
+            unsigned h = (unsigned)c * 0x9E3779B1u >> 19;
+            for (;;) {
+                int old = vkey[h];   // most are there already
+                if (old == -1) old = atomicCAS(key + h, -1, c);
+                if (old == c) break;
+                if (old == -1) {
+                    const int p = atomicAdd(&cnt, 1);
+                    if (p < BL_HMAX) list[p] = c;
+                    break;
+                }
+                h = (h + 1) & (BB_TAB - 1);
             }
-            h = (h + 1) & (BB_TAB - 1);
         }
     }
     __syncthreads();
@@ -134,28 +146,32 @@ __global__ void __launch_bounds__(BB_T) k_block_build(
         }
         const int64_t ob = (int64_t)off4[s] * 32 + lane;
         for (int j = 0; j * 4 < w; ++j) {
+            int c[4];
             uint32_t ix[4], a[4], b[4];
             float va[4], vb[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const int k = 4 * j + t;
-                ix[t] = (uint32_t)(r < n ? r - r0 : 0);   // past the row: itself, times zero
-                a[t] = b[t] = 0u;
-                va[t] = vb[t] = 0.f;
-                if (k < m) {
-                    const int64_t e = eb + (int64_t)k * 32;
-                    const int c = col[e];
-                    if (c >= r0 && c < r1) {
-                        ix[t] = (uint32_t)(c - r0);
-                    } else {
-                        unsigned h = (unsigned)c * 0x9E3779B1u >> 19;
-                        while (key[h] != c) h = (h + 1) & (BB_TAB - 1);
-                        ix[t] = loc[h];
-                    }
-                    a[t] = __half_as_ushort(hA[e]);
-                    b[t] = __half_as_ushort(hB[e]);
-                    va[t] = fA[e];
-                    vb[t] = fB[e];
+                const int64_t e = eb + (int64_t)(k < m ? k : -1) * 32;   // past the row: the diagonal's place
+                c[t] = col[e];
+                a[t] = __half_as_ushort(hA[e]);
+                b[t] = __half_as_ushort(hB[e]);
+                va[t] = fA[e];
+                vb[t] = fB[e];
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const bool in = 4 * j + t < m;
+                if (!in) {   // itself, times zero
+                    a[t] = b[t] = 0u;
+                    va[t] = vb[t] = 0.f;
+                }
+                if (!in || (c[t] >= r0 && c[t] < r1)) {
+                    ix[t] = (uint32_t)(in ? c[t] - r0 : (r < n ? r - r0 : 0));
+                } else {
+                    unsigned h = (unsigned)c[t] * 0x9E3779B1u >> 19;
+                    while (key[h] != c[t]) h = (h + 1) & (BB_TAB - 1);
+                    ix[t] = loc[h];
                 }
             }
             const int64_t o = ob + (int64_t)j * 32;
