@@ -358,7 +358,8 @@ struct RowSkip {
 };
 void block_sweep(apcloud_ctx *c, int which, const float *x, float *y, const float *b, const GmresState *st,
                  RowSkip skip, int keep, bool pdl);
-void block_product(apcloud_ctx *c, int which, const float *x, float *y, const GmresState *st, RowSkip skip);
+// pdl: launched as a programmatic dependent of the sweep before it
+void block_product(apcloud_ctx *c, int which, const float *x, float *y, const GmresState *st, RowSkip skip, bool pdl);
 int block_keep(double fraction);   // the `keep` of block_sweep that keeps this fraction of the matrix in L2
 double *poisson_rhs(apcloud_ctx *c, const double *g);  // b of the Poisson system into c->b
 apcloud_status tune_spmv(apcloud_ctx *c, double *ms_out);      // ms per sweep at 64/128/256/512 threads

@@ -1957,7 +1957,9 @@ void arnoldi_product(apcloud_ctx *c, const T *val, const Krylov<T> &K, const T *
     const int n = c->n_tot;
     if constexpr (sizeof(T) == 4) {
         if (K.blocks >= 0) {
-            block_product(c, K.blocks, (const float *)z, (float *)K.w, (const GmresState *)st, skip);
+            // right after the polynomial's sweeps, which write nothing it reads before its wait but z
+            block_product(c, K.blocks, (const float *)z, (float *)K.w, (const GmresState *)st, skip,
+                          K.pdeg > 1 && c->pdl_on);
             return;
         }
     }

@@ -387,14 +387,20 @@ void block_sweep(apcloud_ctx *c, int which, const float *x, float *y, const floa
                    b, st, skip, keep);
 }
 
-void block_product(apcloud_ctx *c, int which, const float *x, float *y, const GmresState *st, RowSkip skip) {
+void block_product(apcloud_ctx *c, int which, const float *x, float *y, const GmresState *st, RowSkip skip, bool pdl) {
     const int nblk = div_up(c->n_tot, BL_ROWS);
     auto kern = k_block_rows<false, float4>;
     const float4 *val = ptr<float4>(which ? c->bl_A32 : c->bl_B32);
-    APC_LAUNCH(c, K_SPMV, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
-               (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
-               (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx), val, c->n_tot, x, y,
-               (const float *)nullptr, st, skip, 0);
+    if (pdl)
+        APC_LAUNCH_PDL(c, K_SPMV, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
+                       (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
+                       (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx), val, c->n_tot, x,
+                       y, (const float *)nullptr, st, skip, 0);
+    else
+        APC_LAUNCH(c, K_SPMV, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
+                   (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
+                   (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx), val, c->n_tot, x, y,
+                   (const float *)nullptr, st, skip, 0);
 }
 
 int block_keep(double fraction) { return fraction >= 1.0 ? BL_KEEP : (int)(BL_KEEP * fraction); }
