@@ -219,7 +219,10 @@ apcloud_status gather_field(apcloud_ctx *c, double *phi_p, double *ex, double *e
     const int64_t dstride = ((int64_t)n + 31) / 32 * 32;
     const double ext = c->P.hi[0] - c->P.lo[0];
     const double unit = ldexp(ext, -(KEY_DEPTH + 1));
-    APC_LAUNCH(c, K_DERIV, div_up(n, 128), 128, 0, k_derivs, ptr<uint32_t>(c->slice_w), ptr<uint32_t>(c->slice_off),
+    // few nodes: single warps, so that their FP64 work spreads over the SMs (1500
+    // nodes in blocks of 128 are 12 SMs' work: 43 us)
+    const int db = n < 128 * 4 * sm_count() ? 32 : 128;
+    APC_LAUNCH(c, K_DERIV, div_up(n, db), db, 0, k_derivs, ptr<uint32_t>(c->slice_w), ptr<uint32_t>(c->slice_off),
                ptr<int32_t>(c->ell_col), ptr<double>(c->D), dstride, ptr<double>(c->phi), n, nf,
                ptr<int4>(c->node_ic), c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, nf32);
     if (mixed)

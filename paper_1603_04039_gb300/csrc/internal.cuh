@@ -345,6 +345,7 @@ apcloud_status build_octree(apcloud_ctx *c, const double *x, const double *y, co
                             const int64_t *h_offsets, int nbeams);
 apcloud_status node_beams(apcloud_ctx *c, int32_t *out);
 apcloud_status refresh_lowp(apcloud_ctx *c);          // FP32/FP16 matrix copies from the FP64 values
+int sm_count();   // SMs of the current device
 // Block-local copy of the sweep matrix (sweep.cu): its chunk count (to
 // *d_total), then, with bl_chunks known, the copy
 apcloud_status count_blocks(apcloud_ctx *c, uint32_t *d_total);

@@ -377,25 +377,26 @@ __device__ __forceinline__ int leaf_at(const int32_t *first, int lo, int hi, int
 
 // Leaf and key-sorted position of every particle in the caller's order (read
 // by the gather and the deposit, so that neither needs a search or a gather
-// through the permutation), a tile of PL_TILE sorted particles per block.
-// While the two arrays fit L2 the 4-byte stores go straight to their random
-// places.  Larger sets (BUCKET) would fetch and write back a 32-byte sector
+// through the permutation), a tile of sorted particles per block.  While the
+// two arrays fit L2 the 4-byte stores go straight to their random places (tiles
+// of PL_SMALL, so that small sets reach all SMs: 15 us for 1e5 particles, 26 in
+// tiles of 8192; 192 and 202 for 1e7).  Larger sets (BUCKET) would fetch and write back a 32-byte sector
 // per store: the tile is ordered by destination window first and appended to
 // the windows' lists (a permutation fills every window exactly), and
 // k_particle_place stores window by window, inside L2.
-constexpr int PL_TILE = 8192, PL_T = 1024, PL_WIN = 2048;   // most windows
+constexpr int PL_SMALL = 1024, PL_TILE = 8192, PL_T = 1024, PL_WIN = 2048;   // most windows
 constexpr int PL_WBITS = 14;                               // particles per window: 128 KB of the two arrays
 template <bool BUCKET>
 __global__ void __launch_bounds__(PL_T) k_particle_leaf(const int32_t *__restrict__ first, int n_leaf,
                                                         const uint32_t *__restrict__ perm, int64_t n,
                                                         int32_t *__restrict__ pleaf, int32_t *__restrict__ spos,
-                                                        int wbits, uint32_t *__restrict__ cursor,
+                                                        int tile, int wbits, uint32_t *__restrict__ cursor,
                                                         uint32_t *__restrict__ bp) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int range[2];
     __shared__ uint32_t wtot[PL_T / 32];
-    const int64_t i0 = (int64_t)blockIdx.x * PL_TILE;
-    const int m = (int)(n - i0 < PL_TILE ? n - i0 : PL_TILE);
+    const int64_t i0 = (int64_t)blockIdx.x * tile;   // BUCKET: tile = PL_TILE
+    const int m = (int)(n - i0 < tile ? n - i0 : tile);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     uint32_t *cnt = reinterpret_cast<uint32_t *>(smem), *gof = cnt + PL_WIN;
     if (tid < 2) range[tid] = leaf_at(first, 0, n_leaf, (int)(tid == 0 ? i0 : i0 + m - 1));
@@ -405,7 +406,7 @@ __global__ void __launch_bounds__(PL_T) k_particle_leaf(const int32_t *__restric
     const int ja = range[0], jb = range[1] + 1;
     if (!BUCKET) {
 #pragma unroll 4
-        for (int t = tid; t < m; t += PL_T) {
+        for (int t = tid; t < m; t += blockDim.x) {
             const int i = (int)(i0 + t);
             const uint32_t p = __ldcs(perm + i);
             if (p >= n) continue;   // only after a sort that gave up
@@ -793,8 +794,8 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
     const uint32_t *perm = ptr<uint32_t>(c->val[c->kbuf]);
     if (n > 0) {
         if (8 * n <= PL_DIRECT_BYTES) {
-            APC_LAUNCH(c, K_TREE, div_up(n, PL_TILE), PL_T, 0, k_particle_leaf<false>, (const int32_t *)lf, (int)nleaf,
-                       perm, n, pl, sp, 0, (uint32_t *)nullptr, (uint32_t *)nullptr);
+            APC_LAUNCH(c, K_TREE, div_up(n, PL_SMALL), PL_SMALL / 4, 0, k_particle_leaf<false>, (const int32_t *)lf,
+                       (int)nleaf, perm, n, pl, sp, PL_SMALL, 0, (uint32_t *)nullptr, (uint32_t *)nullptr);
         } else {
             int wbits = PL_WBITS;
             while ((n - 1) >> wbits >= PL_WIN) ++wbits;
@@ -806,7 +807,7 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
             APC_CUDA(c, cudaFuncSetAttribute(k_particle_leaf<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             APC_CUDA(c, cudaFuncSetAttribute(k_particle_place, cudaFuncAttributeMaxDynamicSharedMemorySize, wsm));
             APC_LAUNCH(c, K_TREE, div_up(n, PL_TILE), PL_T, smem, k_particle_leaf<true>, (const int32_t *)lf,
-                       (int)nleaf, perm, n, pl, sp, wbits, cursor, bp);
+                       (int)nleaf, perm, n, pl, sp, PL_TILE, wbits, cursor, bp);
             if (wbits == PL_WBITS)
                 APC_LAUNCH(c, K_TREE, div_up(n, 1 << PL_WBITS), 1024, wsm, k_particle_place, (const uint32_t *)bp, n,
                            pl, sp);

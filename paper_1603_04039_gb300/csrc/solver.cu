@@ -116,8 +116,8 @@ __device__ void final_sums(const double *partial, int nblk, int nk, double *sm, 
 //    charge goes to its key-sorted position (recorded by the tree build); the
 //    scattered stores land in an array that L2 keeps (evict-last hint) while
 //    the caller's charges stream through (evict-first);
-//  * k_deposit, one thread per leaf: the leaf's sorted charges (a contiguous
-//    range) summed in order, one FP64 add per particle -- a warp-wide tree
+//  * k_deposit, one thread per leaf (few leaves: one warp): the leaf's sorted charges (a contiguous
+//    range) summed in a fixed order, one FP64 add per particle -- a warp-wide tree
 //    reduction per leaf would cost 32 lanes of FP64 adds at every step on
 //    this GPU's narrow FP64 pipe.
 // The summation order is fixed, so the result does not depend on timing.
@@ -176,6 +176,30 @@ __global__ void __launch_bounds__(256) k_deposit(const double *__restrict__ qs, 
     }
     const double p3 = __longlong_as_double((long long)(1023 + 3 * ic[j].w) << 52);
     rho_m[j] = (Q * inv_ext3) * p3;
+}
+
+// The same with a warp per leaf, for few leaves: they may hold thousands of
+// particles each, which a thread of its own reads at memory latency (92 us for
+// 1e5 particles on 1400 leaves), and the FP64 pipe has room for a tree of adds
+// per leaf.
+__global__ void __launch_bounds__(256) k_deposit_warp(const double *__restrict__ qs, const int32_t *__restrict__ first,
+                                                      const int32_t *__restrict__ count, const int4 *__restrict__ ic,
+                                                      int n_int, double inv_ext3, double *__restrict__ rho_m) {
+    const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (j >= n_int) return;
+    const int c = count[j];
+    const double *q = qs + first[j];
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < c; i += 64) {
+        const double a = __ldcs(q + i), b = i + 32 < c ? __ldcs(q + i + 32) : 0.0;
+        s0 += a;
+        s1 += b;
+    }
+    s0 += s1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    if (lane == 0) rho_m[j] = (s0 * inv_ext3) * __longlong_as_double((long long)(1023 + 3 * ic[j].w) << 52);
 }
 
 __global__ void k_bcopy(const int32_t *__restrict__ owner, int n_int, int n_bnd, double *__restrict__ v) {
@@ -1166,12 +1190,16 @@ __global__ void k_add_f32(double *__restrict__ u, float *__restrict__ e, int n) 
     if (i < n) { u[i] += (double)e[i]; e[i] = 0.f; }
 }
 
+}  // namespace
+
 int sm_count() {
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms > 0 ? sms : 152;
 }
+
+namespace {
 
 constexpr double KEEP_ALL = 0.75, KEEP_PART = 0.3;   // sweep_keep_bytes
 
@@ -2347,9 +2375,14 @@ apcloud_status deposit(apcloud_ctx *c, const double *q, double q_uniform) {
         APC_LAUNCH(c, K_DEPOSIT, div_up(c->N, 256 * CS_PER), 256, 0, k_charge_sort, q,
                    (const int32_t *)ptr<int32_t>(c->spos), c->N, qs);
     }
-    APC_LAUNCH(c, K_DEPOSIT, div_up(n, 256), 256, 0, k_deposit, (const double *)qs, q_uniform,
-               ptr<int32_t>(c->leaf_first), ptr<int32_t>(c->leaf_count), ptr<int4>(c->node_ic), n,
-               1.0 / (ext * ext * ext), rm);
+    // a warp per leaf while its five extra adds per leaf stay below 5 us of the FP64 pipe
+    if (qs && n < 64 * sm_count())
+        APC_LAUNCH(c, K_DEPOSIT, div_up(n, 8), 256, 0, k_deposit_warp, (const double *)qs, ptr<int32_t>(c->leaf_first),
+                   ptr<int32_t>(c->leaf_count), ptr<int4>(c->node_ic), n, 1.0 / (ext * ext * ext), rm);
+    else
+        APC_LAUNCH(c, K_DEPOSIT, div_up(n, 256), 256, 0, k_deposit, (const double *)qs, q_uniform,
+                   ptr<int32_t>(c->leaf_first), ptr<int32_t>(c->leaf_count), ptr<int4>(c->node_ic), n,
+                   1.0 / (ext * ext * ext), rm);
     APC_LAUNCH(c, K_DEPOSIT, div_up(c->n_bnd, 256), 256, 0, k_bcopy, ptr<int32_t>(c->bowner), n, c->n_bnd, rm);
     // sorted position and charge per particle, rho_M per node
     account(c, K_DEPOSIT, (q ? 12.0 * c->N : 0.0) + 8.0 * nt, q ? (double)c->N : (double)n);
