@@ -355,7 +355,7 @@ apcloud_status apcloud_set_graphs(apcloud_ctx *ctx, int enable);
  * the loads of 1 or 4 stencil entries issued ahead of their multiply-adds
  * (the sum keeps its order either way), and -- for the FP16 sweeps and FP32
  * Arnoldi products of the mixed form -- on the sliced ELL and on its
- * block-local copy (a block's distinct columns in shared memory, 16-bit
+ * block-local copy (a block's distinct columns in shared memory, 12-bit
  * indices; one launch shape; same entries in the same order per row).  The
  * solves run on scratch vectors and the
  * graphs they capture are released; bit 1 times the stencil build (neighbour
@@ -379,12 +379,12 @@ apcloud_status apcloud_set_launch_shape(apcloud_ctx *ctx, int spmv_block, int sp
 /* L2 residency of the FP16 sweep matrix (block-local copy, the mixed form's
  * polynomial preconditioner).  The sweeps of one polynomial application read
  * the whole matrix one after another; a sweep loads keep_bytes of matrix bytes
- * (4 per stored entry, rounded down to sixteenths of the matrix) as ordinary
+ * (3.5 per stored entry, rounded down to sixteenths of the matrix) as ordinary
  * loads and the rest as evict-first lines, so that the rest replaces itself in
  * L2 and the kept part, evenly spread over the matrix, is still there for the
  * next sweep.  keep_bytes = -1 (the default): all of the matrix when it and
- * the sweep's vectors (12 bytes per row) take at most 3/4 of the L2, else 0.3
- * of the L2; 0: every matrix load evict-first; larger than the matrix: none.
+ * the sweep's vectors (12 bytes per row) take at most 3/4 of the L2, 0.3 of the
+ * L2 up to twice the L2, none beyond; 0: every matrix load evict-first; larger than the matrix: none.
  * Results are bit-identical for every value (the same loads in the same
  * order).  APCLOUD_E_INVALID for keep_bytes < -1.  The getter writes the
  * value in effect for the current node set (the automatic choice resolved;

@@ -236,10 +236,10 @@ struct apcloud_ctx {
     apc::DBuf ell_A32, ell_B32;  // FP32 copies for the inner iterations of the mixed form
     apc::DBuf ell_A16, ell_B16;  // FP16 copies for the preconditioner sweeps of the mixed form
     // block-local copy of the sweep matrix (sweep.cu): slice offsets in chunks, row
-    // lengths, the blocks' lists of other blocks' nodes, 16-bit indices, FP16 and
+    // lengths, the blocks' lists of other blocks' nodes, 12-bit indices, FP16 and
     // FP32 values; tried: built since the operators were, ok: every block's list fits
     apc::DBuf bl_w4, bl_off, bl_len, bl_hlist, bl_hcnt, bl_idx, bl_A, bl_B, bl_A32, bl_B32;
-    int64_t bl_chunks = 0;     // 32-lane chunks of 4 entries
+    int64_t bl_chunks = 0;     // 32-lane chunks of 8 entries
     bool bl_ok = false, bl_tried = false;
     apc::DBuf stencil_ovf;     // nodes whose k-ring outgrew MAXC_FAST candidates
     apc::DBuf beam_part;        // per-beam norms: partial sums, BSQ_CH per beam

@@ -1211,24 +1211,24 @@ int64_t l2_bytes() {
 }
 
 // Bytes a sweep reads per stored entry of the block-local copy (FP16 value and
-// 16-bit index) and per row (x and b read, y written, FP32).
-constexpr double SWEEP_ENTRY_BYTES = 4.0, SWEEP_ROW_BYTES = 12.0;
+// 12-bit index) and per row (x and b read, y written, FP32).
+constexpr double SWEEP_ENTRY_BYTES = 3.5, SWEEP_ROW_BYTES = 12.0;
 
-double sweep_matrix_bytes(const apcloud_ctx *c) { return SWEEP_ENTRY_BYTES * 128.0 * (double)c->bl_chunks; }
+double sweep_matrix_bytes(const apcloud_ctx *c) { return SWEEP_ENTRY_BYTES * 256.0 * (double)c->bl_chunks; }
 
 }  // namespace
 
 // Matrix bytes the sweeps read with ordinary loads when left to the library:
 // all of them when the matrix and the sweep's vectors fit in KEEP_ALL of the
-// L2; else KEEP_PART of the L2 (the rest holds the vectors and the streamed
-// lines).  Solve times with 0, 20, 40, 50 MB and all of it kept: 21.3, 19.4,
-// 18.8, 18.6, 18.4 ms at 4.9e5 rows; 48.9, 46.9, 45.5, 45.9, 55.5 ms at 1.05e6;
-// 127.6, 127.6, 129.3, 129.2, 130.6 ms at 4.5e6.
+// L2; KEEP_PART of the L2 up to twice the L2 (the rest holds the vectors and the
+// streamed lines); none beyond.  Solve times with 0, 20, 40, 50 MB and all of it
+// kept: 21.3, 19.4, 18.8, 18.6, 18.4 ms at 4.9e5 rows; 48.9, 46.9, 45.5, 45.9,
+// 55.5 ms at 1.05e6; 127.6, 127.6, 129.3, 129.2, 130.6 ms at 4.5e6.
 int64_t sweep_keep_bytes(const apcloud_ctx *c) {
     if (c->sweep_keep >= 0) return c->sweep_keep;
     const double l2 = (double)l2_bytes();
     const double tot = sweep_matrix_bytes(c) + SWEEP_ROW_BYTES * (double)c->n_tot;
-    return tot <= KEEP_ALL * l2 ? INT64_MAX : (int64_t)(KEEP_PART * l2);
+    return tot <= KEEP_ALL * l2 ? INT64_MAX : (tot <= 2.0 * l2 ? (int64_t)(KEEP_PART * l2) : 0);
 }
 
 namespace {
@@ -2315,8 +2315,8 @@ apcloud_status gmres_core(apcloud_ctx *c, const T *val, const T *b, T *u, double
             const double sweeps = (K.pdeg <= 1 || K.ilu) ? 0.0 : (double)(K.pdeg - 1) * (je + (K.Z ? 0 : 1));
             const double prods = je + 1.0;
             const double sb = K.hval ? 2.0 : vb;
-            const double cb = K.blocks >= 0 ? 2.0 : 4.0;   // index bytes per entry of a sweep or product
-            const double pcb = K.blocks >= 0 ? (2.0 * je + 4.0) / prods : 4.0;   // the residual's are 4
+            const double cb = K.blocks >= 0 ? 1.5 : 4.0;   // index bytes per entry of a sweep or product
+            const double pcb = K.blocks >= 0 ? (1.5 * je + 4.0) / prods : 4.0;   // the residual's are 4
             account(c, K_SPMV, ((vb + pcb) * nnz + 2.0 * vb * dn) * prods, 2.0 * nnz * prods);
             account(c, K_SWEEP, ((sb + cb) * nnz + 3.0 * vb * dn) * sweeps, 2.0 * nnz * sweeps);
         }
