@@ -547,7 +547,7 @@ __global__ void k_copy_nf(const double *__restrict__ nf, int n, double *__restri
     if (t >= (int64_t)n * NCOL) return;
     int64_t j = t / NCOL;
     int r = (int)(t % NCOL);
-    o[t] = nf[j * 12 + 1 + r];
+    o[t] = nf[j * NODE_RECORD + 1 + r];
 }
 }  // namespace
 

@@ -21,7 +21,11 @@ namespace apc {
 
 namespace {
 
-constexpr int NF = 12;  // per-node record: phi, 9 derivatives, 2 pad
+// per-node record: phi, 9 derivatives, the node's centre, 1 pad.  A centre
+// computed per particle from the integer coordinates cost 9 of the 33 FP64
+// instructions of the FP64 particle pass, which the FP64 pipe bounds (824 us for
+// 2e7 particles, 1183 before); here each node computes it once, the same way.
+constexpr int NF = NODE_RECORD;
 // compact per-node record of the mixed form's particle pass, 80 bytes in 4-byte
 // words: phi and the node centre (FP64, words 0-7), gradient and Hessian
 // fx fy fz fxx fxy fxz fyy fyz fzz (FP32, words 8-16), pad
@@ -57,13 +61,17 @@ __global__ void k_derivs(const uint32_t *__restrict__ sw, const uint32_t *__rest
     o[0] = p0;
 #pragma unroll
     for (int r = 0; r < NCOL; ++r) o[1 + r] = acc[r];
-    o[10] = 0.0;
-    o[11] = 0.0;
+    const int4 q = ic[j];
+    const double c0 = __dadd_rn(lo0, __dmul_rn((double)q.x, unit)), c1 = __dadd_rn(lo1, __dmul_rn((double)q.y, unit)),
+                 c2d = __dadd_rn(lo2, __dmul_rn((double)q.z, unit));
+    o[10] = c0;
+    o[11] = c1;
+    o[12] = c2d;
+    o[13] = 0.0;
     if (nf32) {
-        const int4 q = ic[j];
         double2 *c2 = reinterpret_cast<double2 *>(nf32 + (int64_t)j * NF32);
-        c2[0] = make_double2(p0, __dadd_rn(lo0, __dmul_rn((double)q.x, unit)));
-        c2[1] = make_double2(__dadd_rn(lo1, __dmul_rn((double)q.y, unit)), __dadd_rn(lo2, __dmul_rn((double)q.z, unit)));
+        c2[0] = make_double2(p0, c0);
+        c2[1] = make_double2(c1, c2d);
         float4 *f4 = reinterpret_cast<float4 *>(nf32 + (int64_t)j * NF32 + 8);
         f4[0] = make_float4((float)acc[0], (float)acc[1], (float)acc[2], (float)acc[3]);
         f4[1] = make_float4((float)acc[4], (float)acc[5], (float)acc[6], (float)acc[7]);
@@ -82,10 +90,11 @@ __device__ __forceinline__ int leaf_of(const uint64_t *anchor, int n, uint64_t v
 
 // Second-order Taylor expansion about the leaf centre (Section 3.2 step 3):
 // phi_p = phi + g.r + r.H.r / 2, E_p = g + H r (E = grad phi, Section 2).
-__device__ __forceinline__ void taylor(const double *__restrict__ nf, int j, double r0, double r1, double r2,
+__device__ __forceinline__ void taylor(const double *__restrict__ nf, int j, double x0, double x1, double x2,
                                        double &php, double &ex, double &ey, double &ez) {
     const double2 *f2 = reinterpret_cast<const double2 *>(nf + (int64_t)j * NF);
-    const double2 a = f2[0], b = f2[1], c = f2[2], d = f2[3], e = f2[4];
+    const double2 a = f2[0], b = f2[1], c = f2[2], d = f2[3], e = f2[4], ctr = f2[5];
+    const double r0 = x0 - ctr.x, r1 = x1 - ctr.y, r2 = x2 - f2[6].x;
     // a = (phi, fx), b = (fy, fz), c = (fxx, fxy), d = (fxz, fyy), e = (fyz, fzz)
     const double hr0 = c.x * r0 + c.y * r1 + d.x * r2;
     const double hr1 = c.y * r0 + d.y * r1 + e.x * r2;
@@ -99,19 +108,14 @@ __device__ __forceinline__ void taylor(const double *__restrict__ nf, int j, dou
 
 __global__ void __launch_bounds__(256) k_gather_leaf(
     const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z, int64_t n,
-    double lo0, double lo1, double lo2, double unit, const int32_t *__restrict__ pleaf, const int4 *__restrict__ ic,
-    const double *__restrict__ nf, double *__restrict__ php, double *__restrict__ ex, double *__restrict__ ey,
+    const int32_t *__restrict__ pleaf, const double *__restrict__ nf, double *__restrict__ php, double *__restrict__ ex, double *__restrict__ ey,
     double *__restrict__ ez) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int j = __ldcs(pleaf + i);
     const double p0 = __ldcs(x + i), p1 = __ldcs(y + i), p2 = __ldcs(z + i);
     double v, gx, gy, gz;
-    const int4 q = ic[j];
-    const double r0 = p0 - __dadd_rn(lo0, __dmul_rn((double)q.x, unit));
-    const double r1 = p1 - __dadd_rn(lo1, __dmul_rn((double)q.y, unit));
-    const double r2 = p2 - __dadd_rn(lo2, __dmul_rn((double)q.z, unit));
-    taylor(nf, j, r0, r1, r2, v, gx, gy, gz);
+    taylor(nf, j, p0, p1, p2, v, gx, gy, gz);
     if (php) __stcs(php + i, v);
     if (ex) __stcs(ex + i, gx);
     if (ey) __stcs(ey + i, gy);
@@ -171,8 +175,8 @@ __global__ void __launch_bounds__(GT) k_gather_leaf32(
 }
 
 __global__ void k_gather(const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
-                         int64_t n, double lo0, double lo1, double lo2, double s, int shift, double unit,
-                         const int64_t *__restrict__ offs, int nb, int L, const uint64_t *__restrict__ anchor, int n_int, const int4 *__restrict__ ic,
+                         int64_t n, double lo0, double lo1, double lo2, double s, int shift,
+                         const int64_t *__restrict__ offs, int nb, int L, const uint64_t *__restrict__ anchor, int n_int,
                          const double *__restrict__ nf, double *__restrict__ php, double *__restrict__ ex,
                          double *__restrict__ ey, double *__restrict__ ez) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -196,12 +200,8 @@ __global__ void k_gather(const double *__restrict__ x, const double *__restrict_
         pre = (uint64_t)lo << (3 * L);
     }
     const int j = leaf_of(anchor, n_int, pre | morton(cc[0], cc[1], cc[2]));
-    const int4 q = ic[j];
-    const double r0 = p[0] - __dadd_rn(lo0, __dmul_rn((double)q.x, unit));
-    const double r1 = p[1] - __dadd_rn(lo1, __dmul_rn((double)q.y, unit));
-    const double r2 = p[2] - __dadd_rn(lo2, __dmul_rn((double)q.z, unit));
     double v, gx, gy, gz;
-    taylor(nf, j, r0, r1, r2, v, gx, gy, gz);
+    taylor(nf, j, p[0], p[1], p[2], v, gx, gy, gz);
     if (php) php[i] = v;
     if (ex) ex[i] = gx;
     if (ey) ey[i] = gy;
@@ -230,15 +230,14 @@ apcloud_status gather_field(apcloud_ctx *c, double *phi_p, double *ex, double *e
                    (const int32_t *)ptr<int32_t>(c->pleaf), (const float *)nf32, phi_p, ex, ey, ez);
     else
         APC_LAUNCH(c, K_GATHER, div_up(c->N, 256), 256, 0, k_gather_leaf, c->px, c->py, c->pz, c->N,
-                   c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, (const int32_t *)ptr<int32_t>(c->pleaf),
-                   ptr<int4>(c->node_ic), (const double *)nf, phi_p, ex, ey, ez);
+                   (const int32_t *)ptr<int32_t>(c->pleaf), (const double *)nf, phi_p, ex, ey, ez);
     // node pass: operator (72 B), column (4 B) and neighbour value (8 B) per
-    // stencil entry plus the 96 B record (and the 80 B compact record of the
+    // stencil entry plus the 112 B record (and the 80 B compact record of the
     // mixed form); particle pass: leaf index and position in (28 B), phi and E
-    // out (32 B), and each leaf's record once (FP64: 96 B and the 16 B centre;
-    // mixed: the 80 B compact record)
-    account(c, K_DERIV, 84.0 * c->sum_m + (mixed ? 200.0 : 104.0) * n, 19.0 * c->sum_m);
-    account(c, K_GATHER, 60.0 * c->N + (mixed ? 80.0 : 112.0) * n, 38.0 * c->N);
+    // out (32 B), and each leaf's record once (FP64: 112 B; mixed: the 80 B
+    // compact record)
+    account(c, K_DERIV, 84.0 * c->sum_m + (mixed ? 216.0 : 136.0) * n, 19.0 * c->sum_m);
+    account(c, K_GATHER, 60.0 * c->N + (mixed ? 80.0 : 112.0) * n, 29.0 * c->N);
     return cuda_check(c, cudaGetLastError(), "gather");
 }
 
@@ -296,10 +295,8 @@ apcloud_status interpolate_phi(apcloud_ctx *c, const double *x, const double *y,
                                double *phi) {
     const double ext = c->P.hi[0] - c->P.lo[0];
     const double s = ldexp(1.0, KEY_DEPTH) / ext;
-    const double unit = ldexp(ext, -(KEY_DEPTH + 1));
     APC_LAUNCH(c, K_GATHER, div_up(n, 256), 256, 0, k_gather, x, y, z, n, c->P.lo[0], c->P.lo[1], c->P.lo[2], s,
-               KEY_DEPTH - c->L, unit, (const int64_t *)nullptr, 1, c->L, ptr<uint64_t>(c->leaf_anchor), c->n_int,
-               ptr<int4>(c->node_ic),
+               KEY_DEPTH - c->L, (const int64_t *)nullptr, 1, c->L, ptr<uint64_t>(c->leaf_anchor), c->n_int,
                ptr<double>(c->nodefield), phi, (double *)nullptr, (double *)nullptr, (double *)nullptr);
     return cuda_check(c, cudaGetLastError(), "interpolate");
 }
