@@ -2317,8 +2317,9 @@ apcloud_status gmres_core(apcloud_ctx *c, const T *val, const T *b, T *u, double
             const double sb = K.hval ? 2.0 : vb;
             const double cb = K.blocks >= 0 ? 1.5 : 4.0;   // index bytes per entry of a sweep or product
             const double pcb = K.blocks >= 0 ? (1.5 * je + 4.0) / prods : 4.0;   // the residual's are 4
-            account(c, K_SPMV, ((vb + pcb) * nnz + 2.0 * vb * dn) * prods, 2.0 * nnz * prods);
-            account(c, K_SWEEP, ((sb + cb) * nnz + 3.0 * vb * dn) * sweeps, 2.0 * nnz * sweeps);
+            const double ent = K.blocks >= 0 ? nnz - dn : nnz;             // the copy holds no diagonal
+            account(c, K_SPMV, ((vb + pcb) * ent + 2.0 * vb * dn) * prods, 2.0 * nnz * prods);
+            account(c, K_SWEEP, ((sb + cb) * ent + 3.0 * vb * dn) * sweeps, 2.0 * nnz * sweeps);
         }
         const bool dcgs = gs_dcgs(K, jmax) || bdcgs_on(K, jmax), fused = gs_fused(K, jmax) && !dcgs;
         for (int j = 0; j < je; ++j) {
