@@ -397,7 +397,7 @@ void apcloud_destroy(apcloud_ctx *c) {
                     &c->pz0, &c->pz1, &c->pt, &c->zbasis, &c->ell_rd, &c->ell_A16, &c->ell_B16, &c->beam_off, &c->leaf_beam,
                     &c->beam_rng, &c->beam_norm, &c->beam_r2, &c->beam_done, &c->node_beam, &c->tile_act,
                     &c->bk_items, &c->bk_ioff, &c->bk_d, &c->bk_i, &c->bl_w4, &c->bl_off, &c->bl_len, &c->bl_hlist, &c->bl_hcnt, &c->bl_idx, &c->stencil_ovf,
-                    &c->bl_A, &c->bl_B, &c->bl_A32, &c->bl_B32, &c->tune_b, &c->tune_x, &c->beam_part, &c->ilu_lrows, &c->ilu_urows, &c->ilu_lrp, &c->ilu_urp,
+                    &c->bl_A, &c->bl_B, &c->bl_A32, &c->bl_B32, &c->bl_dg, &c->tune_b, &c->tune_x, &c->beam_part, &c->ilu_lrows, &c->ilu_urows, &c->ilu_lrp, &c->ilu_urp,
                     &c->ilu_lcol, &c->ilu_ucol, &c->ilu_lval, &c->ilu_uval, &c->ilu_dinv,
                     &c->ilu_loff, &c->ilu_uoff, &c->res_words, &c->res_state};
     for (DBuf *b : bufs) free_buf(c, *b);

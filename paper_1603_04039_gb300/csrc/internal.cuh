@@ -71,7 +71,7 @@ struct GraphKey {
     int tsize, n, jmax, pdeg, nblk, spmv_bs, pdl;
     unsigned mask;
     int64_t ldv, skeep;
-    const void *p[32];
+    const void *p[40];
 };
 
 // Arnoldi step j >= 1 of a captured cycle sits in an IF node whose condition
@@ -241,7 +241,8 @@ struct apcloud_ctx {
     // FP32 values; tried: built since the operators were, ok: every block's list fits
     apc::DBuf bl_w4, bl_off, bl_len, bl_hlist, bl_hcnt, bl_idx, bl_A, bl_B, bl_A32, bl_B32;
     int64_t bl_chunks = 0;     // 32-lane chunks of 8 entries
-    bool bl_ok = false, bl_tried = false;
+    bool bl_ok = false, bl_tried = false, bl_unit = true;   // unit: every diagonal is 1
+    apc::DBuf bl_dg;           // diagonals: sweeps B, A, products B, A
     apc::DBuf stencil_ovf;     // nodes whose k-ring outgrew MAXC_FAST candidates
     apc::DBuf beam_part;        // per-beam norms: partial sums, BSQ_CH per beam
     apc::DBuf tune_b, tune_x;   // autotuner: right-hand side and iterate of its timed restart cycles

@@ -2243,7 +2243,8 @@ apcloud_status run_cycle(apcloud_ctx *c, const T *val, const T *b, T *u, const K
                            K.blocks >= 0 ? c->bl_hlist.p : nullptr, K.blocks >= 0 ? c->bl_off.p : nullptr,
                            K.blocks >= 0 ? c->bl_len.p : nullptr, K.blocks >= 0 ? c->bl_hcnt.p : nullptr,
                            K.blocks >= 0 ? (K.blocks ? c->bl_A.p : c->bl_B.p) : nullptr,
-                           K.blocks >= 0 ? (K.blocks ? c->bl_A32.p : c->bl_B32.p) : nullptr};
+                           K.blocks >= 0 ? (K.blocks ? c->bl_A32.p : c->bl_B32.p) : nullptr,
+                           K.blocks >= 0 && !c->bl_unit ? c->bl_dg.p : nullptr};
         static_assert(sizeof p <= sizeof key.p, "graph key holds every buffer address");
         for (size_t i = 0; i < sizeof p / sizeof p[0]; ++i) key.p[i] = p[i];
         GraphEntry *g = find_graph(c, key);

@@ -27,7 +27,7 @@
 // (chunk j of lane l at 32 j + l in its slice): 16 bytes of FP16 values, 8 and 4
 // bytes of indices (the products load FP32 values instead).  Nine rows in ten
 // have 17 to 24 entries, three chunks.  The diagonal, first in every row and 1
-// after the scaling, is not stored.  Rows keep their entries in stored order: the
+// after the scaling, is stored apart and read only where it is not.  Rows keep their entries in stored order: the
 // results have the same bits as on the ELL.  Lanes past their row's length load
 // nothing.
 #include <cuda_fp16.h>
@@ -54,8 +54,9 @@ constexpr int BB_T = 512, BB_TAB = 8192, BB_LIST = 4096;   // threads, hash slot
 static_assert(BL_HMAX <= BB_LIST, "sorted in whole powers of two");
 
 // One block's columns outside its rows, sorted, and its entries in the layout
-// above.  A block with more than BL_HMAX such columns, or a diagonal that is not
-// 1, sets *bad: the system then stays on the ELL.
+// above.  A block with more than BL_HMAX such columns sets bit 0 of *bad: the
+// system then stays on the ELL.  A diagonal that is not 1 (column-scaled systems)
+// sets bit 1: the kernels then read the rows' diagonals from dg.
 // 281 us at 1.05e6 rows, most of it latency (350 with one column and one chunk's
 // values in flight per lane): three blocks per SM, a bitonic sort of some 1200
 // nodes each.
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(BB_T) k_block_build(
     const float *__restrict__ fB, const int32_t *__restrict__ msz, int n_int, int n, int nsl,
     const uint32_t *__restrict__ off4, int32_t *__restrict__ hlist, int32_t *__restrict__ hcnt,
     uint8_t *__restrict__ len, uint2 *__restrict__ idx, uint32_t *__restrict__ idx4, uint4 *__restrict__ A2,
-    uint4 *__restrict__ B2, float4 *__restrict__ A4, float4 *__restrict__ B4, unsigned *bad) {
+    uint4 *__restrict__ B2, float4 *__restrict__ A4, float4 *__restrict__ B4, float *__restrict__ dg, unsigned *bad) {
     extern __shared__ __align__(16) unsigned char smem[];
     int *key = reinterpret_cast<int *>(smem);                       // BB_TAB
     int *list = key + BB_TAB;                                       // BB_LIST
@@ -145,7 +146,12 @@ __global__ void __launch_bounds__(BB_T) k_block_build(
         const int64_t eb = (int64_t)soff[s] * 32 + lane + 32;   // past the diagonal
         if (r < n) {
             len[r] = (uint8_t)m;
-            if (fA[eb - 32] != 1.f || fB[eb - 32] != 1.f) atomicOr(bad, 1u);
+            // of the sweeps (FP16 values), then of the products, B before A
+            dg[r] = __half2float(hB[eb - 32]);
+            dg[n + r] = __half2float(hA[eb - 32]);
+            dg[2 * (int64_t)n + r] = fB[eb - 32];
+            dg[3 * (int64_t)n + r] = fA[eb - 32];
+            if (fA[eb - 32] != 1.f || fB[eb - 32] != 1.f) atomicOr(bad, 2u);
         }
         const int64_t ob = (int64_t)off4[s] * 32 + lane;
         for (int j = 0; j * BL_CE < w; ++j) {
@@ -306,12 +312,12 @@ struct Chunk32 {
 // The product has no work before its loads to hide behind and takes a third
 // more registers: three blocks per SM (38.3 us, 40.0 at four with half a row in
 // flight).
-template <bool SWEEP, class V>
+// DIAG: a diagonal that is not 1, from dg.
+template <bool SWEEP, class V, bool DIAG>
 __global__ void __launch_bounds__(BL_T, SWEEP ? 4 : 3) k_block_rows(
     const uint32_t *__restrict__ off4, const uint8_t *__restrict__ len, const int32_t *__restrict__ hlist,
     const int32_t *__restrict__ hcnt, const uint2 *__restrict__ idx, const uint32_t *__restrict__ idx4,
-    const V *__restrict__ val, int n,
-    const float *x, float *__restrict__ y, const float *__restrict__ b, const GmresState *__restrict__ st,
+    const V *__restrict__ val, const float *__restrict__ dg, int n, const float *x, float *__restrict__ y, const float *__restrict__ b, const GmresState *__restrict__ st,
     RowSkip skip, int keep) {
     __shared__ float xs[BL_ROWS + BL_HMAX];
     const int tid = threadIdx.x, blk = blockIdx.x, r0 = blk * BL_ROWS;
@@ -368,7 +374,7 @@ __global__ void __launch_bounds__(BL_T, SWEEP ? 4 : 3) k_block_rows(
     for (int q = 0; q < BL_RPT; ++q) {
         const int r = r0 + q * BL_T + tid, q1 = q + 1 < BL_RPT ? q + 1 : 0;
         const float own = xs[q * BL_T + tid];
-        float acc = own + 0.f;   // the diagonal's term
+        float acc = DIAG && act[q] ? fmaf(dg[r], own, 0.f) : own + 0.f;   // the diagonal's term
 #pragma unroll
         for (int j = 0; j < BL_CH; ++j) {
             if (j < nch[q]) acc = ch[j].dot(acc, xs);
@@ -404,7 +410,8 @@ apcloud_status build_blocks(apcloud_ctx *c) {
     uint2 *ix = reinterpret_cast<uint2 *>(ib);
     uint4 *A2 = ensure<uint4>(c, c->bl_A, ch + 1), *B2 = ensure<uint4>(c, c->bl_B, ch + 1);
     float4 *A4 = ensure<float4>(c, c->bl_A32, 2 * ch + 1), *B4 = ensure<float4>(c, c->bl_B32, 2 * ch + 1);
-    if (!hl || !hc || !len || !ib || !A2 || !B2 || !A4 || !B4) return APCLOUD_E_NOMEM;
+    float *dg = ensure<float>(c, c->bl_dg, 4 * (int64_t)n + 1);
+    if (!hl || !hc || !len || !ib || !A2 || !B2 || !A4 || !B4 || !dg) return APCLOUD_E_NOMEM;
     const int smem = BB_TAB * 4 + BB_LIST * 4 + BB_TAB * 2;
     APC_CUDA(c, cudaFuncSetAttribute(k_block_build, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     unsigned *bad = ptr<uint32_t>(c->dsmall) + 14;
@@ -414,11 +421,12 @@ apcloud_status build_blocks(apcloud_ctx *c) {
                (const __half *)ptr<__half>(c->ell_A16), (const __half *)ptr<__half>(c->ell_B16),
                (const float *)ptr<float>(c->ell_A32), (const float *)ptr<float>(c->ell_B32),
                (const int32_t *)ptr<int32_t>(c->msz), c->n_int, n, c->n_slices,
-               (const uint32_t *)ptr<uint32_t>(c->bl_off), hl, hc, len, ix, ib + 2 * ch, A2, B2, A4, B4, bad);
+               (const uint32_t *)ptr<uint32_t>(c->bl_off), hl, hc, len, ix, ib + 2 * ch, A2, B2, A4, B4, dg, bad);
     APC_CUDA(c, cudaGetLastError());
     unsigned b = 0;
     APC_TRY(read_back(c, &b, bad, sizeof b));
-    c->bl_ok = b == 0;
+    c->bl_ok = (b & 1u) == 0;
+    c->bl_unit = (b & 2u) == 0;
     c->bl_tried = true;
     return APCLOUD_OK;
 }
@@ -426,37 +434,39 @@ apcloud_status build_blocks(apcloud_ctx *c) {
 void block_sweep(apcloud_ctx *c, int which, const float *x, float *y, const float *b, const GmresState *st,
                  RowSkip skip, int keep, bool pdl) {
     const int nblk = div_up(c->n_tot, BL_ROWS);
-    auto kern = k_block_rows<true, uint4>;
+    auto kern = c->bl_unit ? k_block_rows<true, uint4, false> : k_block_rows<true, uint4, true>;
     const uint4 *val = ptr<uint4>(which ? c->bl_A : c->bl_B);
+    const float *dg = ptr<float>(c->bl_dg) + (int64_t)(which ? 1 : 0) * c->n_tot;
     if (pdl)
         APC_LAUNCH_PDL(c, K_SWEEP, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
                        (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
                        (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx),
-                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, c->n_tot, x,
+                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, dg, c->n_tot, x,
                        y, b, st, skip, keep);
     else
         APC_LAUNCH(c, K_SWEEP, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
                    (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
                    (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx),
-                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, c->n_tot, x, y,
+                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, dg, c->n_tot, x, y,
                    b, st, skip, keep);
 }
 
 void block_product(apcloud_ctx *c, int which, const float *x, float *y, const GmresState *st, RowSkip skip, bool pdl) {
     const int nblk = div_up(c->n_tot, BL_ROWS);
-    auto kern = k_block_rows<false, float4>;
+    auto kern = c->bl_unit ? k_block_rows<false, float4, false> : k_block_rows<false, float4, true>;
     const float4 *val = ptr<float4>(which ? c->bl_A32 : c->bl_B32);
+    const float *dg = ptr<float>(c->bl_dg) + (int64_t)(which ? 3 : 2) * c->n_tot;
     if (pdl)
         APC_LAUNCH_PDL(c, K_SPMV, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
                        (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
                        (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx),
-                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, c->n_tot, x,
+                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, dg, c->n_tot, x,
                        y, (const float *)nullptr, st, skip, 0);
     else
         APC_LAUNCH(c, K_SPMV, nblk, BL_T, 0, kern, (const uint32_t *)ptr<uint32_t>(c->bl_off),
                    (const uint8_t *)ptr<uint8_t>(c->bl_len), (const int32_t *)ptr<int32_t>(c->bl_hlist),
                    (const int32_t *)ptr<int32_t>(c->bl_hcnt), (const uint2 *)ptr<uint2>(c->bl_idx),
-                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, c->n_tot, x, y,
+                       (const uint32_t *)(ptr<uint32_t>(c->bl_idx) + 64 * c->bl_chunks), val, dg, c->n_tot, x, y,
                    (const float *)nullptr, st, skip, 0);
 }
 

@@ -42,3 +42,21 @@ def test_block_local_copy_gives_the_bits_of_the_ell(beams, n, depth, c, kw):
         out.append((rho.clone(), phi.clone(), i0["iters"], i1["iters"]))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert out[0][2:] == out[1][2:] and out[0][3] > 0
+
+
+def test_column_scaled_system():
+    """The closed-form column scaling leaves a diagonal that is not 1."""
+    from paper_1603_04039_gb300 import MPNN
+    ap = _cloud(1, 30000, 6, 0.3)
+    ap.deposit(q_uniform=1.0 / 30000, rtol=1e-10)
+    net = MPNN(seed=1)
+    out = []
+    for sorted_ in (0, 1):
+        ap.set_launch_shape(256, 4, 4, sorted_)
+        plain, i0 = ap.solve(rtol=1e-10)
+        scaled, i1 = ap.solve_learned(net, use=4, rtol=1e-10)
+        again, i2 = ap.solve(rtol=1e-10)
+        assert torch.equal(plain, again) and i0["status"] == 0 and i1["status"] == 0 and i1["iters"] > 0
+        out.append((plain, scaled, i0["iters"], i1["iters"]))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert out[0][2:] == out[1][2:]
