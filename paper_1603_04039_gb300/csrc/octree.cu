@@ -380,18 +380,37 @@ __device__ __forceinline__ int leaf_at(const int32_t *first, int lo, int hi, int
 // through the permutation), a tile of sorted particles per block.  While the
 // two arrays fit L2 the 4-byte stores go straight to their random places (tiles
 // of PL_SMALL, so that small sets reach all SMs: 15 us for 1e5 particles, 26 in
-// tiles of 8192; 192 and 202 for 1e7).  Larger sets (BUCKET) would fetch and write back a 32-byte sector
-// per store: the tile is ordered by destination window first and appended to
-// the windows' lists (a permutation fills every window exactly), and
-// k_particle_place stores window by window, inside L2.
+// tiles of 8192; 187 and 202 for 1e7, 200 with windows).  Larger sets (BUCKET)
+// would fetch and write back a 32-byte sector per store: the tile is ordered by
+// destination window first and appended to the windows' lists (a permutation
+// fills every window exactly), and k_particle_place stores window by window,
+// inside L2.  A list entry is one word; as three words in a row it took 402
+// instead of 310 us for 2e7 particles, both kernels.  Sets whose three fields
+// need more than 64 bits are stored directly.
 constexpr int PL_SMALL = 1024, PL_TILE = 8192, PL_T = 1024, PL_WIN = 2048;   // most windows
 constexpr int PL_WBITS = 14;                               // particles per window: 128 KB of the two arrays
+// A particle of a window's list in one word: its place in the window, its leaf
+// and its key-sorted position (w, l and s bits)
+struct PackBits {
+    int w, l, s;
+    __device__ __forceinline__ uint64_t pack(uint32_t p, int leaf, int64_t pos) const {
+        return (uint64_t)(p & ((1u << w) - 1u)) << (l + s) | (uint64_t)leaf << s | (uint64_t)pos;
+    }
+    __device__ __forceinline__ uint32_t low(uint64_t e) const { return (uint32_t)(e >> (l + s)) & ((1u << w) - 1u); }
+    __device__ __forceinline__ int32_t leaf(uint64_t e) const { return (int32_t)(e >> s & ((1ull << l) - 1ull)); }
+    __device__ __forceinline__ int32_t pos(uint64_t e) const { return (int32_t)(e & ((1ull << s) - 1ull)); }
+};
+static int bits_of(uint64_t v) {
+    int b = 0;
+    while (v >> b) ++b;
+    return b;
+}
 template <bool BUCKET>
 __global__ void __launch_bounds__(PL_T) k_particle_leaf(const int32_t *__restrict__ first, int n_leaf,
                                                         const uint32_t *__restrict__ perm, int64_t n,
                                                         int32_t *__restrict__ pleaf, int32_t *__restrict__ spos,
-                                                        int tile, int wbits, uint32_t *__restrict__ cursor,
-                                                        uint32_t *__restrict__ bp) {
+                                                        int tile, PackBits pb, uint32_t *__restrict__ cursor,
+                                                        uint64_t *__restrict__ bp) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int range[2];
     __shared__ uint32_t wtot[PL_T / 32];
@@ -415,8 +434,9 @@ __global__ void __launch_bounds__(PL_T) k_particle_leaf(const int32_t *__restric
         }
         return;
     }
-    uint32_t *sp = gof + PL_WIN;
-    int32_t *sj = reinterpret_cast<int32_t *>(sp + PL_TILE), *si = sj + PL_TILE;
+    uint64_t *sw = reinterpret_cast<uint64_t *>(gof + PL_WIN);
+    uint16_t *win_of = reinterpret_cast<uint16_t *>(sw + PL_TILE);
+    const int wbits = pb.w;
     constexpr int PER = PL_TILE / PL_T, WPT = PL_WIN / PL_T;
     uint32_t p[PER], r[PER];
 #pragma unroll
@@ -459,23 +479,19 @@ __global__ void __launch_bounds__(PL_T) k_particle_leaf(const int32_t *__restric
         const int t = tid + u * PL_T;
         if (t < m) {
             const uint32_t at = cnt[p[u] >> wbits] + r[u];
-            sp[at] = p[u];
-            sj[at] = leaf_at(first, ja, jb, (int)(i0 + t));
-            si[at] = (int32_t)(i0 + t);
+            sw[at] = pb.pack(p[u], leaf_at(first, ja, jb, (int)(i0 + t)), i0 + t);
+            win_of[at] = (uint16_t)(p[u] >> wbits);
         }
     }
     __syncthreads();
     for (int t = tid; t < m; t += PL_T) {
-        const uint32_t dst = gof[sp[t] >> wbits] + (uint32_t)t;
-        if (dst >= n) continue;   // only after a sort that gave up
-        bp[3 * (int64_t)dst] = sp[t];
-        bp[3 * (int64_t)dst + 1] = (uint32_t)sj[t];
-        bp[3 * (int64_t)dst + 2] = (uint32_t)si[t];
+        const uint32_t dst = gof[win_of[t]] + (uint32_t)t;
+        if (dst < n) bp[dst] = sw[t];   // else only after a sort that gave up
     }
 }
 
 // A window's list into the two arrays, ordered in shared memory (WBITS = 14)
-__global__ void __launch_bounds__(1024) k_particle_place(const uint32_t *__restrict__ bp, int64_t n,
+__global__ void __launch_bounds__(1024) k_particle_place(const uint64_t *__restrict__ bp, int64_t n, PackBits pb,
                                                          int32_t *__restrict__ pleaf, int32_t *__restrict__ spos) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int W = 1 << PL_WBITS;
@@ -484,10 +500,10 @@ __global__ void __launch_bounds__(1024) k_particle_place(const uint32_t *__restr
     const int m = (int)(n - p0 < W ? n - p0 : W);
 #pragma unroll 4
     for (int t = threadIdx.x; t < m; t += 1024) {
-        const uint32_t *e = bp + 3 * (p0 + t);
-        const uint32_t at = (__ldcs(e) - (uint32_t)p0) & (W - 1);
-        sl[at] = (int32_t)__ldcs(e + 1);
-        ss[at] = (int32_t)__ldcs(e + 2);
+        const uint64_t e = __ldcs(bp + p0 + t);
+        const uint32_t at = pb.low(e);   // pb.w = PL_WBITS
+        sl[at] = pb.leaf(e);
+        ss[at] = pb.pos(e);
     }
     __syncthreads();
     for (int t = threadIdx.x; t < m; t += 1024) {
@@ -498,14 +514,15 @@ __global__ void __launch_bounds__(1024) k_particle_place(const uint32_t *__restr
 
 // The same for more particles than PL_WIN such windows hold: larger windows,
 // the stores to random places of a window that stays in L2
-__global__ void __launch_bounds__(T) k_particle_place_l2(const uint32_t *__restrict__ bp, int64_t n,
+__global__ void __launch_bounds__(T) k_particle_place_l2(const uint64_t *__restrict__ bp, int64_t n, PackBits pb,
                                                          int32_t *__restrict__ pleaf, int32_t *__restrict__ spos) {
     const int64_t i = (int64_t)blockIdx.x * T + threadIdx.x;
     if (i >= n) return;
-    const uint32_t p = __ldcs(bp + 3 * i);
+    const uint64_t e = __ldcs(bp + i);
+    const int64_t p = (i >> pb.w << pb.w) + pb.low(e);   // a window's list fills its place exactly
     if (p >= n) return;   // only after a sort that gave up
-    pleaf[p] = (int32_t)__ldcs(bp + 3 * i + 1);
-    spos[p] = (int32_t)__ldcs(bp + 3 * i + 2);
+    pleaf[p] = pb.leaf(e);
+    spos[p] = pb.pos(e);
 }
 
 // Boundary nodes, ordered by (face, owner): the blocks' counts scanned face
@@ -694,9 +711,8 @@ KeyFix key_fix(const apcloud_params &P) {
 }
 
 // Bytes of the two arrays past which their random stores go window by window:
-// 1e7 particles (80 MB, inside L2) take 0.19 ms straight and 0.22 ms in windows,
-// 2e7 (160 MB) 1.03 ms straight, 0.44 ms in 2 MB windows that stay in L2 and
-// 0.30 ms in windows ordered in shared memory
+// 1e7 particles (80 MB, inside L2) take 0.19 ms straight and 0.20 ms in windows,
+// 2e7 (160 MB) 1.03 ms straight and 0.31 ms in windows ordered in shared memory
 constexpr int64_t PL_DIRECT_BYTES = 100ll << 20;
 
 template <class K>
@@ -793,26 +809,27 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
                lc, ic, lb, bcnt, nblk);
     const uint32_t *perm = ptr<uint32_t>(c->val[c->kbuf]);
     if (n > 0) {
-        if (8 * n <= PL_DIRECT_BYTES) {
+        int wbits = PL_WBITS;
+        while ((n - 1) >> wbits >= PL_WIN) ++wbits;
+        const PackBits pb{wbits, bits_of((uint64_t)nleaf - 1), bits_of((uint64_t)n - 1)};
+        if (8 * n <= PL_DIRECT_BYTES || pb.w + pb.l + pb.s > 64) {
             APC_LAUNCH(c, K_TREE, div_up(n, PL_SMALL), PL_SMALL / 4, 0, k_particle_leaf<false>, (const int32_t *)lf,
-                       (int)nleaf, perm, n, pl, sp, PL_SMALL, 0, (uint32_t *)nullptr, (uint32_t *)nullptr);
+                       (int)nleaf, perm, n, pl, sp, PL_SMALL, pb, (uint32_t *)nullptr, (uint64_t *)nullptr);
         } else {
-            int wbits = PL_WBITS;
-            while ((n - 1) >> wbits >= PL_WIN) ++wbits;
-            uint32_t *bp = ensure<uint32_t>(c, c->bkt, 3 * n + PL_WIN);
+            uint64_t *bp = ensure<uint64_t>(c, c->bkt, n + PL_WIN);
             if (!bp) return APCLOUD_E_NOMEM;
-            uint32_t *cursor = bp + 3 * n;
-            const int smem = (2 * PL_WIN + 3 * PL_TILE) * 4, wsm = 8 << PL_WBITS;
+            uint32_t *cursor = reinterpret_cast<uint32_t *>(bp + n);
+            const int smem = 2 * PL_WIN * 4 + PL_TILE * 10, wsm = 8 << PL_WBITS;
             APC_CUDA(c, cudaMemsetAsync(cursor, 0, PL_WIN * sizeof(uint32_t), c->s));
             APC_CUDA(c, cudaFuncSetAttribute(k_particle_leaf<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             APC_CUDA(c, cudaFuncSetAttribute(k_particle_place, cudaFuncAttributeMaxDynamicSharedMemorySize, wsm));
             APC_LAUNCH(c, K_TREE, div_up(n, PL_TILE), PL_T, smem, k_particle_leaf<true>, (const int32_t *)lf,
-                       (int)nleaf, perm, n, pl, sp, PL_TILE, wbits, cursor, bp);
+                       (int)nleaf, perm, n, pl, sp, PL_TILE, pb, cursor, bp);
             if (wbits == PL_WBITS)
-                APC_LAUNCH(c, K_TREE, div_up(n, 1 << PL_WBITS), 1024, wsm, k_particle_place, (const uint32_t *)bp, n,
+                APC_LAUNCH(c, K_TREE, div_up(n, 1 << PL_WBITS), 1024, wsm, k_particle_place, (const uint64_t *)bp, n, pb,
                            pl, sp);
             else
-                APC_LAUNCH(c, K_TREE, div_up(n, T), T, 0, k_particle_place_l2, (const uint32_t *)bp, n, pl, sp);
+                APC_LAUNCH(c, K_TREE, div_up(n, T), T, 0, k_particle_place_l2, (const uint64_t *)bp, n, pb, pl, sp);
         }
     }
     uint32_t *bpos = bcnt + 6 * (int64_t)nblk;
