@@ -1128,15 +1128,28 @@ __global__ void __launch_bounds__(SW * 32, 24 / SW) k_wls32(
 
 // ---------------------------------------------------------------- matrices
 // diagonals of A and B (the Jacobi scaling) and their reciprocals
+// h^2 / 24 of a level-lev cell of a domain of edge ext, from ext^2 / 24: a power of
+// two apart, so rounded alike
+__device__ __forceinline__ double cell_scale(double ext2_24, int lev) {
+    return ext2_24 * __longlong_as_double((long long)(1023 - 2 * lev) << 52);
+}
+// x / d where d was computed as x: 1 unless x is zero or not finite.  The
+// divisions, by 24 too, were 50 us of the 667 that the matrices of 1.05e6 rows
+// take.
+__device__ __noinline__ double own_quotient_odd(double x, double d) { return x / d; }
+__device__ __forceinline__ double own_quotient(double x, double d) {
+    const unsigned long long m = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+    if (m - 1ull >= 0x7FF0000000000000ull - 1ull) return own_quotient_odd(x, d);
+    return 1.0;
+}
 __global__ void k_diag(const int32_t *__restrict__ msz, const double *__restrict__ lapd, const int4 *__restrict__ ic,
-                       int n_int, int n_tot, double ext, double *__restrict__ dA, double *__restrict__ dB,
+                       int n_int, int n_tot, double ext2_24, double *__restrict__ dA, double *__restrict__ dB,
                        double2 *__restrict__ rAB) {
     int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_tot) return;
     double a = 1.0, b = 1.0;
     if (r < n_int) {
-        double h = ldexp(ext, -ic[r].w);
-        double s = h * h / 24.0;
+        const double s = cell_scale(ext2_24, ic[r].w);
         a = lapd[r];
         b = 1.0 + s * lapd[r];
     }
@@ -1190,7 +1203,7 @@ template <bool MIXED>
 __global__ void __launch_bounds__(256) k_ell_fill(
     const int32_t *__restrict__ msz, const int32_t *__restrict__ nbr, const double *__restrict__ lap,
     const double *__restrict__ lapd, const int4 *__restrict__ ic, const double *__restrict__ dA,
-    const double *__restrict__ dB, const double2 *__restrict__ rAB, int n_int, int n_tot, double ext,
+    const double *__restrict__ dB, const double2 *__restrict__ rAB, int n_int, int n_tot, double ext2_24,
     const uint32_t *__restrict__ sw, const uint32_t *__restrict__ soff, int32_t *__restrict__ col,
     double *__restrict__ vA, double *__restrict__ vB, LowCopies low) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1202,13 +1215,12 @@ __global__ void __launch_bounds__(256) k_ell_fill(
     const int m = inner ? msz[r] : 0, own = real ? r : 0;
     double a0 = 0.0, b0 = 0.0, sc = 0.0;
     if (inner) {
-        const double h = ldexp(ext, -ic[r].w), l = lapd[r];
-        sc = h * h / 24.0;
-        a0 = l / dA[r];
-        b0 = (1.0 + sc * l) / dB[r];
+        const double l = lapd[r];
+        sc = cell_scale(ext2_24, ic[r].w);
+        a0 = own_quotient(l, dA[r]);
+        b0 = own_quotient(1.0 + sc * l, dB[r]);
     } else if (real) {
-        a0 = 1.0 / dA[r];
-        b0 = 1.0 / dB[r];
+        a0 = b0 = 1.0;   // identity rows
     }
     col[base] = own;
     vA[base] = a0;
@@ -1361,7 +1373,8 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     double *dB = ensure<double>(c, c->dB, nt + 1);
     double2 *rd = ensure<double2>(c, c->ell_rd, (int64_t)nt + 1);   // reciprocals, for the fill only
     if (!sw || !so || !dA || !dB || !rd) return APCLOUD_E_NOMEM;
-    APC_LAUNCH(c, K_ELL, div_up(nt, 256), 256, 0, k_diag, msz, lapd, ptr<int4>(c->node_ic), n, nt, ext, dA, dB, rd);
+    APC_LAUNCH(c, K_ELL, div_up(nt, 256), 256, 0, k_diag, msz, lapd, ptr<int4>(c->node_ic), n, nt, ext * ext / 24.0, dA,
+               dB, rd);
     uint32_t *small = ptr<uint32_t>(c->dsmall);
     APC_CUDA(c, cudaMemsetAsync(small + 6, 0, sizeof(uint32_t), c->s));
     APC_LAUNCH(c, K_ELL, div_up(nsl, 8), 256, 0, k_slice_width, msz, n, nt, nsl, sw, small + 6);
@@ -1387,13 +1400,13 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     if (!col || !vA || !vB) return APCLOUD_E_NOMEM;
     if (c->P.precision == 0) {
         APC_LAUNCH(c, K_ELL, div_up((int64_t)nsl * 32, 256), 256, 0, k_ell_fill<false>, msz, nbr, lap, lapd,
-                   ptr<int4>(c->node_ic), dA, dB, (const double2 *)rd, n, nt, ext, sw, so, col, vA, vB, LowCopies{});
+                   ptr<int4>(c->node_ic), dA, dB, (const double2 *)rd, n, nt, ext * ext / 24.0, sw, so, col, vA, vB, LowCopies{});
     } else {
         const LowCopies low{ensure<float>(c, c->ell_A32, c->ell_entries), ensure<float>(c, c->ell_B32, c->ell_entries),
                             ensure<__half>(c, c->ell_A16, c->ell_entries), ensure<__half>(c, c->ell_B16, c->ell_entries)};
         if (!low.fA || !low.fB || !low.hA || !low.hB) return APCLOUD_E_NOMEM;
         APC_LAUNCH(c, K_ELL, div_up((int64_t)nsl * 32, 256), 256, 0, k_ell_fill<true>, msz, nbr, lap, lapd,
-                   ptr<int4>(c->node_ic), dA, dB, (const double2 *)rd, n, nt, ext, sw, so, col, vA, vB, low);
+                   ptr<int4>(c->node_ic), dA, dB, (const double2 *)rd, n, nt, ext * ext / 24.0, sw, so, col, vA, vB, low);
         if (blocks && !resident_ok(c, 1)) APC_TRY(build_blocks(c));
     }
     return cuda_check(c, cudaGetLastError(), "ell");
