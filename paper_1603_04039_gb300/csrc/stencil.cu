@@ -1184,7 +1184,7 @@ __global__ void k_slice_width(const int32_t *__restrict__ msz, int n_int, int n_
 // long.  The mixed form's FP32 and FP16 copies are written along (a pass of their
 // own read the values again and converted to FP16 on the FP64 pipe), a row's
 // four next columns and values come in three loads and a column's two
-// reciprocals in one: at 2.5e7 entries 290 us, fill and copies 262 + 190 before.
+// reciprocals in one: at 2.5e7 entries 270 us, fill and copies 262 + 190 before.
 struct LowCopies {   // null without the mixed form
     float *fA, *fB;
     __half *hA, *hB;

@@ -27,9 +27,9 @@
 // (chunk j of lane l at 32 j + l in its slice): 16 bytes of FP16 values, 8 and 4
 // bytes of indices (the products load FP32 values instead).  Nine rows in ten
 // have 17 to 24 entries, three chunks.  The diagonal, first in every row and 1
-// after the scaling, is stored apart and read only where it is not.  Rows keep their entries in stored order: the
-// results have the same bits as on the ELL.  Lanes past their row's length load
-// nothing.
+// after the scaling, is stored apart and read only where it is not.  Rows keep
+// their entries in stored order: the results have the same bits as on the ELL.
+// Lanes past their row's length load nothing.
 #include <cuda_fp16.h>
 
 #include <algorithm>
