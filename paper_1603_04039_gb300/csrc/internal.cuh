@@ -66,12 +66,16 @@ struct GmresState {
 };
 
 // A captured restart cycle (CUDA graph), keyed by everything its launches
-// depend on: element size, sizes, timing mask and every buffer address.
+// depend on: element size, sizes and counts (addresses inside a buffer that a
+// count enters among them), what a launch takes by value, timing mask and every
+// buffer address.
 struct GraphKey {
     int tsize, n, jmax, pdeg, nblk, spmv_bs, pdl;
     unsigned mask;
-    int64_t ldv, skeep;
-    const void *p[40];
+    int64_t ldv, skeep, chunks;   // chunks: where the block-local copy's 4-byte indices start
+    int nb, nitems;               // batches: beams, items of their Krylov spaces
+    double rtol;                  // batches on one Krylov space: tolerance of the beams' masks
+    const void *p[48];
 };
 
 // Arnoldi step j >= 1 of a captured cycle sits in an IF node whose condition

@@ -2234,17 +2234,23 @@ apcloud_status run_cycle(apcloud_ctx *c, const T *val, const T *b, T *u, const K
         key.spmv_bs = c->spmv_bs * 8 + c->spmv_unroll;
         key.skeep = K.skeep;
         key.pdl = c->pdl_on ? 1 : 0;
-        const void *p[] = {val, b, u, K.V, K.w, K.wraw, K.st, K.partial, K.z0, K.z1, K.t, K.hval,
+        const bool blk = K.blocks >= 0;
+        key.chunks = blk ? c->bl_chunks : -1;
+        key.nb = K.bk ? K.bk->nb : (K.mask ? K.mask->nb : 0);
+        key.nitems = K.bk ? K.bk->nitems : 0;
+        key.rtol = K.mask ? K.mask->rtol : 0.0;
+        const BeamMask bm = K.mask ? *K.mask : BeamMask{};
+        const BKry bk = K.bk ? *K.bk : BKry{};
+        const bool beams = K.mask || K.bk;
+        const void *p[] = {val, b, u, K.V, K.w, K.wraw, K.st, K.partial, K.z0, K.z1, K.t, K.Z, K.hval,
                            c->slice_w.p, c->slice_off.p, c->ell_col.p, K.skip.nbo, K.skip.bdone, K.tact,
-                           K.mask ? K.mask->r2 : nullptr, K.bk ? K.bk->items : nullptr,
-                           K.bk ? K.bk->H : nullptr, K.bk ? K.bk->done : nullptr,
-                           K.bk ? (const void *)(intptr_t)K.bk->nitems : nullptr, K.Z,
-                           (const void *)(intptr_t)(K.blocks + 1), K.blocks >= 0 ? c->bl_idx.p : nullptr,
-                           K.blocks >= 0 ? c->bl_hlist.p : nullptr, K.blocks >= 0 ? c->bl_off.p : nullptr,
-                           K.blocks >= 0 ? c->bl_len.p : nullptr, K.blocks >= 0 ? c->bl_hcnt.p : nullptr,
-                           K.blocks >= 0 ? (K.blocks ? c->bl_A.p : c->bl_B.p) : nullptr,
-                           K.blocks >= 0 ? (K.blocks ? c->bl_A32.p : c->bl_B32.p) : nullptr,
-                           K.blocks >= 0 && !c->bl_unit ? c->bl_dg.p : nullptr};
+                           beams ? c->beam_rng.p : nullptr, beams ? c->beam_part.p : nullptr, bm.b2, bm.r2, bm.bdone,
+                           bm.nbo, bk.items, bk.item_off, bk.nbo, bk.H, bk.done, (const void *)(intptr_t)(K.blocks + 1),
+                           blk ? c->bl_idx.p : nullptr, blk ? c->bl_hlist.p : nullptr, blk ? c->bl_off.p : nullptr,
+                           blk ? c->bl_len.p : nullptr, blk ? c->bl_hcnt.p : nullptr,
+                           blk ? (K.blocks ? c->bl_A.p : c->bl_B.p) : nullptr,
+                           blk ? (K.blocks ? c->bl_A32.p : c->bl_B32.p) : nullptr, blk ? c->bl_dg.p : nullptr,
+                           (const void *)(intptr_t)(blk && !c->bl_unit)};
         static_assert(sizeof p <= sizeof key.p, "graph key holds every buffer address");
         for (size_t i = 0; i < sizeof p / sizeof p[0]; ++i) key.p[i] = p[i];
         GraphEntry *g = find_graph(c, key);
