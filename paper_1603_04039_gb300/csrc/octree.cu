@@ -744,11 +744,12 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
     const double c2 = c->P.c_refine * c->P.c_refine;
     for (int l = 0; l < L; ++l) {
         const double h = ldexp(ext, -l), h2 = h * h;
-        double t = std::ceil(c2 / h2);
+        // at most 4e9, more than there are particles: past 2^53 a step of one changes nothing
+        double t = std::fmin(std::ceil(c2 / h2), 4e9);
         if (!(t >= 1.0)) t = 1.0;
         while (t > 1.0 && (t - 1.0) * h2 >= c2) t -= 1.0;
         while (t < 4e9 && t * h2 < c2) t += 1.0;
-        th.t[l] = t < 4e9 ? (uint32_t)t : 4000000000u;   // more than there are particles
+        th.t[l] = (uint32_t)t;
     }
     CellSet set{};
     uint32_t nopen = 0;

@@ -1,0 +1,28 @@
+"""Trees at the ends of the parameters' ranges."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1603_04039_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+DEV = torch.device("cuda:0")
+
+
+# thresholds of the deeper levels past 2^53 particles, the last two past every level's
+@pytest.mark.parametrize("depth,c", [(21, 140.0), (21, 200.0), (12, 60.0), (8, 1e7), (21, 1e9), (21, 1e200)])
+@pytest.mark.timeout(120)
+def test_large_refinement_constants(depth, c):
+    from paper_1603_04039_gb300 import APCloud
+    x, y, z, _ = inputs.beam_with_halo(20000, 6)
+    ap = APCloud(max_depth=depth, c_refine=c)
+    counts = ap.build_octree(*(torch.from_numpy(a).to(DEV) for a in (x, y, z)))
+    o = oracle.Oracle(max_depth=depth, c_refine=c)
+    o.build(x, y, z)
+    assert counts == (o.n_int, o.n_bnd)
+    g, (key, first, count) = ap.get_leaves(), o.leaves()
+    assert np.array_equal(g["key"].cpu().numpy().astype(np.uint64), key)
+    assert np.array_equal(g["first"].cpu().numpy(), first)
+    assert np.array_equal(g["count"].cpu().numpy(), count)
