@@ -122,53 +122,79 @@ __global__ void __launch_bounds__(256) k_gather_leaf(
     if (ez) __stcs(ez + i, gz);
 }
 
+// the two doubles of a 16-byte part of a record
+__device__ __forceinline__ double f4_lo(const float4 &v) {
+    return __hiloint2double(__float_as_int(v.y), __float_as_int(v.x));
+}
+__device__ __forceinline__ double f4_hi(const float4 &v) {
+    return __hiloint2double(__float_as_int(v.w), __float_as_int(v.z));
+}
+
 // The mixed form: corrections (g.r, H r, r.H.r) in FP32 around the FP64 node
 // potential, from the compact record; its node derivatives carry FP32 accuracy
 // already (FP32 stencils).  The pass stays off the slow FP64 pipe but for the
 // offsets from the centre and the potential's add: the seven double/float
 // conversions run on the integer pipe.
 //
-// Particles come in any order, so a record per lane costs five loads of 32
-// different lines each, 160 L1 look-ups a warp: 312 us at 2e7 particles, twice
-// what the bytes take.  Here a warp fetches its 32 records together, the five
-// 16-byte parts of a record by neighbouring lanes (a third of the look-ups),
-// and hands them over through shared memory (rows of 80 bytes: no bank
-// conflicts): 297 us.  Records of 96 or 128 bytes change nothing, loads past L1
-// (358 us: a tenth of the leaves hold most particles) and asynchronous copies
-// into shared memory (310 us) lose.
+// A record per lane costs five loads of as many lines as the warp has different
+// leaves.  With few leaves (their records in L1) or with particles in cell order
+// that is little.  Particles in any order on many leaves take 160 L1 look-ups a
+// warp; there (STAGED) a warp fetches its 32 records together, the five 16-byte
+// parts of a record by neighbouring lanes (a third of the look-ups), and hands
+// them over through shared memory (rows of 80 bytes: no bank conflicts), which
+// costs the same whatever the leaves.  2e7 particles, a record per lane / staged:
+//     leaves               1128       5104       26202      36807      215111     320804
+//     in any order      241 / 293  251 / 304  292 / 295  301 / 294  312 / 295  313 / 297 us
+//     pairs in a leaf   238 / 287  246 / 289  250 / 289  250 / 288  252 / 288  254 / 291
+//     in cell order     235 / 280  235 / 279  236 / 280  235 / 280  243 / 292  245 / 297
+// Hence STAGED_LEAVES, and staged only where the warps of a sample taken with the
+// tree (c->scattered) hold nearly as many leaves as particles.  A choice by each warp keeps
+// the shared memory out of L1 in either case: 272 in place of 243 us in cell
+// order.  Records of 96 or 128 bytes change nothing; loads past L1 (358 us) and
+// asynchronous copies into shared memory (310 us) lose.
+constexpr int STAGED_LEAVES = 32768;
+template <bool STAGED>
 __global__ void __launch_bounds__(GT) k_gather_leaf32(
     const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z, int64_t n,
     const int32_t *__restrict__ pleaf, const float *__restrict__ nf32, double *__restrict__ php,
     double *__restrict__ ex, double *__restrict__ ey, double *__restrict__ ez) {
-    __shared__ float4 rec[GT * 5];
     const int64_t i = (int64_t)blockIdx.x * GT + threadIdx.x;
-    const int lane = threadIdx.x & 31;
     const bool live = i < n;
+    if (!STAGED && !live) return;
     const int j = live ? __ldcs(pleaf + i) : 0;
     const double p0 = live ? __ldcs(x + i) : 0.0, p1 = live ? __ldcs(y + i) : 0.0, p2 = live ? __ldcs(z + i) : 0.0;
-    float4 *mine = rec + (threadIdx.x - lane) * 5;
-    float4 part[5];
+    float4 f[5];
+    if constexpr (STAGED) {
+        __shared__ float4 rec[GT * 5];
+        const int lane = threadIdx.x & 31;
+        float4 *mine = rec + (threadIdx.x - lane) * 5;
 #pragma unroll
-    for (int t = 0; t < 5; ++t) {
-        const int e = t * 32 + lane, o = e / 5;
-        const int jo = __shfl_sync(0xFFFFFFFFu, j, o);
-        part[t] = __ldg(reinterpret_cast<const float4 *>(nf32 + (int64_t)jo * NF32) + (e - o * 5));
+        for (int t = 0; t < 5; ++t) {
+            const int e = t * 32 + lane, o = e / 5;
+            const int jo = __shfl_sync(0xFFFFFFFFu, j, o);
+            f[t] = __ldg(reinterpret_cast<const float4 *>(nf32 + (int64_t)jo * NF32) + (e - o * 5));
+        }
+#pragma unroll
+        for (int t = 0; t < 5; ++t) mine[t * 32 + lane] = f[t];
+        __syncwarp();
+        if (!live) return;
+#pragma unroll
+        for (int t = 0; t < 5; ++t) f[t] = mine[lane * 5 + t];
+    } else {
+        const float4 *r = reinterpret_cast<const float4 *>(nf32 + (int64_t)j * NF32);
+#pragma unroll
+        for (int t = 0; t < 5; ++t) f[t] = __ldg(r + t);
     }
-#pragma unroll
-    for (int t = 0; t < 5; ++t) mine[t * 32 + lane] = part[t];
-    __syncwarp();
-    if (!live) return;
-    const double2 pc = *reinterpret_cast<const double2 *>(mine + lane * 5);
-    const double2 cc = *reinterpret_cast<const double2 *>(mine + lane * 5 + 1);
-    const float4 u = mine[lane * 5 + 2], w = mine[lane * 5 + 3];
-    const float fzz = mine[lane * 5 + 4].x;
-    const float r0 = f64_to_f32_int(p0 - pc.y), r1 = f64_to_f32_int(p1 - cc.x), r2 = f64_to_f32_int(p2 - cc.y);
+    const double pc = f4_lo(f[0]), cx = f4_hi(f[0]), cy = f4_lo(f[1]), cz = f4_hi(f[1]);
+    const float4 u = f[2], w = f[3];
+    const float fzz = f[4].x;
+    const float r0 = f64_to_f32_int(p0 - cx), r1 = f64_to_f32_int(p1 - cy), r2 = f64_to_f32_int(p2 - cz);
     // u = (fx, fy, fz, fxx), w = (fxy, fxz, fyy, fyz)
     const float hr0 = fmaf(w.y, r2, fmaf(w.x, r1, u.w * r0));
     const float hr1 = fmaf(w.w, r2, fmaf(w.z, r1, w.x * r0));
     const float hr2 = fmaf(fzz, r2, fmaf(w.w, r1, w.y * r0));
     const float corr = fmaf(u.z, r2, fmaf(u.y, r1, u.x * r0)) + 0.5f * fmaf(r2, hr2, fmaf(r1, hr1, r0 * hr0));
-    if (php) __stcs(php + i, pc.x + f32_to_f64_int(corr));
+    if (php) __stcs(php + i, pc + f32_to_f64_int(corr));
     if (ex) __stcs(ex + i, f32_to_f64_int(u.x + hr0));
     if (ey) __stcs(ey + i, f32_to_f64_int(u.y + hr1));
     if (ez) __stcs(ez + i, f32_to_f64_int(u.z + hr2));
@@ -225,8 +251,11 @@ apcloud_status gather_field(apcloud_ctx *c, double *phi_p, double *ex, double *e
     APC_LAUNCH(c, K_DERIV, div_up(n, db), db, 0, k_derivs, ptr<uint32_t>(c->slice_w), ptr<uint32_t>(c->slice_off),
                ptr<int32_t>(c->ell_col), ptr<double>(c->D), dstride, ptr<double>(c->phi), n, nf,
                ptr<int4>(c->node_ic), c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, nf32);
-    if (mixed)
-        APC_LAUNCH(c, K_GATHER, div_up(c->N, GT), GT, 0, k_gather_leaf32, c->px, c->py, c->pz, c->N,
+    if (mixed && n >= STAGED_LEAVES && c->scattered)
+        APC_LAUNCH(c, K_GATHER, div_up(c->N, GT), GT, 0, k_gather_leaf32<true>, c->px, c->py, c->pz, c->N,
+                   (const int32_t *)ptr<int32_t>(c->pleaf), (const float *)nf32, phi_p, ex, ey, ez);
+    else if (mixed)
+        APC_LAUNCH(c, K_GATHER, div_up(c->N, GT), GT, 0, k_gather_leaf32<false>, c->px, c->py, c->pz, c->N,
                    (const int32_t *)ptr<int32_t>(c->pleaf), (const float *)nf32, phi_p, ex, ey, ez);
     else
         APC_LAUNCH(c, K_GATHER, div_up(c->N, 256), 256, 0, k_gather_leaf, c->px, c->py, c->pz, c->N,

@@ -217,6 +217,7 @@ struct apcloud_ctx {
     int64_t ell_entries = 0;
     int64_t sum_m = 0;  // total stencil neighbours over interior nodes
     int64_t n_fp64_wls = 0;  // mixed form: stencils refactored in FP64
+    bool scattered = false;  // particles side by side in the caller's order mostly lie in different leaves
 
     // sorted particle keys (32 or 64 bits) and permutation (result in key[kbuf], val[kbuf])
     apc::DBuf key[2], val[2];

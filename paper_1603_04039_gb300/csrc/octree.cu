@@ -628,12 +628,36 @@ __global__ void __launch_bounds__(T) k_adjacency(const uint64_t *__restrict__ an
     for (int t = tot + f; t < 24; t += 8) out[t] = -1;
 }
 
+// Different leaves among 32 particles side by side in the caller's order, summed
+// over SPREAD_N such groups spread evenly over the set (read by the choice of the
+// gather's form); one block.
+constexpr int SPREAD_N = 128, SPREAD_MOST = 30;
+__device__ __forceinline__ void leaf_spread(const int32_t *pleaf, int64_t n, unsigned *out) {
+    constexpr int PER = SPREAD_N / (T / 32);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int32_t leaf[PER];
+#pragma unroll
+    for (int g = 0; g < PER; ++g) leaf[g] = pleaf[(n - 32) * (w * PER + g) / (SPREAD_N - 1) + lane];
+    unsigned sum = 0;
+#pragma unroll
+    for (int g = 0; g < PER; ++g) {
+        const unsigned peers = __match_any_sync(0xffffffffu, leaf[g]);
+        sum += __popc(__ballot_sync(0xffffffffu, lane == __ffs(peers) - 1));
+    }
+    if (lane == 0) atomicAdd(out, sum);
+}
+
 // Node ranges of every beam: interior nodes [r[b], r[b+1]) (the leaves are
 // beam-sorted) and, per face f, boundary nodes [r[(1+f)(nb+1)+b], ...+1) (the
 // boundary nodes are face-major, leaf-ordered within a face).
 __global__ void k_beam_ranges(const int32_t *__restrict__ beam, int64_t n, int nb, const uint32_t *__restrict__ bpos,
                               int nblk, const uint32_t *__restrict__ nbnd, const int32_t *__restrict__ owner,
-                              int64_t *__restrict__ r) {
+                              int64_t *__restrict__ r, const int32_t *__restrict__ pleaf, int64_t npart,
+                              unsigned *__restrict__ spread) {
+    if (npart >= 32 && blockIdx.x == gridDim.x - 1) {   // a block more than the ranges take
+        leaf_spread(pleaf, npart, spread);
+        return;
+    }
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b > nb) return;
     int64_t lo = b == nb ? n : 0, hi = b == 0 ? 0 : n;   // the first and the last bound need no search
@@ -838,14 +862,15 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
     APC_LAUNCH(c, K_TREE, nblk, T, 0, k_boundary, (const uint32_t *)bcnt, (const uint32_t *)bpos, nblk, nleaf, ic, bo,
                bf, adj);
     APC_LAUNCH(c, K_ADJ, div_up(8 * nleaf, T), T, 0, k_adjacency, la, ll, nleaf, L, adj, derr);
-    APC_LAUNCH(c, K_TREE, div_up(nb + 1, T), T, 0, k_beam_ranges, lb, nleaf, nb, (const uint32_t *)bpos, nblk,
-               (const uint32_t *)(small + 4), (const int32_t *)bo, rng);
+    APC_LAUNCH(c, K_TREE, div_up(nb + 1, T) + 1, T, 0, k_beam_ranges, lb, nleaf, nb, (const uint32_t *)bpos, nblk,
+               (const uint32_t *)(small + 4), (const int32_t *)bo, rng, (const int32_t *)pl, n, derr + 1);
     APC_CUDA(c, cudaGetLastError());
-    // the boundary count and the error word in one read
+    // the boundary count, the particles' spread and the error word in one read
     APC_CUDA(c, cudaMemcpyAsync(derr + 3, small + 4, sizeof(uint32_t), cudaMemcpyDeviceToDevice, c->s));
     unsigned e[4];
     APC_TRY(read_back(c, e, derr, sizeof e));
     c->n_bnd = (int)e[3];
+    c->scattered = e[1] >= SPREAD_MOST * SPREAD_N;
     c->n_tot = c->n_int + c->n_bnd;
     return device_errors(c, e[0]);
 }
