@@ -266,6 +266,7 @@ struct apcloud_ctx {
     // resident solves: tagged words, parameters and report, next unused tag
     apc::DBuf res_words, res_state;
     uint32_t res_tag = 1;
+    bool res_unfit = false;   // a block's share of the current operators does not fit
     // device staging for apcloud_field_host
     apc::DBuf hx, hy, hz, hq, hphi, hex, hey, hez;
     // error word, small host-visible values

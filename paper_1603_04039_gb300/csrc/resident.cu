@@ -951,7 +951,7 @@ void resident_grid(const apcloud_ctx *c, int *spc, int *grid) {
 int64_t resident_red_words(int grid) { return (int64_t)2 * RED_SLOTS * (grid + 1) * 2; }
 
 bool resident_ok(const apcloud_ctx *c, int which) {
-    if (c->nbeams > 1 || c->P.restart > PM || c->ilu_which == which || c->n_tot < 1) return false;
+    if (c->nbeams > 1 || c->P.restart > PM || c->ilu_which == which || c->n_tot < 1 || c->res_unfit) return false;
     int spc = 0, grid = 0, lim = 0, coop = 0, dev = 0;
     resident_grid(c, &spc, &grid);
     cudaGetDevice(&dev);
@@ -1085,7 +1085,10 @@ apcloud_status resident_run(apcloud_ctx *c, ResidentArgs a, const double *b, dou
         in.resume = iters > 0;
         *tag += TAGS_PER_LAUNCH;
         APC_TRY(run_resident(c, a, in, grid, graph, &o));
-        if (o.status == RES_UNFIT && iters == 0) return APCLOUD_OK;
+        if (o.status == RES_UNFIT && iters == 0) {
+            c->res_unfit = true;   // not asked again for these operators
+            return APCLOUD_OK;
+        }
         if (o.status == RES_TIMEOUT || o.abort)
             return fail(c, APCLOUD_E_TIMEOUT, "a block gave up waiting for another's part of a vector");
         iters += o.iters;

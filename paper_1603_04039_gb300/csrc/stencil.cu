@@ -1383,6 +1383,7 @@ apcloud_status build_stencils(apcloud_ctx *c) {
     // the resident solve takes do not need the copy
     c->ell_entries = 0;
     c->bl_ok = c->bl_tried = false;
+    c->res_unfit = false;
     const bool blocks = c->P.precision == 1 && c->P.poly_degree > 1;
     if (blocks) APC_TRY(count_blocks(c, small + 7));
     uint32_t tot[3];   // ELL columns, stencil sizes, chunks
