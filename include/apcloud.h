@@ -364,8 +364,10 @@ apcloud_status apcloud_set_graphs(apcloud_ctx *ctx, int enable);
  * *h_spmv_block, *h_spmv_unroll, *h_sweep_sorted and *h_wls_warps (any may be
  * NULL); h_ms (NULL or 19 doubles) receives the measured milliseconds: 16
  * solves (index = block-size index + 4 * unroll-4 + 8 * sorted; variants not
- * timed stay 0), then three stencil builds.  Results never depend on the
- * shapes.  Runs on the context stream and synchronises.  The paper has no
+ * timed stay 0), then three stencil builds.  Variants that are one and the same
+ * share one timing: all of the block-local copy's, and all 16 where the solve
+ * runs as one kernel, which leaves the shapes as they are.  Results never
+ * depend on the shapes.  Runs on the context stream and synchronises.  The paper has no
  * counterpart (launch mechanics). */
 apcloud_status apcloud_autotune(apcloud_ctx *ctx, unsigned what, int *h_spmv_block, int *h_spmv_unroll,
                                 int *h_sweep_sorted, int *h_wls_warps, double *h_ms);

@@ -2621,10 +2621,6 @@ apcloud_status gmres_solve(apcloud_ctx *c, int which, const double *b, double *x
     return status;
 }
 
-// Times the preconditioner sweep of the active form (FP16 values and FP32
-// vectors in the mixed form, else the matrix's own type; the plain Arnoldi
-// product when the preconditioner is Jacobi) at each block size and keeps the
-// fastest.  Contents of the work vectors do not matter for the timing.
 // right-hand side of the autotuner's solves: 1 + (i mod 7) / 10
 __global__ void k_tune_rhs(double *b, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2632,12 +2628,18 @@ __global__ void k_tune_rhs(double *b, int n) {
 }
 
 // The row-parallel products are timed where they run: for every launch
-// shape, one untimed solve (it captures the cycle graphs) and one timed solve
-// of the Poisson system with the configured solver, to a relative residual of
-// 1e-10 or TUNE_STEPS Arnoldi steps.  Timed in isolation, or over a single
-// restart cycle, the shapes rank differently from a whole solve (shorter
+// shape, one untimed solve (it captures the cycle graphs) and the best of two
+// timed solves of the Poisson system with the configured solver, to a relative
+// residual of 1e-10 or TUNE_STEPS Arnoldi steps.  Timed in isolation, or over a
+// single restart cycle, the shapes rank differently from a whole solve (shorter
 // capped cycles, and in a batch the beams converge one by one and their rows
 // then return at once).  The graphs the solves capture are released.
+//
+// Only what differs is timed.  A solve that runs as one kernel uses none of the
+// shapes: it is timed once, and the shapes stay as they are.  The block-local copy
+// has one shape of its own: it is timed once against the best on the ELL, and
+// where the system has none (a block's list overflowed) the choice between the
+// two stays as it is.
 constexpr int TUNE_STEPS = 1000;
 
 apcloud_status tune_spmv(apcloud_ctx *c, double *ms_out) {
@@ -2656,35 +2658,46 @@ apcloud_status tune_spmv(apcloud_ctx *c, double *ms_out) {
     APC_CUDA(c, cudaEventCreate(&e1));
     const unsigned mask = c->timer.mask;
     c->timer.mask = 0;
-    double best = 1e30;
-    apcloud_status rc = APCLOUD_OK;
-    for (int tu = 0; tu < nvar && rc == APCLOUD_OK; ++tu) {
-        const int t = tu & 3;
-        c->spmv_bs = sizes[t];
-        c->spmv_unroll = unrolls[(tu >> 2) & 1];
-        c->sweep_sorted = tu >> 3;
-        // a capture pass, then the best of two timed passes: shapes that differ by
-        // ~1% of a solve were ranked by single timings at random
-        float ms = 1e30f;
-        for (int rep = 0; rep < 3 && rc == APCLOUD_OK; ++rep) {
+    // the best of two timed solves after one that captures: shapes that differ by
+    // ~1% of a solve were ranked by single timings at random
+    auto time_solve = [&](float *ms) -> apcloud_status {
+        *ms = 1e30f;
+        for (int rep = 0; rep < 3; ++rep) {
             apcloud_solve_info info{};
-            rc = cuda_check(c, cudaMemsetAsync(tx, 0, sizeof(double) * n, c->s), "autotune");
-            if (rc != APCLOUD_OK) break;
+            APC_CUDA(c, cudaMemsetAsync(tx, 0, sizeof(double) * n, c->s));
             cudaEventRecord(e0, c->s);
-            rc = gmres_solve(c, 1, tb, tx, 1e-10, TUNE_STEPS, &info);
-            if (rc < 0) break;
-            rc = APCLOUD_OK;
+            const apcloud_status st = gmres_solve(c, 1, tb, tx, 1e-10, TUNE_STEPS, &info);
+            if (st < 0) return st;
             cudaEventRecord(e1, c->s);
-            rc = cuda_check(c, cudaEventSynchronize(e1), "autotune solve");
-            if (rc != APCLOUD_OK) break;
+            APC_CUDA(c, cudaEventSynchronize(e1));
             float t = 0.f;
             cudaEventElapsedTime(&t, e0, e1);
-            if (rep > 0 && t < ms) ms = t;
+            if (rep > 0 && t < *ms) *ms = t;
         }
-        if (rc != APCLOUD_OK) break;
-        if (ms_out) ms_out[tu] = ms;
-        if (ms < best) { best = ms; pick = sizes[t]; pick_u = unrolls[(tu >> 2) & 1]; pick_s = tu >> 3; }
+        return APCLOUD_OK;
+    };
+    float ms = 0.f, best = 1e30f;
+    int timed = 0;   // variants timed one by one; the rest share one timing
+    apcloud_status rc = APCLOUD_OK;
+    c->sweep_sorted = nvar == 16 ? 1 : saved_s;
+    rc = time_solve(&ms);   // the one kernel, or the block-local copy where there is one
+    if (rc == APCLOUD_OK && !resident_ok(c, 1)) {
+        const bool copy = nvar == 16 && c->bl_ok;
+        for (int tu = 0; tu < 8 && rc == APCLOUD_OK; ++tu) {
+            float t = 0.f;
+            c->spmv_bs = sizes[tu & 3];
+            c->spmv_unroll = unrolls[tu >> 2];
+            c->sweep_sorted = nvar == 16 ? 0 : saved_s;
+            rc = time_solve(&t);
+            if (rc != APCLOUD_OK) break;
+            if (ms_out) ms_out[tu] = t;
+            if (t < best) { best = t; pick = c->spmv_bs; pick_u = c->spmv_unroll; }
+        }
+        timed = 8;
+        if (copy) pick_s = ms < best ? 1 : 0;
     }
+    if (rc == APCLOUD_OK && ms_out)
+        for (int tu = timed; tu < nvar; ++tu) ms_out[tu] = ms;
     free_graphs(c);
     c->jprev[1][0] = c->jprev[1][1] = 0;
     c->timer.mask = mask;
