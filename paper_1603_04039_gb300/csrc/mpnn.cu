@@ -412,22 +412,25 @@ __global__ void k_run_heads(const K *__restrict__ key, int64_t m, uint32_t *__re
     if (i < m) f[i] = (key[i] != (K)~(K)0 && (i == 0 || key[i] != key[i - 1])) ? 1u : 0u;
 }
 
-// unique (row, col) pairs: column, signed out value Ahat_row,col and in value Ahat_col,row
+// unique (row, col) pairs: column, signed out value Ahat_row,col and in value
+// Ahat_col,row.  After a sort that gave up (reported by learned_errors) keys and
+// records may be anything: columns and entries stay in range all the same.
 template <class K>
 __global__ void k_edge_merge(const K *__restrict__ key, const uint32_t *__restrict__ rec, int64_t m, int bits,
                              const uint32_t *__restrict__ f, const uint32_t *__restrict__ pos,
-                             const double *__restrict__ val, int32_t *__restrict__ ecol, float *__restrict__ aout,
-                             float *__restrict__ ain, K *__restrict__ ukey) {
+                             const double *__restrict__ val, int64_t entries, int n, int32_t *__restrict__ ecol,
+                             float *__restrict__ aout, float *__restrict__ ain, K *__restrict__ ukey) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m || !f[i]) return;
     float o = 0.f, in = 0.f;
     for (int64_t t = i; t < m && t < i + 2 && key[t] == key[i]; ++t) {
         const uint32_t r = rec[t];
-        const float v = (float)val[r >> 1];
+        const float v = (r >> 1) < entries ? (float)val[r >> 1] : 0.f;
         if (r & 1u) in = v; else o = v;
     }
     const uint32_t p = pos[i];
-    ecol[p] = (int32_t)(key[i] & (((K)1 << bits) - 1));
+    const int64_t cj = (int64_t)(key[i] & (((K)1 << bits) - 1));
+    ecol[p] = cj < n ? (int32_t)cj : 0;
     aout[p] = o;
     ain[p] = in;
     ukey[p] = key[i];
@@ -851,7 +854,7 @@ apcloud_status build_graph_of(apcloud_ctx *c, int bits) {
     APC_LAUNCH(c, K_MPNN_GRAPH, div_up(m, GT1), GT1, 0, k_run_heads<K>, sk, m, fl);
     APC_TRY(scan_u32(c, fl, pos, m, small + 9));
     APC_LAUNCH(c, K_MPNN_GRAPH, div_up(m, GT1), GT1, 0, k_edge_merge<K>, sk, sr, m, bits, (const uint32_t *)fl,
-               (const uint32_t *)pos, val, ecol, aout, ain, uk);
+               (const uint32_t *)pos, val, c->ell_entries, n, ecol, aout, ain, uk);
     APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n + 1, GT1), GT1, 0, k_rowptr<K>, (const K *)uk, (const uint32_t *)(small + 9),
                n, bits, rp);
     APC_LAUNCH(c, K_MPNN_GRAPH, div_up(n, GT1), GT1, 0, k_row_sums, (const int32_t *)rp, (const float *)aout,
@@ -937,15 +940,30 @@ apcloud_status forward(apcloud_ctx *c, apcloud_mpnn *m, const double *b) {
     return cuda_check(c, cudaGetLastError(), "mpnn forward");
 }
 
-apcloud_status tc_error(apcloud_ctx *c, unsigned e) {
-    if (e) return fail(c, APCLOUD_E_TIMEOUT, "a tensor-core layer gave up waiting for its MMAs");
+// What went wrong on the device: the context's error word (the graph's sort) and
+// the tensor-core layers'.  A graph whose sort gave up is built again next time.
+apcloud_status learned_errors(apcloud_ctx *c, const unsigned (&e)[2]) {
+    if (e[0]) {
+        c->mp_graph_n = -1;
+        APC_CUDA(c, cudaMemsetAsync(c->derr.p, 0, sizeof(unsigned), c->s));
+        APC_TRY(device_errors(c, e[0]));
+    }
+    if (e[1]) return fail(c, APCLOUD_E_TIMEOUT, "a tensor-core layer gave up waiting for its MMAs");
     return APCLOUD_OK;
 }
 
-apcloud_status check_tc(apcloud_ctx *c, apcloud_mpnn *m) {
-    unsigned e;
-    APC_TRY(read_back(c, &e, m->err, sizeof e));
-    return tc_error(c, e);
+// both words side by side at dst (device)
+apcloud_status gather_errors(apcloud_ctx *c, apcloud_mpnn *m, unsigned *dst) {
+    APC_CUDA(c, cudaMemcpyAsync(dst, c->derr.p, sizeof(unsigned), cudaMemcpyDeviceToDevice, c->s));
+    APC_CUDA(c, cudaMemcpyAsync(dst + 1, m->err, sizeof(unsigned), cudaMemcpyDeviceToDevice, c->s));
+    return APCLOUD_OK;
+}
+
+apcloud_status check_learned(apcloud_ctx *c, apcloud_mpnn *m) {
+    unsigned *w = ptr<unsigned>(c->dsmall) + 10, e[2];
+    APC_TRY(gather_errors(c, m, w));
+    APC_TRY(read_back(c, e, w, sizeof e));
+    return learned_errors(c, e);
 }
 
 // loss (and with backward, every gradient into m->grad)
@@ -1009,13 +1027,13 @@ apcloud_status loss_grad(apcloud_ctx *c, apcloud_mpnn *m, const double *b, bool 
         }
     }
     APC_CUDA(c, cudaGetLastError());
-    // the loss and the tensor-core layers' error word in one read
-    APC_CUDA(c, cudaMemcpyAsync(lossv + 4, m->err, sizeof(unsigned), cudaMemcpyDeviceToDevice, c->s));
+    // the loss and the error words in one read
+    APC_TRY(gather_errors(c, m, reinterpret_cast<unsigned *>(lossv + 4)));
     double h[5];
     APC_TRY(read_back(c, h, lossv, sizeof h));
-    unsigned e;
-    memcpy(&e, h + 4, sizeof e);
-    APC_TRY(tc_error(c, e));
+    unsigned e[2];
+    memcpy(e, h + 4, sizeof e);
+    APC_TRY(learned_errors(c, e));
     if (h_loss) { h_loss[0] = h[0]; h_loss[1] = h[1]; h_loss[2] = h[2]; }
     return APCLOUD_OK;
 }
@@ -1181,7 +1199,7 @@ extern "C" apcloud_status apcloud_mpnn_outputs(apcloud_ctx *c, apcloud_mpnn *m, 
     if (d_features)
         APC_CUDA(c, cudaMemcpyAsync(d_features, mp<float>(c, MB_F), (size_t)n * NF * sizeof(float),
                                     cudaMemcpyDeviceToDevice, c->s));
-    APC_TRY(check_tc(c, m));
+    APC_TRY(check_learned(c, m));
     return cuda_check(c, cudaStreamSynchronize(c->s), "mpnn outputs");
 }
 
@@ -1196,7 +1214,7 @@ extern "C" apcloud_status apcloud_solve_learned(apcloud_ctx *c, apcloud_mpnn *m,
     double *phi = ensure<double>(c, c->phi, n + 1);
     if (!b || !phi) return APCLOUD_E_NOMEM;
     APC_TRY(forward(c, m, b));
-    APC_TRY(check_tc(c, m));
+    APC_TRY(check_learned(c, m));
     double *dA = ptr<double>(c->dA);
     // initial guess from the original Jacobi scaling: x0 = gamma b / d
     if (use & 2u)
