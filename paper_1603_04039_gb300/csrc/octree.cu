@@ -707,6 +707,8 @@ int64_t crit_bound(const Thresholds &th, int L, int64_t n, int nb) {
     return (int64_t)s + nb;
 }
 
+constexpr int64_t CELLS_FIRST = 1ll << 27;
+
 // units and guard of the integer keys; off where the domain does not allow them
 KeyFix key_fix(const apcloud_params &P) {
     KeyFix k{};
@@ -777,7 +779,9 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
     }
     CellSet set{};
     uint32_t nopen = 0;
-    int64_t want = std::max<int64_t>(2 * crit_bound(th, L, n, nb), 2048);
+    // the bound counts particles level by level, whatever cells they share: a first
+    // table of at most CELLS_FIRST (1.6 GB), larger ones where the cells outgrow it
+    int64_t want = std::max<int64_t>(std::min(2 * crit_bound(th, L, n, nb), CELLS_FIRST), 2048);
     for (;;) {
         int lg = 11;
         while ((1ll << lg) < want) ++lg;

@@ -26,3 +26,17 @@ def test_large_refinement_constants(depth, c):
     assert np.array_equal(g["key"].cpu().numpy().astype(np.uint64), key)
     assert np.array_equal(g["first"].cpu().numpy(), first)
     assert np.array_equal(g["count"].cpu().numpy(), count)
+
+
+def test_many_particles_in_few_deep_cells():
+    """Every particle opens its cells down to depth 21, but all of them the same few."""
+    from paper_1603_04039_gb300 import APCloud
+    g = torch.Generator(device=DEV).manual_seed(3)
+    few = 2.0 * torch.rand(3, 8, generator=g, dtype=torch.float64, device=DEV) - 1.0
+    res = []
+    for n in (80, 100_000_000):
+        at = torch.arange(n, device=DEV) % 8
+        ap = APCloud(max_depth=21, c_refine=1e-9)
+        res.append((ap.build_octree(*(p[at].contiguous() for p in few)), ap.get_leaves()["key"]))
+        assert ap.get_leaves()["count"].sum().item() == n
+    assert res[0][0] == res[1][0] and torch.equal(res[0][1], res[1][1])
