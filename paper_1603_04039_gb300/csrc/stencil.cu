@@ -517,16 +517,20 @@ __device__ bool wls_column_f64(WS &W, int m, int lane, const GramOwn &own, int4 
         col_solve_upper<double>(R2, Ri2, q);
     }
     col_solve_upper<double>(R, Ri, q);
-    // condition estimate min / max of |R_ii|, to FP32 (it is only compared)
-    float lo = 3e38f, hi = 0.f;
-#pragma unroll
-    for (int e = 0; e < NCOL; ++e) {
-        float d = f64_to_f32_int(R[e * NCOL + e]);
-        if (!small) d *= f64_to_f32_int(R2[e * NCOL + e]);
-        lo = fminf(lo, d);
-        hi = fmaxf(hi, d);
+    // condition estimate min / max of |R_ii|, an entry per lane (R_ii > 0: ordered
+    // like its encoding); below 1e-9 the diagonal of G2's factor is 1 + E_ii / 2
+    double rii = 1.0;
+    if (lane < NCOL) {
+        rii = R[lane * NCOL + lane];
+        if (small) rii = fma(0.5 * rii, f32_to_f64_int(reinterpret_cast<const float *>(G)[pk_idx(lane, lane)]), rii);
+        else rii *= R2[lane * NCOL + lane];
     }
-    rratio = f32_to_f64_int(lo / hi);
+    const unsigned dh = (unsigned)__double2hiint(rii), dl = (unsigned)__double2loint(rii);
+    const bool mine = lane < NCOL;
+    const unsigned lh = __reduce_min_sync(FULL, mine ? dh : ~0u), hh = __reduce_max_sync(FULL, mine ? dh : 0u);
+    const unsigned ll = __reduce_min_sync(FULL, mine && dh == lh ? dl : ~0u),
+                   hl = __reduce_max_sync(FULL, mine && dh == hh ? dl : 0u);
+    rratio = __hiloint2double((int)lh, (int)ll) * recip_f64(__hiloint2double((int)hh, (int)hl));
     const double ih = rh * inv_unit, s1 = wj * ih, s2 = s1 * ih;
 #pragma unroll
     for (int e = 0; e < NCOL; ++e) q[e] *= e < 3 ? s1 : s2;   // wj = 0 past the stencil
