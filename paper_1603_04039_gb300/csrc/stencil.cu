@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "fpconv.cuh"
+#include "fprecip.cuh"
 #include "internal.cuh"
 
 namespace apc {
@@ -381,21 +382,6 @@ __device__ __forceinline__ void gram_f64(const double *A, int m, const GramOwn &
     for (int j = 0; j < m; ++j) s1 = fma(A[j * ASTR + o.a1], A[j * ASTR + o.b1], s1);
     for (int j = lane >> 4; j < m; j += 2) s2 = fma(A[j * ASTR + a2], A[j * ASTR + b2], s2);
     s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
-}
-
-// 1 / sqrt(g) and 1 / x in FP64 from an FP32 start, one third-order step each
-// (Halley's iteration; with e = 1 - g y^2 or 1 - x y, |e| < 2^-22, the
-// neglected terms are below 2^-64): 5 and 3 issue slots of the FP64 pipe, the
-// conversions on the integer pipe.  g and x well inside the FP32 range.
-__device__ __forceinline__ double rsqrt_f64(double g) {
-    const double y = f32_to_f64_int(rsqrtf(f64_to_f32_int(g)));
-    const double e = fma(-(g * y), y, 1.0);
-    return fma(y, fma(e, 0.375, 0.5) * e, y);
-}
-__device__ __forceinline__ double recip_f64(double x) {
-    const double y = f32_to_f64_int(1.0f / f64_to_f32_int(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
 }
 
 // wls_column_f32 in FP64, counted by the FP64 pipe's issue slots (16 cycles per
