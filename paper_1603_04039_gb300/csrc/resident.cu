@@ -424,7 +424,11 @@ __device__ __noinline__ void cgs_rotate(Fixed &S, Rot &q, int j, double thr) {
 // vector, several parts of the rows per vector while there are groups left
 // (a warp per vector would spend more FP64 instructions on its shuffle tree
 // than on a small block's rows).  Results in S.val[k] and S.val[nv + k].
+// FP32 terms are added RUN at a time before the run enters the pair (the
+// launched kernels' chains: a lane has up to 256 terms here, and a plain chain of
+// them carries an error that grows with it).
 // Every thread of the block calls it; the caller's grid_sum is the barrier.
+constexpr int RUN = 8;
 template <class T, bool Two, class F>
 __device__ __forceinline__ void block_dots(Fixed &S, int nv, int R, F vec, const T *x, const T *y) {
     typedef Acc<T> A;
@@ -440,15 +444,31 @@ __device__ __forceinline__ void block_dots(Fixed &S, int nv, int R, F vec, const
         if (on) {
             const int k = t % nv, part = t / nv;
             const T *vk = vec(k);
-            T x0 = (T)0, x1 = (T)0;
+            const int step = LPV * parts;
+            if constexpr (sizeof(T) == 4) {
+                for (int r = gl + LPV * part; r < R; r += RUN * step) {
+                    T x0 = (T)0, x1 = (T)0;
+#pragma unroll
+                    for (int u = 0; u < RUN; ++u) {
+                        const int e = r + u * step;
+                        const T v = e < R ? vk[e] : (T)0;
+                        x0 = fma(v, x[e < R ? e : r], x0);
+                        if (Two) x1 = fma(v, y[e < R ? e : r], x1);
+                    }
+                    b0 = A::add(b0, A::of(x0));
+                    if (Two) b1 = A::add(b1, A::of(x1));
+                }
+            } else {
+                T x0 = (T)0, x1 = (T)0;
 #pragma unroll 8
-            for (int r = gl + LPV * part; r < R; r += LPV * parts) {
-                const T v = vk[r];
-                x0 = fma(v, x[r], x0);
-                if (Two) x1 = fma(v, y[r], x1);
+                for (int r = gl + LPV * part; r < R; r += step) {
+                    const T v = vk[r];
+                    x0 = fma(v, x[r], x0);
+                    if (Two) x1 = fma(v, y[r], x1);
+                }
+                b0 = A::of(x0);
+                if (Two) b1 = A::of(x1);
             }
-            b0 = A::of(x0);
-            if (Two) b1 = A::of(x1);
         }
         if (tid < PT) {
 #pragma unroll
