@@ -84,7 +84,8 @@ __device__ __forceinline__ uint32_t cell_coord(double p, double lo, double hi, d
     const uint64_t d = (b >> 63 ? 0ull - mag : mag) - (uint64_t)k.lo;
     const uint64_t edge = 1ull << k.sh, frac = d & (edge - 1);
     if (!k.on || sft > 10 || frac - 2 >= edge - 2 - k.guard) return cell_coord_f64(p, lo, hi, s);
-    if (d > k.ext) return 0x80000000u;   // outside (below lo wraps around)
+    if (d >= k.ext)   // outside (below lo wraps around), or at hi but for bits lost below the unit
+        return d > k.ext ? 0x80000000u : cell_coord_f64(p, lo, hi, s);
     const uint32_t q = (uint32_t)(d >> k.sh);   // hi - lo may exceed its rounded value
     return q < (1u << KEY_DEPTH) ? q : (1u << KEY_DEPTH) - 1u;
 }

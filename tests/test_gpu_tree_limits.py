@@ -40,3 +40,22 @@ def test_many_particles_in_few_deep_cells():
         res.append((ap.build_octree(*(p[at].contiguous() for p in few)), ap.get_leaves()["key"]))
         assert ap.get_leaves()["count"].sum().item() == n
     assert res[0][0] == res[1][0] and torch.equal(res[0][1], res[1][1])
+
+
+# hi - lo rounds to a power of two, and the doubles past hi lie closer than the units of the
+# integer keys
+@pytest.mark.parametrize("lo,hi", [(-(1.0 - 2.0 ** -11), 2.0 ** -11 + 2.0 ** -60), (-(1.0 - 2.0 ** -20), 2.0 ** -20 + 2.0 ** -60),
+                                   (-(1.0 - 2.0 ** -11), 2.0 ** -11)])
+def test_the_last_bit_past_the_domain(lo, hi):
+    from paper_1603_04039_gb300 import APCloud, APCloudError
+    assert hi - lo == 1.0
+    ap = APCloud(lo=lo, hi=hi, max_depth=5, c_refine=0.1)
+    x = torch.full((1000,), 0.5 * (lo + hi), dtype=torch.float64, device=DEV)
+    y = x.clone()
+    y[777] = hi
+    ap.build_octree(y, y, y)
+    y[777] = np.nextafter(hi, 2.0)
+    for k in range(3):
+        with pytest.raises(APCloudError) as e:
+            ap.build_octree(*(y if d == k else x for d in range(3)))
+        assert e.value.status == -2
