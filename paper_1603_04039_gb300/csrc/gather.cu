@@ -148,11 +148,10 @@ __device__ __forceinline__ double f4_hi(const float4 &v) {
 //     pairs in a leaf   238 / 287  246 / 289  250 / 289  250 / 288  252 / 288  254 / 291
 //     in cell order     235 / 280  235 / 279  236 / 280  235 / 280  243 / 292  245 / 297
 // Hence STAGED_LEAVES, and staged only where the warps of a sample taken with the
-// tree (c->scattered) hold nearly as many leaves as particles.  A choice by each warp keeps
-// the shared memory out of L1 in either case: 272 in place of 243 us in cell
+// tree hold nearly as many leaves as particles (c->scattered).  A choice by each warp
+// keeps the shared memory out of L1 in either case: 272 in place of 243 us in cell
 // order.  Records of 96 or 128 bytes change nothing; loads past L1 (358 us) and
 // asynchronous copies into shared memory (310 us) lose.
-constexpr int STAGED_LEAVES = 32768;
 template <bool STAGED>
 __global__ void __launch_bounds__(GT) k_gather_leaf32(
     const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z, int64_t n,
@@ -251,7 +250,7 @@ apcloud_status gather_field(apcloud_ctx *c, double *phi_p, double *ex, double *e
     APC_LAUNCH(c, K_DERIV, div_up(n, db), db, 0, k_derivs, ptr<uint32_t>(c->slice_w), ptr<uint32_t>(c->slice_off),
                ptr<int32_t>(c->ell_col), ptr<double>(c->D), dstride, ptr<double>(c->phi), n, nf,
                ptr<int4>(c->node_ic), c->P.lo[0], c->P.lo[1], c->P.lo[2], unit, nf32);
-    if (mixed && n >= STAGED_LEAVES && c->scattered)
+    if (mixed && c->scattered)
         APC_LAUNCH(c, K_GATHER, div_up(c->N, GT), GT, 0, k_gather_leaf32<true>, c->px, c->py, c->pz, c->N,
                    (const int32_t *)ptr<int32_t>(c->pleaf), (const float *)nf32, phi_p, ex, ey, ez);
     else if (mixed)

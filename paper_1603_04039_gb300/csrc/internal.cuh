@@ -17,6 +17,7 @@ constexpr int KEY_DEPTH = 21;   // 63-bit Morton keys (Section 4.3)
 constexpr int NCOL = 9;         // unknowns of the 3-D second-order GFD system (Section 3.1)
 constexpr int MMAX = 32;        // widest stencil, one warp lane per neighbour
 constexpr int NODE_RECORD = 14; // FP64 words of a node's record in nodefield (gather.cu)
+constexpr int STAGED_LEAVES = 32768;   // leaves from which the mixed gather may stage their records (gather.cu)
 constexpr int MAXC = 512;       // ring candidates held per node in shared memory
 constexpr int MAXC_FAST = 128;  // the same in the stencil kernel over all nodes (overflow: redone with MAXC)
 constexpr double RANK_TOL = 1e-6;
@@ -217,7 +218,7 @@ struct apcloud_ctx {
     int64_t ell_entries = 0;
     int64_t sum_m = 0;  // total stencil neighbours over interior nodes
     int64_t n_fp64_wls = 0;  // mixed form: stencils refactored in FP64
-    bool scattered = false;  // particles side by side in the caller's order mostly lie in different leaves
+    bool scattered = false;  // many leaves, and particles side by side in the caller's order mostly lie in different ones
 
     // sorted particle keys (32 or 64 bits) and permutation (result in key[kbuf], val[kbuf])
     apc::DBuf key[2], val[2];

@@ -630,22 +630,15 @@ __global__ void __launch_bounds__(T) k_adjacency(const uint64_t *__restrict__ an
 }
 
 // Different leaves among 32 particles side by side in the caller's order, summed
-// over SPREAD_N such groups spread evenly over the set (read by the choice of the
-// gather's form); one block.
-constexpr int SPREAD_N = 128, SPREAD_MOST = 30;
-__device__ __forceinline__ void leaf_spread(const int32_t *pleaf, int64_t n, unsigned *out) {
-    constexpr int PER = SPREAD_N / (T / 32);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int32_t leaf[PER];
-#pragma unroll
-    for (int g = 0; g < PER; ++g) leaf[g] = pleaf[(n - 32) * (w * PER + g) / (SPREAD_N - 1) + lane];
-    unsigned sum = 0;
-#pragma unroll
-    for (int g = 0; g < PER; ++g) {
-        const unsigned peers = __match_any_sync(0xffffffffu, leaf[g]);
-        sum += __popc(__ballot_sync(0xffffffffu, lane == __ffs(peers) - 1));
-    }
-    if (lane == 0) atomicAdd(out, sum);
+// over SPREAD_N such groups spread evenly over the set, a warp each (read by the
+// choice of the gather's form)
+constexpr int SPREAD_N = 128, SPREAD_MOST = 30, SPREAD_BLOCKS = SPREAD_N / (T / 32);
+__device__ __forceinline__ void leaf_spread(const int32_t *pleaf, int64_t n, int group, unsigned *out) {
+    const int lane = threadIdx.x & 31;
+    const int32_t leaf = pleaf[(n - 32) * group / (SPREAD_N - 1) + lane];
+    const unsigned peers = __match_any_sync(0xffffffffu, leaf);
+    const unsigned firsts = __ballot_sync(0xffffffffu, lane == __ffs(peers) - 1);
+    if (lane == 0) atomicAdd(out, (unsigned)__popc(firsts));
 }
 
 // Node ranges of every beam: interior nodes [r[b], r[b+1]) (the leaves are
@@ -653,10 +646,10 @@ __device__ __forceinline__ void leaf_spread(const int32_t *pleaf, int64_t n, uns
 // boundary nodes are face-major, leaf-ordered within a face).
 __global__ void k_beam_ranges(const int32_t *__restrict__ beam, int64_t n, int nb, const uint32_t *__restrict__ bpos,
                               int nblk, const uint32_t *__restrict__ nbnd, const int32_t *__restrict__ owner,
-                              int64_t *__restrict__ r, const int32_t *__restrict__ pleaf, int64_t npart,
+                              int64_t *__restrict__ r, int own, const int32_t *__restrict__ pleaf, int64_t npart,
                               unsigned *__restrict__ spread) {
-    if (npart >= 32 && blockIdx.x == gridDim.x - 1) {   // a block more than the ranges take
-        leaf_spread(pleaf, npart, spread);
+    if ((int)blockIdx.x >= own) {   // blocks past those the ranges take
+        leaf_spread(pleaf, npart, (blockIdx.x - own) * (T / 32) + (threadIdx.x >> 5), spread);
         return;
     }
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -867,8 +860,11 @@ apcloud_status build_tree(apcloud_ctx *c, int64_t n, int nb, int bb) {
     APC_LAUNCH(c, K_TREE, nblk, T, 0, k_boundary, (const uint32_t *)bcnt, (const uint32_t *)bpos, nblk, nleaf, ic, bo,
                bf, adj);
     APC_LAUNCH(c, K_ADJ, div_up(8 * nleaf, T), T, 0, k_adjacency, la, ll, nleaf, L, adj, derr);
-    APC_LAUNCH(c, K_TREE, div_up(nb + 1, T) + 1, T, 0, k_beam_ranges, lb, nleaf, nb, (const uint32_t *)bpos, nblk,
-               (const uint32_t *)(small + 4), (const int32_t *)bo, rng, (const int32_t *)pl, n, derr + 1);
+    const int rblk = div_up(nb + 1, T);
+    const bool sample = nleaf >= STAGED_LEAVES && n >= 32;
+    APC_LAUNCH(c, K_TREE, rblk + (sample ? SPREAD_BLOCKS : 0), T, 0, k_beam_ranges, lb, nleaf, nb,
+               (const uint32_t *)bpos, nblk, (const uint32_t *)(small + 4), (const int32_t *)bo, rng, rblk,
+               (const int32_t *)pl, n, derr + 1);
     APC_CUDA(c, cudaGetLastError());
     // the boundary count, the particles' spread and the error word in one read
     APC_CUDA(c, cudaMemcpyAsync(derr + 3, small + 4, sizeof(uint32_t), cudaMemcpyDeviceToDevice, c->s));
