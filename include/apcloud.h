@@ -340,7 +340,8 @@ apcloud_status apcloud_push_particles(apcloud_ctx *ctx, double *d_x, double *d_y
  * results).  Kernel timers (apcloud_set_timing) also run cycles as direct
  * launches, stopped the same way.  A single-beam solve whose matrix fits the
  * shared memory of the SMs together runs as one cooperative kernel (restart
- * up to 31; about 2.4e5 nodes in the mixed polynomial form, 1.2e5 in FP64),
+ * up to 31; about 2.2e5 nodes in the mixed polynomial form, 1.4e5 in the mixed
+ * Jacobi form, 8.8e4 in FP64),
  * with graphs on replayed as a graph of that one kernel: the same results
  * either way.  Synchronises the context stream.  The
  * paper has no counterpart (launch mechanics). */
@@ -374,7 +375,8 @@ apcloud_status apcloud_autotune(apcloud_ctx *ctx, unsigned what, int *h_spmv_blo
 
 /* Sets the launch shapes directly: spmv_block in {64, 128, 256, 512},
  * spmv_unroll in {1, 4}, sweep_sorted in {0, 1}, wls_warps in {2, 4, 8};
- * APCLOUD_E_INVALID otherwise. */
+ * APCLOUD_E_INVALID otherwise.  The first two shape the products on the sliced
+ * ELL; neither the block-local copy nor a solve in one kernel uses them. */
 apcloud_status apcloud_set_launch_shape(apcloud_ctx *ctx, int spmv_block, int spmv_unroll, int sweep_sorted,
                                         int wls_warps);
 

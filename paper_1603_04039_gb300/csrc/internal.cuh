@@ -184,8 +184,8 @@ struct apcloud_ctx {
     int64_t host_syncs = 0;   // read-backs that waited for the stream
     apc::Timer timer;
     // launch shapes chosen by apcloud_autotune
-    int spmv_bs = 256;     // threads per block of the Arnoldi products and sweeps
-    int spmv_unroll = 1;   // stencil entries whose loads a thread issues ahead (1 or 4)
+    int spmv_bs = 256;     // threads per block of the Arnoldi products and sweeps on the ELL
+    int spmv_unroll = 1;   // stencil entries whose loads a thread issues ahead there (1 or 4)
     int sweep_sorted = 1;  // 1: FP16 sweeps and FP32 products on the block-local copy (autotuner's choice)
     bool pdl_on = true;        // sweeps after the first of a polynomial application as programmatic dependents
     int64_t sweep_keep = -1;   // bytes of that matrix the sweeps read with ordinary loads, the rest streaming (-1: automatic)
@@ -332,7 +332,7 @@ struct RadixDigits {
     int shift[RS_MAX_PASS], bits[RS_MAX_PASS];
 };
 RadixDigits radix_digits(int nbits);
-uint32_t *radix_counts(apcloud_ctx *c, const RadixDigits &dg);
+uint32_t *radix_counts(apcloud_ctx *c);   // [pass][RS_BINS], then the passes' tile counters
 apcloud_status clear_radix_counts(apcloud_ctx *c, const RadixDigits &dg);
 template <class K>
 apcloud_status radix_sort_counted(apcloud_ctx *c, K *k0, uint32_t *v0, K *k1, uint32_t *v1, int64_t n,

@@ -1,8 +1,9 @@
 // resident.cu -- whole GMRES solves in one cooperative kernel, the matrix held
 // in shared memory.
 //
-// For systems whose matrix fits the SMs' shared memory together (up to ~2.6e5
-// rows in the mixed polynomial form, ~1.3e5 in FP64) a solve made of one
+// For systems whose matrix fits the SMs' shared memory together (up to 2.2e5
+// rows in the mixed polynomial form, 1.4e5 in the mixed Jacobi form, 8.8e4 in FP64:
+// the largest seen to run) a solve made of one
 // launch per product and reduction is bound by launches and by the latency of
 // each grid-wide reduction, not by bytes: a 1.1e5-row matrix (16 MB as FP16
 // values and 16-bit indices) streams in 2-3 us, a sweep took 5-7 us and a CGS2
@@ -29,17 +30,21 @@
 // What bounds it: the latency of the exchanges (~1.3 us from the owner's
 // store to the reader's barrier; a degree-16 step makes 16 and one sum, two
 // more hops for more than ~20 blocks), the 16-bit gathers from shared memory
-// once a block holds many rows (1.1e5 rows: 2.8 us per sweep, 1.4 of them
+// once a block holds many rows (1.1e5 rows: 2.9 us per sweep, 1.4 of them
 // exchange), and in FP64 the two lanes per clock of that pipe.
 //
 // Measured (GB300, beam with halo, one solve, launched kernels -> here):
 //   FP64 Jacobi, rtol 1e-12:    1471 nodes, 71 steps    4.5 -> 1.0 ms
 //                              15426 nodes, 657 steps  45.9 -> 10.2 ms
-//   mixed degree 16, 1e-11:    15426 nodes, 32 steps    3.8 -> 1.22 ms
-//                             110059 nodes, 54 steps    6.2 -> 3.19 ms
-//                             157540 nodes, 61 steps   11.2 -> 4.35 ms
-// 384 worker threads: 256 leave the sweeps of 1.1e5 rows at 3.48 ms, 512 make
-// every barrier dearer (1.26 against 1.22 ms on 15426 nodes).
+//                              86686 nodes              74 -> 32 us a step
+//   mixed degree 16, 1e-11:    15426 nodes, 32 steps    3.4 -> 1.25 ms
+//                             110059 nodes, 54 steps    6.4 -> 3.19 ms
+//                             222416 nodes            165 -> 88 us a step
+// 384 worker threads: 256 leave the solve of 1.1e5 rows at 3.48 ms, 512 make
+// every barrier dearer (1.26 against 1.22 ms on 15426 nodes).  Counters of the
+// 1.1e5-row solve: a warp waits 3.2 cycles at barriers and 3.4 for loads between
+// two instructions, the schedulers issue in 31% of the cycles, the shared-memory
+// pipe is 42% busy; of the 1.5e4-row FP64 solve: 18 of 28 at barriers.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -556,9 +561,6 @@ __device__ __forceinline__ unsigned char *carve(unsigned char *&p, size_t bytes)
     return q;
 }
 
-// One solve (or the part of it that fits the step budget).  The exchanges and
-// sums are numbered from a.in->tag0; no number is used twice with the same
-// words.
 // w -= V h over nv basis vectors, own rows
 template <class T>
 __device__ __forceinline__ void project(const T *h_, const Shape &h, int nv, const T *V, int64_t ldv, T *wv, int t0) {
@@ -607,6 +609,9 @@ __device__ __forceinline__ void update_vectors(Fixed &S, const Shape &h, int j, 
     }
 }
 
+// One solve (or the part of it that fits the step budget).  The exchanges and
+// sums are numbered from a.in->tag0; no number is used twice with the same
+// words.
 template <class T, bool POLY>
 __global__ void __launch_bounds__(PB, 1) k_gmres_resident(ResidentArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];

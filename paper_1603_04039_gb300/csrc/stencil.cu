@@ -393,8 +393,11 @@ __device__ __forceinline__ void gram_f64(const double *A, int m, const GramOwn &
 // the rounding of the first pass (kappa^2 eps), and below 1e-9 its square is
 // below 1e-18 and the FP32 rounding of the correction E q below 1e-15 of q.
 // A block with a larger E goes through the full second pass.
-// ~330 slots: 2.8e5 nodes 12.76 -> 5.13 ms, the FP64 pipe's own time for them
-// (fewer resident warps change nothing).
+// ~335 slots: 2.8e5 nodes 12.76 -> 5.13 ms, the FP64 pipe's own time for them
+// (fewer resident warps change nothing).  Against QR in extended precision the
+// operator's rows are off by 1.9e-16 to 2.6e-16 of their norm on average (the full
+// second pass: 2.4e-16 to 3.5e-16) from condition estimates of 0.02 up, by 2.0e-14
+// (2.1e-14) where they fall to 3e-4; the estimate itself by 6e-16 to 1.9e-15.
 template <class WS>
 __device__ bool wls_column_f64(WS &W, int m, int lane, const GramOwn &own, int4 c0, const int4 *__restrict__ ic,
                                double inv_unit, double ec, double inv_1mec, double (&q)[NCOL], double &lapj,
